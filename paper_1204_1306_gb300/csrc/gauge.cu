@@ -170,22 +170,75 @@ __device__ __forceinline__ long long shifted(const Geom &g, const int x[4], int 
     return site_index(g, y);
 }
 
-// sum of the 6 staples: ReTr(U(x,mu) A) = sum of the plaquettes holding U(x,mu)
-__device__ M3 staple(const Geom &g, const double2 *U, const int x[4], int mu) {
-    M3 A;
+// One entry per product of three links: fused multiply-adds throughout, so a
+// 3x3 complex product is 108 FP64 instructions.
+__device__ __forceinline__ M3 mul_nd(const M3 &a, const M3 &b) {  // a b^dagger
+    M3 r;
+#pragma unroll
     for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            C z = cjmul(b.e[j][0], a.e[i][0]);
+            z = cjfma(b.e[j][1], a.e[i][1], z);
+            r.e[i][j] = cjfma(b.e[j][2], a.e[i][2], z);
+        }
+    return r;
+}
+
+__device__ __forceinline__ M3 mul_dd(const M3 &a, const M3 &b) {  // a^dagger b^dagger = (b a)^dagger
+    M3 r;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            C z = cmul(b.e[j][0], a.e[0][i]);
+            z = cfma(b.e[j][1], a.e[1][i], z);
+            z = cfma(b.e[j][2], a.e[2][i], z);
+            r.e[i][j] = cc(z);
+        }
+    return r;
+}
+
+__device__ __forceinline__ void fma_nd(M3 &r, const M3 &a, const M3 &b) {  // r += a b^dagger
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) r.e[i][j] = cjfma(b.e[j][k], a.e[i][k], r.e[i][j]);
+}
+
+__device__ __forceinline__ void fma_nn(M3 &r, const M3 &a, const M3 &b) {  // r += a b
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) r.e[i][j] = cfma(a.e[i][k], b.e[k][j], r.e[i][j]);
+}
+
+// sum of the 6 staples: ReTr(U(x,mu) A) = sum of the plaquettes holding U(x,mu)
+__device__ __forceinline__ M3 staple(const Geom &g, const double2 *U, const int x[4], long long s, int mu) {
+    M3 A;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
         for (int j = 0; j < 3; ++j) A.e[i][j] = {0, 0};
-    const long long s = site_index(g, x);
-    for (int nu = 0; nu < 4; ++nu) {
-        if (nu == mu) continue;
+#pragma unroll 1
+    for (int d = 1; d < 4; ++d) {
+        const int nu = (mu + d) & 3;
         const long long sp_mu = shifted(g, x, mu, 1, nu, 0);
         const long long sp_nu = shifted(g, x, nu, 1, mu, 0);
         const long long sm_nu = shifted(g, x, nu, -1, mu, 0);
         const long long spm = shifted(g, x, mu, 1, nu, -1);
-        M3 up = mul(mul(ldU(U, g.V, nu, sp_mu), dagm(ldU(U, g.V, mu, sp_nu))), dagm(ldU(U, g.V, nu, s)));
-        M3 dn = mul(mul(dagm(ldU(U, g.V, nu, spm)), dagm(ldU(U, g.V, mu, sm_nu))), ldU(U, g.V, nu, sm_nu));
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j) A.e[i][j] = ca(A.e[i][j], ca(up.e[i][j], dn.e[i][j]));
+        {
+            const M3 t = mul_nd(ldU(U, g.V, nu, sp_mu), ldU(U, g.V, mu, sp_nu));
+            fma_nd(A, t, ldU(U, g.V, nu, s));
+        }
+        {
+            const M3 t = mul_dd(ldU(U, g.V, nu, spm), ldU(U, g.V, mu, sm_nu));
+            fma_nn(A, t, ldU(U, g.V, nu, sm_nu));
+        }
     }
     return A;
 }
@@ -209,54 +262,89 @@ __device__ __forceinline__ C2 q2m(double q0, double q1, double q2, double q3) {
 __device__ __forceinline__ C2 mul2(const C2 &a, const C2 &b) {
     C2 r;
     for (int i = 0; i < 2; ++i)
-        for (int j = 0; j < 2; ++j) r.e[i][j] = ca(cm(a.e[i][0], b.e[0][j]), cm(a.e[i][1], b.e[1][j]));
+        for (int j = 0; j < 2; ++j) r.e[i][j] = cfma(a.e[i][1], b.e[1][j], cmul(a.e[i][0], b.e[0][j]));
     return r;
 }
 
+__device__ __forceinline__ C sel(bool c, C a, C b) { return {c ? a.re : b.re, c ? a.im : b.im}; }
+
 constexpr int MAX_ATTEMPTS = 1000;
 constexpr double KP_THRESHOLD = 2.0;
+constexpr int CM_NT = 32;
 
-__global__ void cm_update_kernel(Geom g, const BlockInfo *binfo, double2 *U, int mu, int parity, int colour, int all,
-                                 double beta, int kind, uint64_t seed, uint64_t sweep, int *failed) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= g.Vh) return;
-    const long long s = (long long)parity * g.Vh + t;
+// Update of the active links (x, mu) of one parity: thread t takes entry
+// t % n_act of the list of active sites (index within the block's half, the
+// same for every block) of block rank rank_lo + t / n_act.
+//
+// GB300 has two FP64 lanes per SM, so the ~1650 (overrelaxation) to ~2600
+// (heatbath) FP64 instructions of an update bound this kernel and a lane
+// that only tests whether its link is active costs a full one: launched over
+// the list, every lane of a warp updates a link (4^4 blocks: 9.4 % of the
+// links are active; over all sites a warp did the work of a full one for
+// three of them).  The SU(2) subgroup of a step is picked by selects between
+// rows (a runtime index would put the link in local memory), only the 2 x 2
+// part of U A that it needs is formed, and all products are fused
+// multiply-adds.  One warp per CTA spreads a short list over all SMs.
+template <int KIND>
+__global__ void __launch_bounds__(CM_NT) cm_update_kernel(Geom g, const BlockInfo *binfo, double2 *U,
+                                                          const int *act, int n_act, int mu, int parity, int rank_lo,
+                                                          int n_ranks, int colour, double beta, uint64_t seed,
+                                                          uint64_t sweep, int *failed) {
+    const unsigned t = blockIdx.x * CM_NT + threadIdx.x;  // at most V / 2 < 2^30 + one CTA
+    const unsigned rl = t / (unsigned)n_act;
+    if (rl >= (unsigned)n_ranks) return;
+    const long long s = (long long)parity * g.Vh + (long long)(rank_lo + rl) * g.Vbh + act[t - rl * n_act];
     int p, r, j, y[4], x[4];
     decode(g, binfo, s, p, r, j, y, x);
     if (colour >= 0) {
         const BlockInfo &bi = binfo[r];
         if (((bi.B[0] + bi.B[1] + bi.B[2] + bi.B[3]) & 1) != colour) return;
     }
-    if (!link_active(g, y, mu, all)) return;
-    const M3 A = staple(g, U, x, mu);
+    const M3 A = staple(g, U, x, s, mu);
     M3 Ul = ldU(U, g.V, mu, s);
     const uint64_t link = (uint64_t)(4 * lex_index(g, x) + mu);
-    const bool forward = uniforms(seed, TAG_HB, sweep, link, 0, 0).u[0] < 0.5;
+    const bool fwd = uniforms(seed, TAG_HB, sweep, link, 0, 0).u[0] < 0.5;
     int nfail = 0;
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const int sgi = forward ? k : 2 - k;
-        const int i0 = (sgi == 2) ? 1 : 0;
-        const int j0 = (sgi == 0) ? 1 : 2;
-        // W = Ul A, 2x2 sub-block (i0, j0)
-        M3 W = mul(Ul, A);
-        C w00 = W.e[i0][i0], w01 = W.e[i0][j0], w10 = W.e[j0][i0], w11 = W.e[j0][j0];
-        double r0 = 0.5 * (w00.re + w11.re);
-        double r1 = 0.5 * (w01.im + w10.im);
-        double r2 = 0.5 * (w01.re - w10.re);
-        double r3 = 0.5 * (w00.im - w11.im);
-        const double kn = sqrt(r0 * r0 + r1 * r1 + r2 * r2 + r3 * r3);
+        // subgroups (0,1), (0,2), (1,2) forward or reversed: rows (columns of
+        // A) i0 < j0; the middle one is (0,2) either way
+        C ri[3], rj[3], ai[3], aj[3];
+        const bool f01 = (k == 0) == fwd;  // k != 1: subgroup (0,1), else (1,2)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            ri[c] = k == 1 ? Ul.e[0][c] : sel(f01, Ul.e[0][c], Ul.e[1][c]);
+            rj[c] = k == 1 ? Ul.e[2][c] : sel(f01, Ul.e[1][c], Ul.e[2][c]);
+            ai[c] = k == 1 ? A.e[c][0] : sel(f01, A.e[c][0], A.e[c][1]);
+            aj[c] = k == 1 ? A.e[c][2] : sel(f01, A.e[c][1], A.e[c][2]);
+        }
+        // the 2 x 2 sub-block of W = Ul A
+        C w00 = cmul(ri[0], ai[0]), w01 = cmul(ri[0], aj[0]), w10 = cmul(rj[0], ai[0]), w11 = cmul(rj[0], aj[0]);
+#pragma unroll
+        for (int c = 1; c < 3; ++c) {
+            w00 = cfma(ri[c], ai[c], w00);
+            w01 = cfma(ri[c], aj[c], w01);
+            w10 = cfma(rj[c], ai[c], w10);
+            w11 = cfma(rj[c], aj[c], w11);
+        }
+        double r0_ = 0.5 * (w00.re + w11.re);
+        double r1_ = 0.5 * (w01.im + w10.im);
+        double r2_ = 0.5 * (w01.re - w10.re);
+        double r3_ = 0.5 * (w00.im - w11.im);
+        const double kn = sqrt(r0_ * r0_ + r1_ * r1_ + r2_ * r2_ + r3_ * r3_);
         if (!(kn > 0.0)) continue;
         const double ik = 1.0 / kn;
-        C2 vdag = q2m(r0 * ik, -r1 * ik, -r2 * ik, -r3 * ik);
+        C2 vdag = q2m(r0_ * ik, -r1_ * ik, -r2_ * ik, -r3_ * ik);
         C2 R;
-        if (kind == 0) {
+        if (KIND == 0) {
             const double alpha = 2.0 * beta * kn / 3.0;
             double a0 = 1.0;
             bool ok = false;
+#pragma unroll 1
             for (int att = 0; att < MAX_ATTEMPTS; ++att) {
                 uni4 u = uniforms(seed, TAG_HB, sweep, link, (uint64_t)(1 + 2 * k), (uint64_t)att);
                 if (alpha >= KP_THRESHOLD) {
-                    const double cth = cos(2.0 * M_PI * u.u[1]);
+                    const double cth = cospi(2.0 * u.u[1]);
                     const double xx = -(log(u.u[0]) + cth * cth * log(u.u[2])) / alpha;
                     if (u.u[3] * u.u[3] <= 1.0 - 0.5 * xx) {
                         a0 = 1.0 - xx;
@@ -279,32 +367,75 @@ __global__ void cm_update_kernel(Geom g, const BlockInfo *binfo, double2 *U, int
             uni4 d = uniforms(seed, TAG_HB, sweep, link, (uint64_t)(2 + 2 * k), 0);
             const double cth = 2.0 * d.u[0] - 1.0;
             const double sth = sqrt(fmax(0.0, 1.0 - cth * cth));
-            const double phi = 2.0 * M_PI * d.u[1];
+            double sp, cp;
+            sincospi(2.0 * d.u[1], &sp, &cp);
             const double rad = sqrt(fmax(0.0, 1.0 - a0 * a0));
-            C2 X = q2m(a0, rad * sth * cos(phi), rad * sth * sin(phi), rad * cth);
+            C2 X = q2m(a0, rad * sth * cp, rad * sth * sp, rad * cth);
             R = mul2(X, vdag);
         } else {
             R = mul2(vdag, vdag);
         }
+#pragma unroll
         for (int c = 0; c < 3; ++c) {
-            C ri = Ul.e[i0][c], rj = Ul.e[j0][c];
-            Ul.e[i0][c] = ca(cm(R.e[0][0], ri), cm(R.e[0][1], rj));
-            Ul.e[j0][c] = ca(cm(R.e[1][0], ri), cm(R.e[1][1], rj));
+            const C ni = cfma(R.e[0][1], rj[c], cmul(R.e[0][0], ri[c]));
+            const C nj = cfma(R.e[1][1], rj[c], cmul(R.e[1][0], ri[c]));
+            if (k == 1) {
+                Ul.e[0][c] = ni;
+                Ul.e[2][c] = nj;
+            } else {
+                Ul.e[0][c] = sel(f01, ni, Ul.e[0][c]);
+                Ul.e[1][c] = sel(f01, nj, ni);
+                Ul.e[2][c] = sel(f01, Ul.e[2][c], nj);
+            }
         }
     }
     stU(U, g.V, mu, s, Ul);
     if (nfail && failed) atomicAdd(failed, nfail);
 }
 
-__global__ void reunit_active_kernel(Geom g, const BlockInfo *binfo, double2 *U, int all) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 4 * g.V) return;
-    const long long s = t >> 2;
-    const int mu = (int)(t & 3);
-    int p, r, j, y[4], x[4];
-    decode(g, binfo, s, p, r, j, y, x);
-    if (!link_active(g, y, mu, all)) return;
+// reunitarise the links of the list act (direction mu, one parity)
+__global__ void __launch_bounds__(128) reunit_active_kernel(Geom g, double2 *U, const int *act, int n_act, int mu,
+                                                            int parity) {
+    const unsigned t = blockIdx.x * 128 + threadIdx.x;
+    const unsigned r = t / (unsigned)n_act;
+    if (r >= (unsigned)g.nblocks) return;
+    const long long s = (long long)parity * g.Vh + (long long)r * g.Vbh + act[t - r * n_act];
     stU(U, g.V, mu, s, reunit(ldU(U, g.V, mu, s)));
+}
+
+// Active sites of every (mu, parity): indices within a block's half, block
+// after block alike.  Built once per context and active set.
+struct ActiveList {
+    const int *d = nullptr;  // device, the eight lists back to back
+    int off[4][2], n[4][2];
+};
+
+static ActiveList active_list(psms_ctx *c, int all) {
+    const Geom &g = c->g;
+    ActiveList a;
+    std::vector<int> h;
+    for (int mu = 0; mu < 4; ++mu)
+        for (int p = 0; p < 2; ++p) {
+            a.off[mu][p] = (int)h.size();
+            for (int j = 0; j < g.Vbh; ++j) {
+                int y[4], ll = 2 * j;
+                y[3] = ll & (g.l[3] - 1);
+                y[2] = (ll >> g.lsh[3]) & (g.l[2] - 1);
+                y[1] = (ll >> (g.lsh[3] + g.lsh[2])) & (g.l[1] - 1);
+                y[0] = ll >> (g.lsh[3] + g.lsh[2] + g.lsh[1]);
+                if (((y[0] + y[1] + y[2] + y[3]) & 1) != p) y[3] += 1;
+                if (link_active(g, y, mu, all)) h.push_back(j);
+            }
+            a.n[mu][p] = (int)h.size() - a.off[mu][p];
+        }
+    const std::string name = all ? "act_all" : "act_blocks";
+    const auto it = c->scratch.find(name);
+    const bool have = it != c->scratch.end() && it->second.p;
+    int *d = (int *)scratch(c, name, sizeof(int) * (h.empty() ? 1 : h.size()));
+    if (!have && !h.empty())
+        cuda_check(cudaMemcpy(d, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice), "active list");
+    a.d = d;
+    return a;
 }
 
 int gauge_sweep(psms_ctx *c, double2 *U, int active_set, int n_iter, int n_or, double beta, uint64_t seed,
@@ -321,15 +452,26 @@ int gauge_sweep(psms_ctx *c, double2 *U, int active_set, int n_iter, int n_or, d
     for (int col = 0; col < ncol; ++col)
         for (int mu = 0; mu < 4; ++mu)
             for (int p = 0; p < 2; ++p) subs.push_back({mu, p, ncol == 2 ? col : -1});
+    const ActiveList act = active_list(c, all);
     int *failed = (int *)scratch(c, "hb_failed", sizeof(int));
     cuda_check(cudaMemsetAsync(failed, 0, sizeof(int), c->stream), "hb memset");
-    const int NT = 128;
-    const unsigned nb = (unsigned)((g.Vh + NT - 1) / NT);
     auto sweep = [&](int kind, bool rev, uint64_t sid) {
         for (size_t i = 0; i < subs.size(); ++i) {
             const Sub &q = subs[rev ? subs.size() - 1 - i : i];
-            cm_update_kernel<<<nb, NT, 0, c->stream>>>(g, c->d_binfo, U, q.mu, q.p, q.colour, all, beta, kind, seed,
-                                                       sid, failed);
+            const int n = act.n[q.mu][q.p];
+            if (n == 0) continue;
+            // one colour of a checkerboard is a range of ranks; without a
+            // checkerboard the kernel tests the colour
+            const bool range = q.colour >= 0 && g.coloured;
+            const int lo = range ? q.colour * g.nbh : 0, nr = range ? g.nbh : g.nblocks;
+            const unsigned nb = (unsigned)(((long long)nr * n + CM_NT - 1) / CM_NT);
+            const int *list = act.d + act.off[q.mu][q.p];
+            if (kind == 0)
+                cm_update_kernel<0><<<nb, CM_NT, 0, c->stream>>>(g, c->d_binfo, U, list, n, q.mu, q.p, lo, nr,
+                                                                 range ? -1 : q.colour, beta, seed, sid, failed);
+            else
+                cm_update_kernel<1><<<nb, CM_NT, 0, c->stream>>>(g, c->d_binfo, U, list, n, q.mu, q.p, lo, nr,
+                                                                 range ? -1 : q.colour, beta, seed, sid, failed);
             PSMS_LAUNCH_CHECK("cm_update_kernel");
         }
     };
@@ -340,9 +482,14 @@ int gauge_sweep(psms_ctx *c, double2 *U, int active_set, int n_iter, int n_or, d
         for (int k = 0; k < n_or; ++k) sweep(1, true, s++);
         sweep(0, true, s++);
     }
-    const long long n = 4 * g.V;
-    reunit_active_kernel<<<(unsigned)((n + 127) / 128), 128, 0, c->stream>>>(g, c->d_binfo, U, all);
-    PSMS_LAUNCH_CHECK("reunit");
+    for (int mu = 0; mu < 4; ++mu)
+        for (int p = 0; p < 2; ++p) {
+            const int n = act.n[mu][p];
+            if (n == 0) continue;
+            reunit_active_kernel<<<(unsigned)(((long long)g.nblocks * n + 127) / 128), 128, 0, c->stream>>>(
+                g, U, act.d + act.off[mu][p], n, mu, p);
+            PSMS_LAUNCH_CHECK("reunit");
+        }
     int h = 0;
     cuda_check(cudaMemcpyAsync(&h, failed, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "hb failed");
     cuda_check(cudaStreamSynchronize(c->stream), "hb sync");
