@@ -12,8 +12,10 @@ namespace psms {
 struct BCS {
     double2 rho, alpha, omega, beta;
     double rr, target;
-    int active, iters;
+    int active, iters, stalled;
 };
+
+constexpr int BCG_SUMS = 7;  // sums of one reduction (see bcg_stage)
 
 __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
     const double d = b.x * b.x + b.y * b.y;
@@ -23,68 +25,96 @@ __device__ __forceinline__ double2 cmul2(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// stage: 0 alpha = rho / <rh, v>; 1 omega = <t, s> / <t, t>;
-//        2 rho_new = <rh, r>, rr = |r|^2, beta, convergence
-__device__ __forceinline__ void bcg_stage(BCS *st, int k, double re, double im, double aa, int stage, int maxit, int *flags) {
+// stage 0: sums 0, 1: <rh, v>; alpha = rho / <rh, v>
+// stage 1: sums 0, 1: <t, s>; 2: |t|^2; 3, 4: <rh, t>; 5, 6: <rh, s>;
+//          omega = <t, s> / |t|^2, rho' = <rh, s - omega t> and beta = (rho' /
+//          rho)(alpha / omega), so that x, r and p are updated in one pass.
+//          (<rh, s> = 0 but for rounding; dropping it stalls the solver at
+//          16^4.)
+// stage 2: sum 2: |r|^2 of the new residual, convergence
+__device__ __forceinline__ void bcg_stage(BCS *st, int k, const double v[BCG_SUMS], int stage, int maxit, int *flags) {
     BCS s = st[k];
-    const double2 d = make_double2(re, im);
     if (stage == 0) {
-        if (!(re * re + im * im > 0.0)) {
+        if (!(v[0] * v[0] + v[1] * v[1] > 0.0)) {
             s.active = 0;  // breakdown: <rh, v> = 0
         } else {
-            s.alpha = cdiv(s.rho, d);
+            s.alpha = cdiv(s.rho, make_double2(v[0], v[1]));
         }
     } else if (stage == 1) {
-        s.omega = aa > 0.0 ? make_double2(re / aa, im / aa) : make_double2(0.0, 0.0);
+        s.omega = v[2] > 0.0 ? make_double2(v[0] / v[2], v[1] / v[2]) : make_double2(0.0, 0.0);
+        const double2 w = cmul2(s.omega, make_double2(v[3], v[4]));
+        const double2 rho = make_double2(v[5] - w.x, v[6] - w.y);
+        s.stalled = !(s.omega.x * s.omega.x + s.omega.y * s.omega.y > 0.0) || !(rho.x * rho.x + rho.y * rho.y > 0.0);
+        s.beta = s.stalled ? make_double2(0.0, 0.0) : cmul2(cdiv(rho, s.rho), cdiv(s.alpha, s.omega));
+        s.rho = rho;
     } else {
-        // the partials are sum conj(r) rh = conj(<rh, r>) and |r|^2 of the
-        // new residual
-        const double2 dr = make_double2(re, -im);
         s.iters += 1;
-        s.rr = aa;
-        const bool stalled = !(s.omega.x * s.omega.x + s.omega.y * s.omega.y > 0.0) ||
-                             !(re * re + im * im > 0.0);
-        if (!stalled) s.beta = cmul2(cdiv(dr, s.rho), cdiv(s.alpha, s.omega));
-        s.rho = dr;
-        if (aa <= s.target || s.iters >= maxit || stalled || !(aa == aa)) s.active = 0;
+        s.rr = v[2];
+        if (v[2] <= s.target || s.iters >= maxit || s.stalled || !(v[2] == v[2])) s.active = 0;
     }
     st[k] = s;
     flags[k] = s.active;
 }
 
+// Sums over a warp of P values per lane (P = 1, 2, 4, 8): while there are
+// several, half of them go to the other half of the lanes, so that 8 sums
+// take 9 FP64 additions and not 40 (a warp's FP64 addition occupies the two
+// FP64 lanes of an SM for 16 clocks).  Lane l ends with value wsum_index<P>(l).
+template <int P>
+__device__ __forceinline__ double wsum(const double *v) {
+    const int l = threadIdx.x & 31;
+    double r[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) r[i] = v[i];
+    int o = 16;
+#pragma unroll
+    for (int m = P; m > 1; m >>= 1, o >>= 1) {
+        const bool up = l & o;
+#pragma unroll
+        for (int i = 0; i < m / 2; ++i) {
+            const double keep = up ? r[i + m / 2] : r[i], give = up ? r[i] : r[i + m / 2];
+            r[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) r[0] += __shfl_xor_sync(0xffffffffu, r[0], o);
+    return r[0];
+}
+template <int P>
+__device__ __forceinline__ int wsum_index(int l) {  // the leading bits of the lane number
+    return P == 1 ? 0 : P == 2 ? l >> 4 : P == 4 ? l >> 3 : l >> 2;
+}
+
 // Writes this CTA's partials of system k; the last CTA of the system to
 // finish (a counter per system, no waiting) sums all partials in a fixed
 // order and applies the scalar stage, so the result does not depend on
-// which CTA finishes last.
-template <int NT>
-__device__ __forceinline__ void bcg_partials_and_stage(BCS *st, double re, double im, double aa, double *p_re,
-                                                       double *p_im, double *p_aa, unsigned int *counters, int stage,
-                                                       int maxit, int *flags, double (*sh)[NT / 32], int k,
-                                                       int cta, int nct) {
+// which CTA finishes last.  part: BCG_SUMS arrays of part_n doubles; the sums
+// [LO, HI) are taken.  Ends at a barrier.
+template <int NT, int LO, int HI>
+__device__ __forceinline__ void bcg_partials_and_stage(BCS *st, const double in[BCG_SUMS], double *part,
+                                                       long long part_n, unsigned int *counters, int stage, int maxit,
+                                                       int *flags, double (*sh)[NT / 32], int k, int cta, int nct) {
     const long long slot = (long long)k * nct + cta;
     __shared__ int last;
+    constexpr int N = HI - LO, P = N > 4 ? 8 : N > 2 ? 4 : N;
+    const int l = threadIdx.x & 31, wi = wsum_index<P>(l);
+    const bool lead = l == wi * (32 / P) && wi < N;
+    auto warp_sums = [&](const double *v) {
+        double x[P];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        re += __shfl_xor_sync(0xffffffffu, re, o);
-        im += __shfl_xor_sync(0xffffffffu, im, o);
-        aa += __shfl_xor_sync(0xffffffffu, aa, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        sh[0][threadIdx.x >> 5] = re;
-        sh[1][threadIdx.x >> 5] = im;
-        sh[2][threadIdx.x >> 5] = aa;
-    }
+        for (int a = 0; a < P; ++a) x[a] = a < N ? v[LO + a] : 0.0;
+        const double t = wsum<P>(x);
+        if (lead) sh[LO + wi][threadIdx.x >> 5] = t;
+    };
+    warp_sums(in);
     __syncthreads();
     if (threadIdx.x == 0) {
-        double t0 = 0, t1 = 0, t2 = 0;
-        for (int w = 0; w < NT / 32; ++w) {
-            t0 += sh[0][w];
-            t1 += sh[1][w];
-            t2 += sh[2][w];
+#pragma unroll
+        for (int a = LO; a < HI; ++a) {
+            double t = 0;
+            for (int w = 0; w < NT / 32; ++w) t += sh[a][w];
+            part[a * part_n + slot] = t;
         }
-        p_re[slot] = t0;
-        p_im[slot] = t1;
-        p_aa[slot] = t2;
         __threadfence();
         last = atomicAdd(&counters[k], 1u) == (unsigned int)nct - 1u;
     }
@@ -92,32 +122,27 @@ __device__ __forceinline__ void bcg_partials_and_stage(BCS *st, double re, doubl
     if (!last) return;
     __threadfence();
     // the other CTAs' partials, read past L1 (written by other SMs)
-    const int m = nct;
-    double v[3] = {0, 0, 0};
-    for (int i = threadIdx.x; i < m; i += NT) {
-        const long long q = (long long)k * m + i;
-        v[0] += __ldcg(p_re + q);
-        v[1] += __ldcg(p_im + q);
-        v[2] += __ldcg(p_aa + q);
-    }
-    double tot[3];
+    double v[BCG_SUMS];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        double x = v[a];
+    for (int a = 0; a < BCG_SUMS; ++a) v[a] = 0;
+    for (int i = threadIdx.x; i < nct; i += NT) {
+        const long long q = (long long)k * nct + i;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) sh[a][threadIdx.x >> 5] = x;
-        __syncthreads();
-        double t = 0;
-        for (int w = 0; w < NT / 32; ++w) t += sh[a][w];
-        tot[a] = t;
+        for (int a = LO; a < HI; ++a) v[a] += __ldcg(part + a * part_n + q);
     }
-    const double r0 = tot[0], r1 = tot[1], r2 = tot[2];
+    warp_sums(v);
+    __syncthreads();
     if (threadIdx.x == 0) {
+#pragma unroll
+        for (int a = LO; a < HI; ++a) {
+            double t = 0;
+            for (int w = 0; w < NT / 32; ++w) t += sh[a][w];
+            v[a] = t;
+        }
         counters[k] = 0;
-        bcg_stage(st, k, r0, r1, r2, stage, maxit, flags);
+        bcg_stage(st, k, v, stage, maxit, flags);
     }
+    __syncthreads();
 }
 
 }  // namespace psms

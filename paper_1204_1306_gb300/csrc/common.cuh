@@ -398,6 +398,35 @@ __device__ __forceinline__ void store_spinor(typename S::elem *p, long long cs, 
     }
 }
 
+// one 16-byte unit (2^VSH complex numbers)
+template <class S>
+__device__ __forceinline__ void load_unit(const typename S::elem *p, cpx<typename S::R> *v) {
+    if constexpr (S::VSH == 0) {
+        v[0] = S::ldi(p, 0);
+    } else if constexpr (S::VSH == 1) {
+        const float4 w = *reinterpret_cast<const float4 *>(p);
+        v[0] = {w.x, w.y};
+        v[1] = {w.z, w.w};
+    } else {
+        const uint4 w = *reinterpret_cast<const uint4 *>(p);
+        v[0] = bf_lo(w.x), v[1] = bf_lo(w.y), v[2] = bf_lo(w.z), v[3] = bf_lo(w.w);
+    }
+}
+
+template <class S>
+__device__ __forceinline__ void store_unit(typename S::elem *p, const cpx<typename S::R> *v) {
+    if constexpr (S::VSH == 0) {
+        S::sti(p, 0, v[0]);
+    } else if constexpr (S::VSH == 1) {
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0].re, v[0].im, v[1].re, v[1].im);
+    } else {
+        __nv_bfloat162 h[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) h[m] = __floats2bfloat162_rn(v[m].re, v[m].im);
+        *reinterpret_cast<uint4 *>(p) = *reinterpret_cast<const uint4 *>(h);
+    }
+}
+
 template <class S>
 __device__ __forceinline__ SU3<typename S::R> load_link(const typename S::elem *U, long long V, int mu, long long s) {
     SU3<typename S::R> u;

@@ -32,7 +32,8 @@ struct HopArgs {
     int dot;
     View<E> dx;
     BCS *dst;
-    double *dre, *dim, *daa;
+    double *dpart;
+    long long dpart_n;
     unsigned int *dcnt;
     int dstage, dmaxit;
     int *dflags;
@@ -133,6 +134,54 @@ __device__ __forceinline__ void hop_dirs(const HopArgs<E> &a, const Geom &g, con
     }
 }
 
+// The dot products of an output spinor o, its 12 components summed in the
+// inner precision (threads and CTAs in FP64): dot 1: <x, o>; dot 2: <o, y>,
+// |o|^2, <x, o>, <x, y>
+template <class R>
+__device__ __forceinline__ void hop_dots(int dot, const Spinor<R> &o, const Spinor<R> &x, const Spinor<R> &y,
+                                         double sum[BCG_SUMS]) {
+    R xr = 0, xi = 0, yr = 0, yi = 0, aa = 0, zr = 0, zi = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const cpx<R> ov = o.c[q][c], xv = x.c[q][c];
+            xr += xv.re * ov.re + xv.im * ov.im;
+            xi += xv.re * ov.im - xv.im * ov.re;
+            if (dot == 2) {
+                const cpx<R> yv = y.c[q][c];
+                yr += ov.re * yv.re + ov.im * yv.im;
+                yi += ov.re * yv.im - ov.im * yv.re;
+                aa += ov.re * ov.re + ov.im * ov.im;
+                zr += xv.re * yv.re + xv.im * yv.im;
+                zi += xv.re * yv.im - xv.im * yv.re;
+            }
+        }
+    if (dot == 1) {
+        sum[0] = (double)xr;
+        sum[1] = (double)xi;
+    } else {
+        sum[0] = (double)yr;
+        sum[1] = (double)yi;
+        sum[2] = (double)aa;
+        sum[3] = (double)xr;
+        sum[4] = (double)xi;
+        sum[5] = (double)zr;
+        sum[6] = (double)zi;
+    }
+}
+
+template <int NT, class E>
+__device__ __forceinline__ void hop_stage(const HopArgs<E> &a, const double sum[BCG_SUMS], double (*sh)[NT / 32], int k,
+                                          int bx) {
+    if (a.dot == 1)
+        bcg_partials_and_stage<NT, 0, 2>(a.dst, sum, a.dpart, a.dpart_n, a.dcnt, a.dstage, a.dmaxit, a.dflags, sh, k,
+                                         bx, a.nct);
+    else
+        bcg_partials_and_stage<NT, 0, BCG_SUMS>(a.dst, sum, a.dpart, a.dpart_n, a.dcnt, a.dstage, a.dmaxit, a.dflags,
+                                                sh, k, bx, a.nct);
+}
+
 // ALL = 1: specialised for HOP_ALL (every neighbour exists): the eight
 // neighbour indices are computed first and the eight hops run as one
 // branch-free sequence, so the compiler can issue later directions' loads
@@ -165,7 +214,7 @@ __global__ void __launch_bounds__(NT, MINB) hop_kernel(const HopArgs<typename S:
     const int half = SPLIT ? (int)(threadIdx.x >= SN) : 0;
     const long long t = (long long)bx * SN + (threadIdx.x - half * SN);
     double nrm = 0.0;
-    double d_re = 0.0, d_im = 0.0, d_aa = 0.0;  // fused BiCGStab dot partials
+    double dsum[BCG_SUMS] = {};  // fused BiCGStab dot partials
     bool work = t < total;
     int p = 0, r = 0, j = 0;
     if (work) {
@@ -313,24 +362,10 @@ __global__ void __launch_bounds__(NT, MINB) hop_kernel(const HopArgs<typename S:
         }
         store_spinor<S>(a.out.p + k * a.out.bs, a.out.cs, s - a.out.off, o);
         if (a.dot) {
-            // the BiCGStab dot product of the output: the 12 components
-            // summed in the inner precision (threads and CTAs in FP64)
-            const Spinor<R> w = a.dot == 1 ? load_spinor<S>(a.dx.p + k * a.dx.bs, a.dx.cs, s - a.dx.off)
-                                           : load_spinor<S>(a.y.p + k * a.y.bs, a.y.cs, s - a.y.off);
-            R tre = 0, tim = 0, taa = 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const cpx<R> x = a.dot == 1 ? w.c[q][c] : o.c[q][c];
-                    const cpx<R> y = a.dot == 1 ? o.c[q][c] : w.c[q][c];
-                    tre += x.re * y.re + x.im * y.im;
-                    tim += x.re * y.im - x.im * y.re;
-                    taa += x.re * x.re + x.im * x.im;
-                }
-            d_re = (double)tre;
-            d_im = (double)tim;
-            d_aa = (double)taa;
+            const Spinor<R> x = load_spinor<S>(a.dx.p + k * a.dx.bs, a.dx.cs, s - a.dx.off);
+            Spinor<R> yv;
+            if (a.dot == 2) yv = load_spinor<S>(a.y.p + k * a.y.bs, a.y.cs, s - a.y.off);
+            hop_dots(a.dot, o, x, yv, dsum);
         }
         if (a.partial) {
 #pragma unroll
@@ -344,9 +379,11 @@ __global__ void __launch_bounds__(NT, MINB) hop_kernel(const HopArgs<typename S:
         if (threadIdx.x == 0) a.partial[(long long)k * a.nct + bx] = tot;
     }
     if (a.dot) {
-        __shared__ double shd[3][NT / 32];
-        bcg_partials_and_stage<NT>(a.dst, d_re, d_im, d_aa, a.dre, a.dim, a.daa, a.dcnt, a.dstage, a.dmaxit,
-                                   a.dflags, shd, k, bx, a.nct);
+        __shared__ double shd[BCG_SUMS][NT / 32];
+        hop_stage<NT>(a, dsum, shd, k, bx);
+    }
+}
+
     }
 }
 
@@ -592,15 +629,14 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     a.dot = h.dot.dot;
     a.dx = cv(h.dot.x);
     a.dst = h.dot.st;
-    a.dre = h.dot.re;
-    a.dim = h.dot.im;
-    a.daa = h.dot.aa;
+    a.dpart = h.dot.part;
+    a.dpart_n = h.dot.part_n;
     a.dcnt = h.dot.cnt;
     a.dstage = h.dot.stage;
     a.dmaxit = h.dot.maxit;
     a.dflags = h.dot.flags;
     if (a.dot && (h.prec != P32 || h.p < 0 || !h.dot.st || !h.dot.cnt || (a.dot == 2 && !h.y.p) ||
-                  (a.dot == 1 && !h.dot.x.p)))
+                  !h.dot.x.p))
         fail(PSMS_EINVAL, "hop_launch: a fused reduction needs FP32 storage, one parity and its vectors");
     if (shared_links) {
         if (h.prec == P64 || !h.li.U1 || !h.li.ab || !h.li.flag)
@@ -627,7 +663,7 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
         // the output sites of the systems still active
         const double sp = 12.0 * sizeof(E), lk = 9.0 * sizeof(typename SL::elem);
         const double links = 4 * lk * (h.p < 0 ? 1 : 2);
-        bytes = 2 * sp + (h.y.p ? sp : 0) + (h.y2.p ? sp : 0) + (a.dot == 1 ? sp : 0) + links;
+        bytes = 2 * sp + (h.y.p ? sp : 0) + (h.y2.p ? sp : 0) + (a.dot ? sp : 0) + links;
         slot = prof_begin(c);
         a.prof_sites = prof_counter(c, slot);
     }

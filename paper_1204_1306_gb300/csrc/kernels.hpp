@@ -30,15 +30,16 @@ struct LinkInterp {
 };
 
 struct BCS;
-// A BiCGStab reduction fused into a single-parity hop (FP32 storage):
-// dot = 1 sums conj(x) out (x = the vector `x`), dot = 2 sums conj(out) y and
-// |out|^2; per-CTA partials go to re/im/aa (n_cta per system) and the last
-// CTA of each system applies the scalar `stage` to st (counters cnt).
+// A BiCGStab reduction fused into a single-parity hop (FP32 storage), x = the
+// vector `x`: dot = 1 sums conj(x) out; dot = 2 sums conj(out) y, |out|^2,
+// conj(x) out and conj(x) y.  Per-CTA partials go to part (BCG_SUMS arrays of part_n) and
+// the last CTA of each system applies the scalar `stage` to st (counters cnt).
 struct HopDot {
     int dot = 0;
     View<void> x;
     BCS *st = nullptr;
-    double *re = nullptr, *im = nullptr, *aa = nullptr;
+    double *part = nullptr;
+    long long part_n = 0;
     unsigned int *cnt = nullptr;
     int stage = 0, maxit = 0;
     int *flags = nullptr;

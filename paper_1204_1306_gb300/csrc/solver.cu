@@ -543,13 +543,15 @@ static void inner_cg_full(psms_ctx *c, int n_sys, const void *Uin, long long U_b
 // ---------------------------------------------------------------------------
 // BiCGStab on the even-odd operator Dhat (the paper leaves the solver open):
 // per system, with complex scalars kept on the device,
-//   rho = <rh, r>;  beta = (rho / rho_old)(alpha / omega);  p = r + beta (p - omega v)
 //   v = Dhat p;  alpha = rho / <rh, v>;  s = r - alpha v
-//   t = Dhat s;  omega = <t, s> / <t, t>;  x += alpha p + omega s;  r = s - omega t
-// with rh = r_0 = bhat.  A breakdown (<rh, v> = 0, omega = 0) or the
-// iteration cap ends the inner solve; the FP64 defect correction around it
-// restarts from the true residual.  Reductions: per-CTA partials in FP64,
-// finished in a fixed order (deterministic).
+//   t = Dhat s;  omega = <t, s> / <t, t>;  rho' = <rh, s> - omega <rh, t>;
+//   beta = (rho' / rho)(alpha / omega);  x += alpha p + omega s;
+//   r = s - omega t;  p = r + beta (p - omega v)
+// with rh = r_0 = bhat (rho' = <rh, r>, taken before r is formed so that x, r
+// and p are updated in one pass over the vectors).  A breakdown (<rh, v> = 0,
+// omega = 0) or the iteration cap ends the inner solve; the FP64 defect
+// correction around it restarts from the true residual.  Reductions: per-CTA
+// partials in FP64, finished in a fixed order (deterministic).
 // ---------------------------------------------------------------------------
 __global__ void bcg_init_kernel(BCS *st, const double *bb, int n, double delta, const int *act, int *flags) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -561,20 +563,17 @@ __global__ void bcg_init_kernel(BCS *st, const double *bb, int n, double delta, 
     s.rr = bb[k];
     s.target = delta * delta * bb[k];
     s.active = (act ? act[k] : 1) && bb[k] > 0.0;
-    s.iters = 0;
+    s.iters = s.stalled = 0;
     st[k] = s;
     flags[k] = s.active;
 }
 
-// mode 0: s = r - alpha v
-// mode 1: x += alpha p + omega s, r = s - omega t
-// mode 2: p = r + beta (p - omega v)
+// s = r - alpha v.  The vector kernels move whole spinors with 16-byte loads
+// and stores (one site per thread) and are bound by memory.
 template <class S, int NT>
-__global__ void __launch_bounds__(NT) bcg_axpy_kernel(const BCS *st, int mode, View<typename S::elem> x,
-                                                      View<typename S::elem> p, View<typename S::elem> r,
-                                                      View<typename S::elem> s_, View<typename S::elem> v,
-                                                      View<typename S::elem> t, long long s_lo, long long n,
-                                                      const int *map, const int *rank_active, int vbh_sh) {
+__global__ void __launch_bounds__(NT) bcg_s_kernel(const BCS *st, View<typename S::elem> r, View<typename S::elem> v,
+                                                   View<typename S::elem> s_, long long s_lo, long long n,
+                                                   const int *map, const int *rank_active, int vbh_sh) {
     using R = typename S::R;
     const int k = map ? map[blockIdx.y] : (int)blockIdx.y;
     if (!st[k].active) return;
@@ -582,99 +581,124 @@ __global__ void __launch_bounds__(NT) bcg_axpy_kernel(const BCS *st, int mode, V
     if (i >= n) return;
     if (rank_active && !rank_active[(int)(i >> vbh_sh)]) return;
     const long long sx = s_lo + i;
-    const BCS bs = st[k];
-    auto ld = [&](const View<typename S::elem> &w, int c) { return S::ldi(w.p, k * w.bs + S::idx(c, w.cs, sx - w.off)); };
-    auto st_ = [&](View<typename S::elem> &w, int c, cpx<R> val) { S::sti(w.p, k * w.bs + S::idx(c, w.cs, sx - w.off), val); };
-    const cpx<R> al = {(R)bs.alpha.x, (R)bs.alpha.y}, om = {(R)bs.omega.x, (R)bs.omega.y},
-                 be = {(R)bs.beta.x, (R)bs.beta.y};
-    for (int c = 0; c < 12; ++c) {
-        if (mode == 0) {
-            st_(s_, c, ld(r, c) - cmul(al, ld(v, c)));
-        } else if (mode == 1) {
-            const cpx<R> sv = ld(s_, c);
-            st_(x, c, ld(x, c) + cmul(al, ld(p, c)) + cmul(om, sv));
-            st_(r, c, sv - cmul(om, ld(t, c)));
-        } else {
-            st_(p, c, ld(r, c) + cmul(be, ld(p, c) - cmul(om, ld(v, c))));
-        }
-    }
+    const double2 a = st[k].alpha;
+    const cpx<R> al = {(R)a.x, (R)a.y};
+    Spinor<R> rv = load_spinor<S>(r.p + k * r.bs, r.cs, sx - r.off);
+    const Spinor<R> vv = load_spinor<S>(v.p + k * v.bs, v.cs, sx - v.off);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) rv.c[q][c] = rv.c[q][c] - cmul(al, vv.c[q][c]);
+    store_spinor<S>(s_.p + k * s_.bs, s_.cs, sx - s_.off, rv);
 }
 
-// <a, b> partials (sum conj(a) b, and |a|^2) and the scalar stage
+// the dot products of a stage over whole vectors, for storage precisions
+// whose hops do not take them: stage 0: <rh, v>; 1: <t, s>, |t|^2, <rh, t>, <rh, s>
+// (a = v or t, b = s)
 template <class S, int NT>
-__global__ void __launch_bounds__(NT) bcg_dot_stage_kernel(BCS *st, View<typename S::elem> a,
-                                                           View<typename S::elem> b, long long s_lo, long long n,
-                                                           double *p_re, double *p_im, double *p_aa,
-                                                           unsigned int *counters, int stage, int maxit, int *flags,
-                                                           const int *map, const int *rank_active, int vbh_sh) {
+__global__ void __launch_bounds__(NT) bcg_dot_stage_kernel(BCS *st, View<typename S::elem> a, View<typename S::elem> b,
+                                                           View<typename S::elem> rh, long long s_lo, long long n,
+                                                           double *part, long long part_n, unsigned int *counters,
+                                                           int stage, int maxit, int *flags, const int *map,
+                                                           const int *rank_active, int vbh_sh) {
     using R = typename S::R;
-    __shared__ double sh[3][NT / 32];
+    __shared__ double sh[BCG_SUMS][NT / 32];
     const int k = map ? map[blockIdx.y] : (int)blockIdx.y;
     if (!st[k].active) return;
-    double re = 0, im = 0, aa = 0;
+    double sum[BCG_SUMS] = {};
     const long long i = (long long)blockIdx.x * NT + threadIdx.x;
     if (i < n && (!rank_active || rank_active[(int)(i >> vbh_sh)])) {
         const long long sx = s_lo + i;
-        R tre = 0, tim = 0, taa = 0;
-        for (int c = 0; c < 12; ++c) {
-            const cpx<R> x = S::ldi(a.p, k * a.bs + S::idx(c, a.cs, sx - a.off));
-            const cpx<R> y = S::ldi(b.p, k * b.bs + S::idx(c, b.cs, sx - b.off));
-            tre += x.re * y.re + x.im * y.im;
-            tim += x.re * y.im - x.im * y.re;
-            taa += x.re * x.re + x.im * x.im;
+        const Spinor<R> av = load_spinor<S>(a.p + k * a.bs, a.cs, sx - a.off);
+        const Spinor<R> hv = load_spinor<S>(rh.p + k * rh.bs, rh.cs, sx - rh.off);
+        R xr = 0, xi = 0, yr = 0, yi = 0, aa = 0, zr = 0, zi = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const cpx<R> o = av.c[q][c], h = hv.c[q][c];
+                xr += h.re * o.re + h.im * o.im;
+                xi += h.re * o.im - h.im * o.re;
+            }
+        if (stage == 1) {
+            const Spinor<R> bv = load_spinor<S>(b.p + k * b.bs, b.cs, sx - b.off);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const cpx<R> o = av.c[q][c], y = bv.c[q][c], h = hv.c[q][c];
+                    yr += o.re * y.re + o.im * y.im;
+                    yi += o.re * y.im - o.im * y.re;
+                    aa += o.re * o.re + o.im * o.im;
+                    zr += h.re * y.re + h.im * y.im;
+                    zi += h.re * y.im - h.im * y.re;
+                }
+            sum[0] = (double)yr;
+            sum[1] = (double)yi;
+            sum[2] = (double)aa;
+            sum[3] = (double)xr;
+            sum[4] = (double)xi;
+            sum[5] = (double)zr;
+            sum[6] = (double)zi;
+        } else {
+            sum[0] = (double)xr;
+            sum[1] = (double)xi;
         }
-        re = (double)tre;
-        im = (double)tim;
-        aa = (double)taa;
     }
-    bcg_partials_and_stage<NT>(st, re, im, aa, p_re, p_im, p_aa, counters, stage, maxit, flags, sh, k,
-                               (int)blockIdx.x, (int)gridDim.x);
+    bcg_partials_and_stage<NT, 0, BCG_SUMS>(st, sum, part, part_n, counters, stage, maxit, flags, sh, k,
+                                            (int)blockIdx.x, (int)gridDim.x);
 }
 
-// x += alpha p + omega s, r = s - omega t, then the partials of
-// sum conj(r) rh and |r|^2 and scalar stage 2
+// x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), then
+// |r|^2 and stage 2.  Eight passes over memory bound it; a thread takes its
+// site unit by unit, which keeps it at few registers and the SMs full (whole
+// spinors at once: 12 % occupancy and 60 us for 12 systems at 16^4), with one
+// FP64 reduction per site (one per unit: 71 us).
 template <class S, int NT>
 __global__ void __launch_bounds__(NT) bcg_update_stage_kernel(BCS *st, View<typename S::elem> x,
                                                               View<typename S::elem> p, View<typename S::elem> r,
                                                               View<typename S::elem> s_, View<typename S::elem> t,
-                                                              View<typename S::elem> rh, long long s_lo, long long n,
-                                                              double *p_re, double *p_im, double *p_aa,
-                                                              unsigned int *counters, int maxit, int *flags,
-                                                              const int *map, const int *rank_active, int vbh_sh) {
+                                                              View<typename S::elem> v, long long s_lo, long long n,
+                                                              double *part, long long part_n, unsigned int *counters,
+                                                              int maxit, int *flags, const int *map,
+                                                              const int *rank_active, int vbh_sh) {
     using R = typename S::R;
-    __shared__ double sh[3][NT / 32];
+    constexpr int NC = 1 << S::VSH;  // complex numbers per unit
+    __shared__ double sh[BCG_SUMS][NT / 32];
     const int k = map ? map[blockIdx.y] : (int)blockIdx.y;
     if (!st[k].active) return;
-    const BCS bs = st[k];
-    const cpx<R> al = {(R)bs.alpha.x, (R)bs.alpha.y}, om = {(R)bs.omega.x, (R)bs.omega.y};
-    double re = 0, im = 0, aa = 0;
+    double sum[BCG_SUMS] = {};
     const long long i = (long long)blockIdx.x * NT + threadIdx.x;
     if (i < n && (!rank_active || rank_active[(int)(i >> vbh_sh)])) {
+        const double2 a = st[k].alpha, o = st[k].omega, b = st[k].beta;
+        const cpx<R> al = {(R)a.x, (R)a.y}, om = {(R)o.x, (R)o.y}, be = {(R)b.x, (R)b.y};
         const long long sx = s_lo + i;
-        auto ld = [&](const View<typename S::elem> &w, int c) {
-            return S::ldi(w.p, k * w.bs + S::idx(c, w.cs, sx - w.off));
-        };
-        auto stv = [&](View<typename S::elem> &w, int c, cpx<R> val) {
-            S::sti(w.p, k * w.bs + S::idx(c, w.cs, sx - w.off), val);
-        };
-        R tre = 0, tim = 0, taa = 0;
-        for (int c = 0; c < 12; ++c) {
-            const cpx<R> sv = ld(s_, c);
-            stv(x, c, ld(x, c) + cmul(al, ld(p, c)) + cmul(om, sv));
-            cpx<R> rv = sv - cmul(om, ld(t, c));
-            stv(r, c, rv);
-            rv = ld(r, c);  // the stored value (rounded to the storage precision)
-            const cpx<R> hv = ld(rh, c);
-            tre += rv.re * hv.re + rv.im * hv.im;
-            tim += rv.re * hv.im - rv.im * hv.re;
-            taa += rv.re * rv.re + rv.im * rv.im;
+        R aa = 0;
+#pragma unroll 1
+        for (int u = 0; u < 12 / NC; ++u) {
+            auto at = [&](const View<typename S::elem> &w) { return w.p + k * w.bs + (u * w.cs + sx - w.off) * NC; };
+            cpx<R> sv[NC], tv[NC], pv[NC], vv[NC], xv[NC];
+            load_unit<S>(at(s_), sv);
+            load_unit<S>(at(t), tv);
+            load_unit<S>(at(p), pv);
+            load_unit<S>(at(v), vv);
+            load_unit<S>(at(x), xv);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                xv[c] = xv[c] + cmul(al, pv[c]) + cmul(om, sv[c]);
+                const cpx<R> rv = sv[c] - cmul(om, tv[c]);
+                pv[c] = rv + cmul(be, pv[c] - cmul(om, vv[c]));
+                sv[c] = rv;
+                aa += rv.re * rv.re + rv.im * rv.im;
+            }
+            store_unit<S>(at(x), xv);
+            store_unit<S>(at(r), sv);
+            store_unit<S>(at(p), pv);
         }
-        re = (double)tre;
-        im = (double)tim;
-        aa = (double)taa;
+        sum[2] = (double)aa;
     }
-    bcg_partials_and_stage<NT>(st, re, im, aa, p_re, p_im, p_aa, counters, 2, maxit, flags, sh, k,
-                               (int)blockIdx.x, (int)gridDim.x);
+    bcg_partials_and_stage<NT, 2, 3>(st, sum, part, part_n, counters, 2, maxit, flags, sh, k, (int)blockIdx.x,
+                                     (int)gridDim.x);
 }
 
 __global__ void iters_bcg_kernel(const BCS *st, int *out, int n) {
@@ -740,9 +764,9 @@ static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long lo
     const long long n = Vh;
     const int nb = (int)((n + NT - 1) / NT);
     dim3 grid(nb, n_sys);
-    double *q_re = (double *)scratch(c, "fs_qre", sizeof(double) * (size_t)nb * n_sys);
-    double *q_im = (double *)scratch(c, "fs_qim", sizeof(double) * (size_t)nb * n_sys);
-    double *q_aa = (double *)scratch(c, "fs_qaa", sizeof(double) * (size_t)nb * n_sys);
+    // partial sums of the reductions, per CTA of the vector kernels or hops
+    const long long part_n = (long long)std::max(nb, nct) * n_sys;
+    double *part = (double *)scratch(c, "fs_part", sizeof(double) * (size_t)part_n * BCG_SUMS);
     // per-system completion counters of the fused reductions (each launch
     // leaves them at zero)
     unsigned int *cnt = (unsigned int *)scratch(c, "fs_bcnt", sizeof(unsigned int) * n_sys);
@@ -752,14 +776,8 @@ static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long lo
     // last CTA of a system applies the stage), saving two passes over two
     // vectors per iteration
     const bool fuse = prec == P32;
-    double *f_re = nullptr, *f_im = nullptr, *f_aa = nullptr;
-    if (fuse) {
-        f_re = (double *)scratch(c, "fs_fre", sizeof(double) * (size_t)nct * n_sys);
-        f_im = (double *)scratch(c, "fs_fim", sizeof(double) * (size_t)nct * n_sys);
-        f_aa = (double *)scratch(c, "fs_faa", sizeof(double) * (size_t)nct * n_sys);
-    }
     // w = Dhat u = A u + c4 H_o(H_e u); dot 1: stage 0 on <x, w>; dot 2:
-    // stage 1 on <w, u>, |w|^2
+    // stage 1 on <w, u>, |w|^2, <x, w>
     auto apply_dhat = [&](View<void> u, View<void> w, int dot, View<void> x, int stage) {
         h.dag = 0;
         h.p = 0;
@@ -781,9 +799,8 @@ static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long lo
             h.dot.dot = dot;
             h.dot.x = x;
             h.dot.st = st;
-            h.dot.re = f_re;
-            h.dot.im = f_im;
-            h.dot.aa = f_aa;
+            h.dot.part = part;
+            h.dot.part_n = part_n;
             h.dot.cnt = cnt;
             h.dot.stage = stage;
             h.dot.maxit = maxit;
@@ -810,28 +827,26 @@ static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long lo
             // alpha = rho / <rh, v>
             apply_dhat(pp, vv, 1, rh, 0);
             if (!fuse) {
-                bcg_dot_stage_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(rh), tv(vv), Vh, n, q_re, q_im, q_aa,
-                                                                          cnt, 0, maxit, flags, map, rank_active, vsh);
+                bcg_dot_stage_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(vv), tv(ss), tv(rh), Vh, n, part,
+                                                                          part_n, cnt, 0, maxit, flags, map,
+                                                                          rank_active, vsh);
                 PSMS_LAUNCH_CHECK("bcg_alpha");
             }
-            bcg_axpy_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, 0, tv(e), tv(pp), tv(r), tv(ss), tv(vv),
-                                                                 tv(tt), Vh, n, map, rank_active, vsh);
+            bcg_s_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(r), tv(vv), tv(ss), Vh, n, map, rank_active, vsh);
             PSMS_LAUNCH_CHECK("bcg_s");
-            // omega = <t, s> / <t, t>
-            apply_dhat(ss, tt, 2, View<void>(), 1);
+            // omega, rho, beta
+            apply_dhat(ss, tt, 2, rh, 1);
             if (!fuse) {
-                bcg_dot_stage_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(tt), tv(ss), Vh, n, q_re, q_im, q_aa,
-                                                                          cnt, 1, maxit, flags, map, rank_active, vsh);
+                bcg_dot_stage_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(tt), tv(ss), tv(rh), Vh, n, part,
+                                                                          part_n, cnt, 1, maxit, flags, map,
+                                                                          rank_active, vsh);
                 PSMS_LAUNCH_CHECK("bcg_omega");
             }
-            // x, r updates with <rh, r>, |r|^2 and beta / convergence
+            // x, r, p and convergence
             bcg_update_stage_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(e), tv(pp), tv(r), tv(ss), tv(tt),
-                                                                         tv(rh), Vh, n, q_re, q_im, q_aa, cnt,
-                                                                         maxit, flags, map, rank_active, vsh);
+                                                                         tv(vv), Vh, n, part, part_n, cnt, maxit,
+                                                                         flags, map, rank_active, vsh);
             PSMS_LAUNCH_CHECK("bcg_update");
-            bcg_axpy_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, 2, tv(e), tv(pp), tv(r), tv(ss), tv(vv),
-                                                                 tv(tt), Vh, n, map, rank_active, vsh);
-            PSMS_LAUNCH_CHECK("bcg_p");
         }
         cuda_check(cudaMemcpyAsync(hflags.data(), flags, sizeof(int) * n_sys, cudaMemcpyDeviceToHost, c->stream),
                    "bcg flags");
