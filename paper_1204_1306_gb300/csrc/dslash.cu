@@ -384,9 +384,6 @@ __global__ void __launch_bounds__(NT, MINB) hop_kernel(const HopArgs<typename S:
     }
 }
 
-    }
-}
-
 // Staged variant for whole-lattice launches on blocks of 2 x 128 sites (4^4):
 // one CTA per (block, output parity, system).  The block's own input sites
 // of the other parity (the neighbours of 3/4 of the hops) are copied into
