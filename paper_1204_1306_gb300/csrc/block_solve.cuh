@@ -6,6 +6,7 @@
 // they compile in parallel; solver.cu only declares them.
 #pragma once
 
+#include "fixed_hop.cuh"
 #include "kernels.hpp"
 #include "solver.hpp"
 
@@ -259,6 +260,8 @@ struct BlockSolveArgs {
     View<double2> r64;               // FP64 residual scratch (full layout)
     const double2 *U64;
     long long U64_bs;
+    const int4 *fx;                  // the FP64 links in fixed point (nullable)
+    long long fx_bs;
     const void *Uin;
     long long Uin_bs;
     void *vin;                       // inner scratch base
@@ -366,6 +369,22 @@ __device__ void block_solve_item(const BlockSolveArgs &a, const int rl, const in
                         S64::st(r64, q, a.r64.cs, s - a.r64.off, S64::ld(b, q, a.b.cs, s - a.b.off));
                 }
             rn = bn;
+        } else if (a.fx) {
+            // the same in fixed point: r64 = (b + H(x)/2) - A x in one pass
+            const FxHop h{x, a.x.cs, a.x.off, a.fx + k * a.fx_bs, HOP_INTRA, 0};
+            for (int p = 0; p < 2; ++p)
+                for (int j = jlo + threadIdx.x; j < jhi; j += NT) {
+                    const long long s = blo[p] + j;
+                    double2 hx[12];
+                    fx_site<true>(h, g, bi, r, p, j, 0.5, hx);
+                    for (int q = 0; q < 12; ++q) {
+                        const cpx<double> bv = S64::ld(b, q, a.b.cs, s - a.b.off), xv = S64::ld(x, q, a.x.cs, s - a.x.off);
+                        const cpx<double> rv = {(bv.re + hx[q].x) - A * xv.re, (bv.im + hx[q].y) - A * xv.im};
+                        S64::st(r64, q, a.r64.cs, s - a.r64.off, rv);
+                        rn += norm2(rv);
+                    }
+                }
+            rn = cl_sum<NT, CL>(rn, sh);
         } else {
         for (int p = 0; p < 2; ++p) {
             hop_call<HV, S64, S64, S64>(g, bi, r, p, 0, x, a.x.cs, a.x.off, r64, a.r64.cs, a.r64.off, b, a.b.cs,

@@ -14,6 +14,7 @@
 #define PSMS_HAVE_NVTX 1
 #endif
 #include "estimator.hpp"
+#include "fixed.cuh"
 #include "gauge.hpp"
 #include "gaugefix.hpp"
 #include "hyp.hpp"
@@ -58,6 +59,23 @@ float2 *links32(psms_ctx *c, int f) {
         c->u32_ok[f] = 1;
     }
     return c->U32[f];
+}
+
+const int4 *links_fx(psms_ctx *c, int f) {
+    check_field(c, f);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cuda_check(cudaStreamIsCapturing(c->stream, &cap), "capture status");
+    if (cap != cudaStreamCaptureStatusNone) return nullptr;
+    if (!c->Ufx[f] && cudaMalloc(&c->Ufx[f], sizeof(int4) * (size_t)fx_field(c->g.V)) != cudaSuccess) {
+        cudaGetLastError();
+        c->Ufx[f] = nullptr;
+        return nullptr;
+    }
+    if (!c->ufx_ok[f]) {
+        links_to_fx(c, c->U64[f], 0, c->Ufx[f], 1);
+        c->ufx_ok[f] = 1;
+    }
+    return c->Ufx[f];
 }
 
 int prof_begin(psms_ctx *c) {
@@ -235,6 +253,8 @@ static void free_ctx(psms_ctx *c) {
         if (p) cudaFree(p);
     for (auto p : c->U32)
         if (p) cudaFree(p);
+    for (auto p : c->Ufx)
+        if (p) cudaFree(p);
     for (auto &kv : c->scratch)
         if (kv.second.p) cudaFree(kv.second.p);
     for (auto e : c->ev_pool) cudaEventDestroy(e);
@@ -304,6 +324,8 @@ psms_status psms_create(const psms_lattice_desc *desc, psms_ctx **out) {
         c->U64.assign(c->n_fields, nullptr);
         c->U32.assign(c->n_fields, nullptr);
         c->u32_ok.assign(c->n_fields, 0);
+        c->Ufx.assign(c->n_fields, nullptr);
+        c->ufx_ok.assign(c->n_fields, 0);
         const long long n = 36 * c->g.V;
         for (int f = 0; f < c->n_fields; ++f) {
             cuda_check(cudaMalloc(&c->U64[f], sizeof(double2) * n), "gauge alloc");
@@ -561,6 +583,7 @@ psms_status psms_dw_apply(psms_ctx *ctx, int field, int op, const void *in, void
     HopCall h;
     h.prec = prec;
     h.U = links_for(ctx, field, prec);
+    if (prec == P64) h.fx = links_fx(ctx, field);
     h.in = View<void>{(void *)in, V, 0, 12 * V};
     h.out = View<void>{out, V, 0, 12 * V};
     h.y = h.in;
@@ -598,6 +621,7 @@ psms_status psms_solve(psms_ctx *ctx, int field, int op, const void *b, void *x,
         q.x = View<double2>{(double2 *)x, V, 0, 12 * V};
         q.U64 = ctx->U64[field];
         q.U32 = U32;
+        q.fx = links_fx(ctx, field);
         q.tol = tol;
         q.maxit = maxit;
         q.inner_prec = inner_prec;
@@ -621,6 +645,7 @@ psms_status psms_solve(psms_ctx *ctx, int field, int op, const void *b, void *x,
         q.x = View<double2>{(double2 *)x, V, 0, 12 * V};
         q.U64 = ctx->U64[field];
         q.U32 = U32;
+        q.fx = links_fx(ctx, field);
         q.tol = tol;
         q.maxit = maxit;
         q.inner_prec = inner_prec;

@@ -47,6 +47,8 @@ struct psms_ctx {
     std::vector<double2 *> U64;   // FP64 links per slot, [mu][e][s]
     std::vector<float2 *> U32;    // FP32 copies, valid when u32_ok
     std::vector<int> u32_ok;
+    std::vector<int4 *> Ufx;      // fixed-point copies (fixed.cuh), valid when ufx_ok
+    std::vector<int> ufx_ok;
     std::vector<psms::BlockInfo> h_binfo;
     psms::BlockInfo *d_binfo = nullptr;
     cudaStream_t stream = nullptr;
@@ -98,7 +100,12 @@ namespace psms {
 void *scratch(psms_ctx *c, const std::string &name, size_t bytes);
 // FP32 copy of a gauge slot (converted on first use after a change)
 float2 *links32(psms_ctx *c, int field);
-inline void touch_field(psms_ctx *c, int f) { c->u32_ok[f] = 0; }
+// fixed-point copy of a gauge slot, made on first use after a change; null
+// when there is no memory for it, or while the stream is captured (a graph
+// has to read the slot itself, which may change before the graph runs):
+// the caller then uses the FP64 links
+const int4 *links_fx(psms_ctx *c, int field);
+inline void touch_field(psms_ctx *c, int f) { c->u32_ok[f] = c->ufx_ok[f] = 0; }
 void check_field(psms_ctx *c, int f);
 
 // profiling hooks around Wilson-operator launches

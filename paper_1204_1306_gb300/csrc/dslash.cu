@@ -7,7 +7,10 @@
 // structure-of-arrays even-odd block-major layout, so a warp reads each
 // component of 32 consecutive sites in one coalesced transaction.
 #include "bicgstab.cuh"
+#include "fixed_hop.cuh"
 #include "kernels.hpp"
+
+#include <type_traits>
 
 namespace psms {
 
@@ -25,6 +28,8 @@ struct HopArgs {
     unsigned long long *prof_sites;  // profiling: output sites of active systems
     const int *sys_map;              // systems launched (null: all, k = blockIdx.y)
     const int *rank_active;          // per rank: 0 skips its output sites (null: none skipped)
+    const longlong2 *fxs;            // P64: the input spinors in fixed point (fixed.cuh)
+    long long fxs_bs;
     LinkInterp li;                   // shared-endpoint FP32 links (li.U0 null: U, U_bs)
     int nsf;                         // > 0: nsf systems fastest in blockIdx.x (gridDim.y = 1)
     int nct;                         // CTAs per system
@@ -86,6 +91,34 @@ __device__ __forceinline__ SU3<typename SL::R> hop_link(const HopArgs<E> &a, con
         }
     }
     return load_link<SL>(U, a.g.V, mu, idx);
+}
+
+// Output site of thread t (parity, rank, index in the block's half); false
+// when there is none or its rank is switched off.
+template <class E>
+__device__ __forceinline__ bool hop_site(const HopArgs<E> &a, const Geom &g, long long t, long long total, int &p,
+                                         int &r, int &j) {
+    p = r = j = 0;
+    if (t >= total) return false;
+    // both parities: block-major order (block, parity, site) so that the two
+    // endpoints of a block's links are processed close in time and each link
+    // is fetched from HBM about once per launch
+    const int both = a.p < 0 ? 1 : 0;
+    r = a.rank_lo + (int)(t >> (g.vbh_sh + both));
+    p = both ? (int)((t >> g.vbh_sh) & 1) : a.p;
+    j = (int)(t & (g.Vbh - 1));
+    if (a.n_ranks == g.nblocks && g.coloured) {
+        // whole lattice: walk the blocks in lexicographic order (colours
+        // interleaved), so that the faces a block reads from its neighbours
+        // were loaded by CTAs that ran just before and are still in L2
+        int B[4], rem = r;
+        for (int m = 3; m >= 0; --m) {
+            B[m] = rem % g.nb[m];
+            rem /= g.nb[m];
+        }
+        r = rank_of_lex(g, r, B);
+    }
+    return !a.rank_active || a.rank_active[r];
 }
 
 template <int NT>
@@ -215,46 +248,8 @@ __global__ void __launch_bounds__(NT, MINB) hop_kernel(const HopArgs<typename S:
     const long long t = (long long)bx * SN + (threadIdx.x - half * SN);
     double nrm = 0.0;
     double dsum[BCG_SUMS] = {};  // fused BiCGStab dot partials
-    bool work = t < total;
-    int p = 0, r = 0, j = 0;
-    if (work) {
-        // both parities: block-major order (block, parity, site) so that the
-        // two endpoints of a block's links are processed close in time and
-        // each link is fetched from HBM about once per launch
-        if (a.p < 0) {
-            r = a.rank_lo + (int)(t >> (g.vbh_sh + 1));
-            p = (int)((t >> g.vbh_sh) & 1);
-            j = (int)(t & (g.Vbh - 1));
-            if (a.n_ranks == g.nblocks) {
-                // whole lattice: walk the blocks in lexicographic order, so
-                // that a block's neighbours (opposite colour) are processed
-                // soon after it and face data is still in L2
-                int B[4], rem = r;
-                for (int m = 3; m >= 0; --m) {
-                    B[m] = rem % g.nb[m];
-                    rem /= g.nb[m];
-                }
-                r = rank_of_lex(g, r, B);
-            }
-        } else {
-            p = a.p;
-            r = a.rank_lo + (int)(t >> g.vbh_sh);
-            j = (int)(t & (g.Vbh - 1));
-            if (a.n_ranks == g.nblocks && g.coloured) {
-                // whole lattice, one parity: walk the blocks in lexicographic
-                // order (colours interleaved), so that the faces a block
-                // reads from its neighbours were loaded by CTAs that ran
-                // just before and are still in L2
-                int B[4], rem = r;
-                for (int m = 3; m >= 0; --m) {
-                    B[m] = rem % g.nb[m];
-                    rem /= g.nb[m];
-                }
-                r = rank_of_lex(g, r, B);
-            }
-        }
-        work = !a.rank_active || a.rank_active[r];
-    }
+    int p, r, j;
+    bool work = hop_site(a, g, t, total, p, r, j);
     if (a.prof_sites) {
         // output sites this warp computes (algorithmic-byte accounting)
         const unsigned cnt = __popc(__ballot_sync(0xffffffffu, work && !half));
@@ -381,6 +376,188 @@ __global__ void __launch_bounds__(NT, MINB) hop_kernel(const HopArgs<typename S:
     if (a.dot) {
         __shared__ double shd[BCG_SUMS][NT / 32];
         hop_stage<NT>(a, dsum, shd, k, bx);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// FP64 hops in fixed point (fixed.cuh, fixed_hop.cuh)
+// ---------------------------------------------------------------------------
+// The spinors a hop reads, in fixed point: n sites from `in` (sites [0, cs) of
+// a field) of the launched systems.  A pass of its own, so that a site is
+// converted once and not by each of its eight neighbours (the conversion is
+// two thirds of a hop's instructions).
+__global__ void __launch_bounds__(256) spinor_fx_kernel(View<double2> in, longlong2 *out, long long out_bs,
+                                                        const int *sys_map, const int *active) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    const int k = sys_map ? sys_map[blockIdx.y] : (int)blockIdx.y;
+    if (i >= in.cs || (active && !active[k])) return;
+    int64_t v[12][2];
+    const int e = fx_load_spinor(in.p + k * in.bs + i, in.cs, v);
+    longlong2 *o = out + k * out_bs;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) o[c * in.cs + i] = make_longlong2(v[c][0], v[c][1]);
+    reinterpret_cast<uint16_t *>(o + 12 * in.cs)[i] = (uint16_t)e;
+}
+
+// one output site in FP64 (numbers out of the fixed-point range); |out|^2
+static __device__ __noinline__ double hop_f64_site(const HopArgs<double2> &a, const FxHop &h, const BlockInfo &bi, int k,
+                                                   int r, int p, int j) {
+    const long long s = (long long)p * a.g.Vh + (long long)r * a.g.Vbh + j;
+    double2 o[12];
+    fx_site_f64(h, a.g, bi, r, p, j, o);
+    double nrm = 0.0;
+    for (int c = 0; c < 12; ++c) {
+        double re = a.b * o[c].x, im = a.b * o[c].y;
+        if (a.y.p) {
+            const double2 w = a.y.p[k * a.y.bs + c * a.y.cs + s - a.y.off];
+            re = fma(a.a, w.x, re);
+            im = fma(a.a, w.y, im);
+        }
+        if (a.y2.p) {
+            const double2 w = a.y2.p[k * a.y2.bs + c * a.y2.cs + s - a.y2.off];
+            re = fma(a.a2, w.x, re);
+            im = fma(a.a2, w.y, im);
+        }
+        a.out.p[k * a.out.bs + c * a.out.cs + s - a.out.off] = make_double2(re, im);
+        nrm = fma(re, re, fma(im, im, nrm));
+    }
+    return nrm;
+}
+
+// One thread per output site: b (sum of hops) in integers, a y + a2 y2 and
+// the result in FP64.
+template <int NT, int MINB, bool DAG>
+__global__ void __launch_bounds__(NT, MINB) hop_fx_kernel(const HopArgs<double2> a) {
+    __shared__ double sh[NT / 32];
+    const int ks = (int)blockIdx.y, bx = (int)blockIdx.x;
+    const int k = a.sys_map ? a.sys_map[ks] : ks;
+    if (a.active && !a.active[k]) {
+        if (a.partial && threadIdx.x == 0) a.partial[(long long)k * a.nct + bx] = 0.0;
+        return;
+    }
+    const Geom &g = a.g;
+    const long long total = (a.p < 0 ? 2 : 1) * (long long)a.n_ranks * g.Vbh;
+    int p, r, j;
+    const bool work = hop_site(a, g, (long long)bx * NT + threadIdx.x, total, p, r, j);
+    if (a.prof_sites) {
+        const unsigned cnt = __popc(__ballot_sync(0xffffffffu, work));
+        if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(a.prof_sites, (unsigned long long)cnt);
+    }
+    double nrm = 0.0;
+    if (work) {
+        const long long s = (long long)p * g.Vh + (long long)r * g.Vbh + j;
+        int y[4];
+        const int ll = local_lex(g, p, j, y);
+        const BlockInfo &bi = a.binfo[r];
+        const FxHop h{a.in.p + k * a.in.bs, a.in.cs, a.in.off, (const int4 *)a.U + k * a.U_bs, a.mode, a.dag,
+                      a.fxs + k * a.fxs_bs, a.in.cs, a.in.off};
+        FxAcc acc;
+        fx_zero(acc);
+        double f;
+        if (fx_dirs<false, DAG>(h, g, bi, r, p, y, ll, s, acc) && fx_factor(acc, a.b, f)) {
+            const double2 *yv = a.y.p ? a.y.p + k * a.y.bs + s - a.y.off : nullptr;
+            const double2 *y2v = a.y2.p ? a.y2.p + k * a.y2.bs + s - a.y2.off : nullptr;
+            double2 *o = a.out.p + k * a.out.bs + s - a.out.off;
+#pragma unroll
+            for (int c = 0; c < 12; ++c) {
+                const int64_t *v = c < 6 ? acc.up[c / 3][c % 3] : acc.dn[(c - 6) / 3][c % 3];
+                double re = f * (double)v[0], im = f * (double)v[1];
+                if (yv) {
+                    const double2 w = yv[c * a.y.cs];
+                    re = fma(a.a, w.x, re);
+                    im = fma(a.a, w.y, im);
+                }
+                if (y2v) {
+                    const double2 w = y2v[c * a.y2.cs];
+                    re = fma(a.a2, w.x, re);
+                    im = fma(a.a2, w.y, im);
+                }
+                o[c * a.out.cs] = make_double2(re, im);
+                if (a.partial) nrm = fma(re, re, fma(im, im, nrm));
+            }
+        } else {
+            nrm = hop_f64_site(a, h, bi, k, r, p, j);
+        }
+    }
+    if (a.partial) {
+        const double tot = block_sum<NT>(nrm, sh);
+        if (threadIdx.x == 0) a.partial[(long long)k * a.nct + bx] = tot;
+    }
+}
+
+// Small launches: one warp per direction, 32 sites per CTA.  The eight
+// partial sums meet in shared memory on their largest exponent, and warp w
+// finishes components 3 w .. 3 w + 2.  (No partial sums of the norm.)
+struct FxSplitShared {
+    int64_t v[24][8][32];
+    int E[8][32], ok[8][32];
+};
+
+template <bool DAG>
+__global__ void __launch_bounds__(256) hop_fx_split_kernel(const HopArgs<double2> a) {
+    extern __shared__ __align__(16) unsigned char fx_smem[];
+    FxSplitShared &sm = *reinterpret_cast<FxSplitShared *>(fx_smem);
+    const int k = a.sys_map ? a.sys_map[blockIdx.y] : (int)blockIdx.y;
+    if (a.active && !a.active[k]) return;
+    const Geom &g = a.g;
+    const int d = (int)(threadIdx.x >> 5), l = (int)(threadIdx.x & 31);
+    const long long total = (a.p < 0 ? 2 : 1) * (long long)a.n_ranks * g.Vbh;
+    int p, r, j;
+    const bool work = hop_site(a, g, (long long)blockIdx.x * 32 + l, total, p, r, j);
+    if (a.prof_sites && d == 0) {
+        const unsigned cnt = __popc(__ballot_sync(0xffffffffu, work));
+        if (l == 0 && cnt) atomicAdd(a.prof_sites, (unsigned long long)cnt);
+    }
+    const long long s = (long long)p * g.Vh + (long long)r * g.Vbh + j;
+    const FxHop h{a.in.p + k * a.in.bs, a.in.cs, a.in.off, (const int4 *)a.U + k * a.U_bs, a.mode, a.dag};
+    FxAcc acc;
+    fx_zero(acc);
+    bool ok = true;
+    if (work) {
+        int y[4];
+        const int ll = local_lex(g, p, j, y);
+        const uint64_t yp = (uint64_t)y[0] | (uint64_t)y[1] << 16 | (uint64_t)y[2] << 32 | (uint64_t)y[3] << 48;
+        ok = fx_dir<true, DAG>(h, g, a.binfo[r], r, p, yp, ll, s, d, acc);
+    }
+    sm.E[d][l] = acc.E;
+    sm.ok[d][l] = ok;
+    __syncthreads();
+    int E = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        E = max(E, sm.E[w][l]);
+        ok = ok && sm.ok[w][l];
+    }
+    const int sft = min(E - acc.E, 63);
+#pragma unroll
+    for (int c = 0; c < 12; ++c)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            sm.v[2 * c + i][d][l] = (c < 6 ? acc.up[c / 3][c % 3][i] : acc.dn[(c - 6) / 3][c % 3][i]) >> sft;
+    __syncthreads();
+    if (!work) return;
+    acc.E = E;
+    double f = a.b;
+    ok = ok && fx_factor(acc, a.b, f);
+    double2 slow[12];
+    if (!ok) fx_site_f64(h, g, a.binfo[r], r, p, j, slow);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int n = 3 * d + i, c = n >> 1, im = n & 1;  // real number n of the site's 24
+        int64_t t = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += sm.v[n][w][l];
+        double o = f * (double)t;
+        if (!ok) o = a.b * (im ? slow[c].y : slow[c].x);
+        if (a.y.p) {
+            const double2 v = a.y.p[k * a.y.bs + c * a.y.cs + s - a.y.off];
+            o = fma(a.a, im ? v.y : v.x, o);
+        }
+        if (a.y2.p) {
+            const double2 v = a.y2.p[k * a.y2.bs + c * a.y2.cs + s - a.y2.off];
+            o = fma(a.a2, im ? v.y : v.x, o);
+        }
+        reinterpret_cast<double *>(a.out.p + k * a.out.bs + c * a.out.cs + s - a.out.off)[im] = o;
     }
 }
 
@@ -581,6 +758,7 @@ __global__ void __launch_bounds__(NT, MINB) hop_staged_kernel(const HopArgs<type
 }
 
 static constexpr int HOP_NT = 128;
+constexpr long long FX_SPLIT_SITES = 152 * 128;  // output sites of all systems
 
 int hop_ctas(psms_ctx *c, const HopCall &h) {
     const int nr = h.n_ranks < 0 ? c->g.nblocks : h.n_ranks;
@@ -621,6 +799,8 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     a.prof_sites = nullptr;
     a.sys_map = h.sys_map;
     a.rank_active = h.rank_active;
+    a.fxs = nullptr;
+    a.fxs_bs = 0;
     const bool shared_links = h.li.U0 != nullptr;
     a.li = h.li;
     a.dot = h.dot.dot;
@@ -643,6 +823,11 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     }
     const int nct = hop_ctas(c, h);
     const int nsys = h.sys_map ? h.n_map : h.n_sys;
+    const bool fixed = std::is_same<S, Store<double>>::value && h.fx != nullptr;
+    if (fixed) {
+        a.U = h.fx;
+        a.U_bs = h.fx_bs;
+    }
     if (nct == 0 || nsys == 0) return 0;
     a.nct = nct;
     // shared-endpoint links: the systems of a launch run side by side (CTA
@@ -663,6 +848,34 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
         bytes = 2 * sp + (h.y.p ? sp : 0) + (h.y2.p ? sp : 0) + (a.dot ? sp : 0) + links;
         slot = prof_begin(c);
         a.prof_sites = prof_counter(c, slot);
+    }
+    if constexpr (std::is_same<S, Store<double>>::value) {
+        if (fixed) {
+            // FP64 hops in fixed point (fixed.cuh).  Few output sites (below
+            // four warps per scheduler over the chip), or a few blocks of a
+            // large lattice: the directions of a site go to eight warps, which
+            // convert what they read; else a pass converts the input first
+            const long long per = (h.p < 0 ? 2LL : 1LL) * a.n_ranks * c->g.Vbh;
+            if (!h.partial && (per * nsys <= FX_SPLIT_SITES || 8LL * a.n_ranks <= c->g.nblocks)) {
+                const auto fn = h.dag ? hop_fx_split_kernel<true> : hop_fx_split_kernel<false>;
+                cuda_check(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)sizeof(FxSplitShared)),
+                           "hop shared memory");
+                fn<<<dim3((unsigned)((per + 31) / 32), nsys), 256, sizeof(FxSplitShared), c->stream>>>(a);
+            } else {
+                const long long fs = fx_spinors(a.in.cs);
+                longlong2 *x = (longlong2 *)scratch(c, "hop_fx", sizeof(longlong2) * (size_t)fs * h.n_sys);
+                spinor_fx_kernel<<<dim3((unsigned)((a.in.cs + 255) / 256), nsys), 256, 0, c->stream>>>(a.in, x, fs, h.sys_map,
+                                                                                                   h.active);
+                PSMS_LAUNCH_CHECK("spinor_fx_kernel");
+                a.fxs = x;
+                a.fxs_bs = fs;
+                (h.dag ? hop_fx_kernel<HOP_NT, 3, true> : hop_fx_kernel<HOP_NT, 3, false>)<<<grid, HOP_NT, 0, c->stream>>>(a);
+            }
+            PSMS_LAUNCH_CHECK("hop_fx_kernel");
+            if (slot >= 0) prof_end(c, slot, bytes);
+            return nct;
+        }
     }
     // Register cap (minimum resident CTAs per SM) chosen by the autotuner:
     // on the first launch of each (precision, parity shape) every variant is

@@ -13,6 +13,7 @@
 // All interpolation steps i are batched into every launch (system index =
 // i), and all blocks of a level are solved by one persistent launch.
 #include "estimator.hpp"
+#include "fixed.cuh"
 #include "interp_plan.hpp"
 #include "gauge.hpp"
 #include "solver.hpp"
@@ -166,52 +167,52 @@ static void check_status(psms_ctx *c, const int *d_status, int n, const char *wh
         if (v) fail(PSMS_ENOCONV, std::string(what) + ": a block solve missed its tolerance");
 }
 
-// interpolated link fields U_0..U_N (FP64, FP32 when needed) in scratch
+// interpolated link fields U_0..U_N in scratch: in fixed point (the FP64 hops
+// and true residuals), FP64 or FP32 (the inner iterations of the block solver)
 struct Interp {
+    int4 *fx;
     double2 *u64;
     float2 *u32;
-    long long bs;  // complex elements per field
+    long long bs;  // complex elements per FP64 / FP32 field
 };
 
 // fields U_{i0} .. U_{i0+n} of Eq. (gfparam) (or U, U' in the independent mode)
-static Interp make_interp(psms_ctx *c, const double2 *U, const double2 *Up, int N, int mode, bool need32,
+static Interp make_interp(psms_ctx *c, const double2 *U, const double2 *Up, int N, int mode, int inner,
                           const char *tag, int i0, int n) {
     const long long nel = 36 * c->g.V;
     Interp it;
     it.bs = nel;
     const int nf = (mode == PSMS_EST_INDEPENDENT) ? 2 : n + 1;
-    it.u64 = (double2 *)scratch(c, std::string("interp64_") + tag, sizeof(double2) * nel * nf);
-    it.u32 = need32 ? (float2 *)scratch(c, std::string("interp32_") + tag, sizeof(float2) * nel * nf) : nullptr;
+    it.fx = (int4 *)scratch(c, std::string("interpfx_") + tag, sizeof(int4) * fx_field(c->g.V) * nf);
+    it.u64 = inner == P64 ? (double2 *)scratch(c, std::string("interp64_") + tag, sizeof(double2) * nel * nf) : nullptr;
+    it.u32 = inner != P64 ? (float2 *)scratch(c, std::string("interp32_") + tag, sizeof(float2) * nel * nf) : nullptr;
     if (mode == PSMS_EST_INDEPENDENT) {
-        interpolate(c, U, Up, it.u64, it.u32, 1, 0, 2);  // field 0 = U, field 1 = U'
+        interpolate(c, U, Up, it.u64, it.u32, 1, 0, 2, it.fx);  // field 0 = U, field 1 = U'
     } else {
-        interpolate(c, U, Up, it.u64, it.u32, N, i0, n + 1);
+        interpolate(c, U, Up, it.u64, it.u32, N, i0, n + 1, it.fx);
     }
     return it;
 }
 
-// link pointers for op(U_i) (first) and op(U_{i+1}) (second) of system i
-struct Pair {
-    const double2 *a64, *b64;
-    const float2 *a32, *b32;
-    long long bs;
+// links of one operator for every system of a chunk
+struct OpLinks {
+    const int4 *fx;
+    const double2 *u64;
+    const float2 *u32;
+    long long bs, fx_bs;  // between the systems
 };
-static Pair pair_of(const Interp &it, int mode) {
-    Pair p;
-    if (mode == PSMS_EST_INDEPENDENT) {
-        p.a64 = it.u64;
-        p.b64 = it.u64 + it.bs;
-        p.a32 = it.u32;
-        p.b32 = it.u32 ? it.u32 + it.bs : nullptr;
-        p.bs = 0;
-    } else {
-        p.a64 = it.u64;
-        p.b64 = it.u64 + it.bs;
-        p.a32 = it.u32;
-        p.b32 = it.u32 ? it.u32 + it.bs : nullptr;
-        p.bs = it.bs;
-    }
-    return p;
+
+// op(U_i) (second = 0) and op(U_{i+1}) (second = 1) of system i
+static OpLinks links_of(psms_ctx *c, const Interp &it, int mode, int second) {
+    const long long fs = fx_field(c->g.V);
+    const bool ind = mode == PSMS_EST_INDEPENDENT;
+    OpLinks l;
+    l.fx = it.fx + second * fs;
+    l.u64 = it.u64 ? it.u64 + second * it.bs : nullptr;
+    l.u32 = it.u32 ? it.u32 + second * it.bs : nullptr;
+    l.bs = ind ? 0 : it.bs;
+    l.fx_bs = ind ? 0 : fs;
+    return l;
 }
 
 static long long block_level_chunk(psms_ctx *c, const double2 *U, const double2 *Up, int N, int i0, int n, int mode,
@@ -221,8 +222,8 @@ static long long block_level_chunk(psms_ctx *c, const double2 *U, const double2 
     const long long V = g.V;
     const long long fs = 12 * V;
     const int nr = g.nblocks;
-    Interp it = make_interp(c, U, Up, N, mode, inner != P64, "blk", i0, n);
-    Pair pr = pair_of(it, mode);
+    const Interp it = make_interp(c, U, Up, N, mode, inner, "blk", i0, n);
+    const OpLinks la = links_of(c, it, mode, 0), lb = links_of(c, it, mode, 1);
     double2 *xi = (double2 *)scratch(c, "bl_xi", sizeof(double2) * fs * n);
     double2 *eta = (double2 *)scratch(c, "bl_eta", sizeof(double2) * fs * n);
     double2 *ysol = (double2 *)scratch(c, "bl_y", sizeof(double2) * fs * n);
@@ -230,8 +231,8 @@ static long long block_level_chunk(psms_ctx *c, const double2 *U, const double2 
     // eta_i = D_blk(U_i) xi_i = A xi - H_intra(xi)/2
     HopCall h;
     h.prec = P64;
-    h.U = pr.a64;
-    h.U_bs = pr.bs;
+    h.fx = la.fx;
+    h.fx_bs = la.fx_bs;
     h.n_sys = n;
     h.p = -1;
     h.mode = HOP_INTRA;
@@ -252,9 +253,11 @@ static long long block_level_chunk(psms_ctx *c, const double2 *U, const double2 
     q.n_sys = n;
     q.b = View<double2>{eta, V, 0, fs};
     q.x = View<double2>{ysol, V, 0, fs};
-    q.U64 = pr.b64;
-    q.U32 = pr.b32;
-    q.U64_bs = pr.bs;
+    q.U64 = lb.u64;
+    q.U32 = lb.u32;
+    q.U64_bs = lb.bs;
+    q.fx = lb.fx;
+    q.fx_bs = lb.fx_bs;
     q.tol = tol;
     q.inner_prec = inner;
     q.iters = iters;
@@ -288,9 +291,9 @@ long long block_level(psms_ctx *c, const double2 *U, const double2 *Up, int N, i
     return tot;
 }
 
-// v = (1 - P Q(U_i)) xi for all systems; links per system via Pair (first = U_i)
-static long long one_minus_PQ(psms_ctx *c, const double2 *U64, const float2 *U32, long long Ubs, int N,
-                              const double2 *xi, double2 *v, double tol, int inner) {
+// v = (1 - P Q(U_i)) xi for all systems
+static long long one_minus_PQ(psms_ctx *c, const OpLinks &l, int N, const double2 *xi, double2 *v, double tol,
+                              int inner) {
     const Geom &g = c->g;
     const long long V = g.V, fs = 12 * V;
     const int nbh = g.nbh;
@@ -308,9 +311,11 @@ static long long one_minus_PQ(psms_ctx *c, const double2 *U64, const float2 *U32
         q.n_sys = N;
         q.b = View<double2>{b, V, 0, fs};
         q.x = View<double2>{x, V, 0, fs};
-        q.U64 = U64;
-        q.U32 = U32;
-        q.U64_bs = Ubs;
+        q.U64 = l.u64;
+        q.U32 = l.u32;
+        q.U64_bs = l.bs;
+        q.fx = l.fx;
+        q.fx_bs = l.fx_bs;
         q.tol = tol;
         q.inner_prec = inner;
         q.iters = iters;
@@ -328,8 +333,8 @@ static long long one_minus_PQ(psms_ctx *c, const double2 *U64, const float2 *U32
     // block iterations are returned in whole-lattice-equivalent units below
     HopCall h;
     h.prec = P64;
-    h.U = U64;
-    h.U_bs = Ubs;
+    h.fx = l.fx;
+    h.fx_bs = l.fx_bs;
     h.n_sys = N;
     h.p = -1;
     h.mode = HOP_INTER;
@@ -355,9 +360,8 @@ static long long one_minus_PQ(psms_ctx *c, const double2 *U64, const float2 *U32
 }
 
 // w = (1 - P Q(U_{i+1}))^-1 v = v - P [D^-1 (0, D_wb v)]_black
-static long long inv_one_minus_PQ(psms_ctx *c, const double2 *U64, const float2 *U32, const LinkInterp &li,
-                                  long long Ubs, int N,
-                                  const double2 *v, double2 *w, double tol, int inner) {
+static long long inv_one_minus_PQ(psms_ctx *c, const OpLinks &l, const LinkInterp &li, int N, const double2 *v,
+                                  double2 *w, double tol, int inner) {
     const Geom &g = c->g;
     const long long V = g.V, fs = 12 * V;
     double2 *y = (double2 *)scratch(c, "ipq_y", sizeof(double2) * fs * N);
@@ -365,8 +369,8 @@ static long long inv_one_minus_PQ(psms_ctx *c, const double2 *U64, const float2 
     cuda_check(cudaMemsetAsync(y, 0, sizeof(double2) * fs * N, c->stream), "ipq memset");
     HopCall h;
     h.prec = P64;
-    h.U = U64;
-    h.U_bs = Ubs;
+    h.fx = l.fx;
+    h.fx_bs = l.fx_bs;
     h.n_sys = N;
     h.p = -1;
     h.mode = HOP_INTER;
@@ -380,10 +384,12 @@ static long long inv_one_minus_PQ(psms_ctx *c, const double2 *U64, const float2 
     q.n_sys = N;
     q.b = View<double2>{y, V, 0, fs};
     q.x = View<double2>{z, V, 0, fs};
-    q.U64 = U64;
-    q.U32 = U32;
+    q.U64 = l.u64;
+    q.U32 = l.u32;
     q.li32 = li;
-    q.U64_bs = Ubs;
+    q.U64_bs = l.bs;
+    q.fx = l.fx;
+    q.fx_bs = l.fx_bs;
     q.tol = tol;
     q.inner_prec = inner;
     psms_solve_info info;
@@ -440,13 +446,13 @@ static long long global_level_chunk(psms_ctx *c, const double2 *U, const double2
                                     double *h_delta) {
     const Geom &g = c->g;
     const long long V = g.V, fs = 12 * V;
-    Interp it = make_interp(c, U, Up, N, mode, inner != P64, "glb", i0, n);
-    Pair pr = pair_of(it, mode);
+    const Interp it = make_interp(c, U, Up, N, mode, inner, "glb", i0, n);
+    const OpLinks la = links_of(c, it, mode, 0), lb = links_of(c, it, mode, 1);
     double2 *xi = (double2 *)scratch(c, "gl_xi", sizeof(double2) * fs * n);
     double2 *v = (double2 *)scratch(c, "gl_v", sizeof(double2) * fs * n);
     double2 *w = (double2 *)scratch(c, "gl_w", sizeof(double2) * fs * n);
     noise(c, xi, n, seed, counter, PSMS_LEVEL_GLOBAL, 1, i0);
-    long long tot = one_minus_PQ(c, pr.a64, pr.a32, pr.bs, n, xi, v, tol, inner);
+    long long tot = one_minus_PQ(c, la, n, xi, v, tol, inner);
     // the whole-lattice FP32 solves read shared endpoint links (op(U_{i+1}))
     LinkInterp li;
     if (inner != P64 && c->shared_links) {
@@ -454,7 +460,7 @@ static long long global_level_chunk(psms_ctx *c, const double2 *U, const double2
         interpolate(c, U, Up, e64, nullptr, 1, 0, 2);
         li = link_interp(c, shared_ends(c, e64, "glb"), N, i0, n, 1, mode, "glb");
     }
-    tot += inv_one_minus_PQ(c, pr.b64, pr.b32, li, pr.bs, n, v, w, tol, inner);
+    tot += inv_one_minus_PQ(c, lb, li, n, v, w, tol, inner);
     double *nw = (double *)scratch(c, "gl_nw", sizeof(double) * n);
     double *nx = (double *)scratch(c, "gl_nx", sizeof(double) * n);
     norm2_batch(c, P64, View<void>{w, V, 0, fs}, 0, V, n, nw);

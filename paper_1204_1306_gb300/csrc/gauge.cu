@@ -3,6 +3,7 @@
 // (checkerboard Cabibbo-Marinari heatbath and overrelaxation on the active
 // links of Sec. 3), random translation, the interpolation of Eq. (gfparam)
 // and the merge of accepted blocks.
+#include "fixed.cuh"
 #include "gauge.hpp"
 
 #include <cmath>
@@ -558,10 +559,10 @@ void translate(psms_ctx *c, const double2 *src, double2 *dst, const int sh[4]) {
 // FP32 link element index of the FP64 element t = (mu * 9 + e) * V + s
 // U_i = ((N - i)/N) U + (i/N) U' for i = i0 .. i0 + n - 1, one thread per
 // link: the link of both endpoints is read once, every system's FP64 copy
-// ([mu][e][s]) and FP32 copy (four 16-byte units of element pairs, then
-// element 8) are written with full coalesced stores
-__global__ void interp_kernel(const double2 *U, const double2 *Up, double2 *out64, float2 *out32, int N, int i0,
-                              int n, long long V) {
+// ([mu][e][s]), FP32 copy (four 16-byte units of element pairs, then element
+// 8) and fixed-point copy (fixed.cuh), as asked for, are written with full coalesced stores
+__global__ void interp_kernel(const double2 *U, const double2 *Up, double2 *out64, float2 *out32, int4 *outfx, int N,
+                              int i0, int n, long long V) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 4 * V) return;
     const int mu = (int)(t / V);
@@ -579,6 +580,16 @@ __global__ void interp_kernel(const double2 *U, const double2 *Up, double2 *out6
         double2 w[9];
 #pragma unroll
         for (int e = 0; e < 9; ++e) w[e] = make_double2(a * u[e].x + b * v[e].x, a * u[e].y + b * v[e].y);
+        if (outfx) {
+            int4 *o = outfx + k * fx_field(V);
+            cpx<double> x[9];
+            int4 q[9];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) x[e] = {w[e].x, w[e].y};
+            fx_exps(o, V)[t] = (uint16_t)fx_link(x, q);
+#pragma unroll
+            for (int e = 0; e < 9; ++e) o[((long long)mu * 9 + e) * V + s] = q[e];
+        }
         if (out64) {
 #pragma unroll
             for (int e = 0; e < 9; ++e) out64[(long long)k * n_el + ((long long)mu * 9 + e) * V + s] = w[e];
@@ -596,9 +607,9 @@ __global__ void interp_kernel(const double2 *U, const double2 *Up, double2 *out6
 }
 
 void interpolate(psms_ctx *c, const double2 *U, const double2 *Up, double2 *out64, float2 *out32, int N, int i0,
-                 int n) {
+                 int n, int4 *outfx) {
     const long long nl = 4 * c->g.V;
-    interp_kernel<<<(unsigned)((nl + 255) / 256), 256, 0, c->stream>>>(U, Up, out64, out32, N, i0, n, c->g.V);
+    interp_kernel<<<(unsigned)((nl + 255) / 256), 256, 0, c->stream>>>(U, Up, out64, out32, outfx, N, i0, n, c->g.V);
     PSMS_LAUNCH_CHECK("interpolate");
 }
 
@@ -625,6 +636,33 @@ void links_to_f32(psms_ctx *c, const double2 *a, float2 *b, long long n_el) {
     const long long V = n_el / 36;
     to_f32_kernel<<<(unsigned)((4 * V + 255) / 256), 256, 0, c->stream>>>(a, b, V);
     PSMS_LAUNCH_CHECK("links_to_f32");
+}
+
+// fixed-point copy (fixed.cuh) of FP64 link fields, one thread per link;
+// blockIdx.y: field
+__global__ void to_fx_kernel(const double2 *src, long long src_bs, int4 *dst, long long V) {
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 4 * V) return;
+    const int mu = (int)(t / V);
+    const long long s = t - (long long)mu * V;
+    const double2 *q = src + blockIdx.y * src_bs + (long long)mu * 9 * V + s;
+    int4 *o = dst + blockIdx.y * fx_field(V);
+    cpx<double> u[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        const double2 v = q[(long long)e * V];
+        u[e] = {v.x, v.y};
+    }
+    int4 w[9];
+    fx_exps(o, V)[t] = (uint16_t)fx_link(u, w);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) o[((long long)mu * 9 + e) * V + s] = w[e];
+}
+
+void links_to_fx(psms_ctx *c, const double2 *src, long long src_bs, int4 *dst, int n_fields) {
+    const long long V = c->g.V;
+    to_fx_kernel<<<dim3((unsigned)((4 * V + 255) / 256), n_fields), 256, 0, c->stream>>>(src, src_bs, dst, V);
+    PSMS_LAUNCH_CHECK("links_to_fx");
 }
 
 // dst = old, except active links of blocks with accept[lex] != 0 taken from prop

@@ -56,6 +56,10 @@ struct HopCall {
     double a = 0, a2 = 0, b = 1;
     const void *U = nullptr;
     long long U_bs = 0;
+    // P64: the links in fixed point (fixed.cuh; replace U / U_bs, strides in
+    // 16-byte elements); null: FP64 links
+    const int4 *fx = nullptr;
+    long long fx_bs = 0;
     int p = -1, rank_lo = 0, n_ranks = -1, mode = HOP_ALL, dag = 0, n_sys = 1;
     const int *active = nullptr;
     double *partial = nullptr;

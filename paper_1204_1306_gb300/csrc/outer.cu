@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "estimator.hpp"
+#include "fixed.cuh"
 #include "gauge.hpp"
 #include "outer.cuh"
 #include "outer.hpp"
@@ -171,6 +172,7 @@ void sub_projected(psms_ctx *c, int mode, double2 *out, const double2 *y, double
 // FP64 and, when asked, their FP32 copies
 struct LinkSet {
     double2 *u64 = nullptr;
+    int4 *fx = nullptr;
     float2 *u32 = nullptr;
     long long nel = 0;
     int nf = 0;
@@ -187,6 +189,8 @@ LinkSet make_links(psms_ctx *c, const double2 *U, const double2 *Up, int N, int 
     else
         interpolate(c, U, Up, ls.u64, nullptr, N, i0, n + 1);
     if (kind) mask_links(c, ls.u64, ls.nel, ls.nf, kind);
+    ls.fx = (int4 *)scratch(c, std::string("olfx_") + tag, sizeof(int4) * fx_field(c->g.V) * ls.nf);
+    links_to_fx(c, ls.u64, ls.nel, ls.fx, ls.nf);
     if (need32) {
         ls.u32 = (float2 *)scratch(c, std::string("ol32_") + tag, sizeof(float2) * ls.nel * ls.nf);
         for (int f = 0; f < ls.nf; ++f) links_to_f32(c, ls.u64 + f * ls.nel, ls.u32 + f * ls.nel, ls.nel);
@@ -199,7 +203,8 @@ LinkSet make_links(psms_ctx *c, const double2 *U, const double2 *Up, int N, int 
 struct LP {
     const double2 *a64, *b64;
     const float2 *a32, *b32;
-    long long bs;
+    const int4 *afx, *bfx;
+    long long bs, fx_bs;
 };
 
 LP pair_of(const LinkSet &ls, int mode) {
@@ -209,6 +214,10 @@ LP pair_of(const LinkSet &ls, int mode) {
     p.a32 = ls.u32;
     p.b32 = ls.u32 ? ls.u32 + ls.nel : nullptr;
     p.bs = mode == PSMS_EST_INDEPENDENT ? 0 : ls.nel;
+    const long long fs = fx_field(ls.nel / 36);
+    p.afx = ls.fx;
+    p.bfx = ls.fx + fs;
+    p.fx_bs = mode == PSMS_EST_INDEPENDENT ? 0 : fs;
     return p;
 }
 
@@ -238,8 +247,8 @@ const int *outer_colour_ranks(psms_ctx *c, int keep) {
 // whole-lattice solve of n systems with the given links; rank_active
 // (optional) restricts it to the inner blocks of one outer colour when the
 // links decouple the colours and b vanishes on the other
-long long solve_all(psms_ctx *c, const double2 *U64, const float2 *U32, long long bs, int n, const double2 *b,
-                    double2 *x, double tol, int inner, const int *rank_active = nullptr,
+long long solve_all(psms_ctx *c, const double2 *U64, const int4 *fx, long long fx_bs, const float2 *U32, long long bs,
+                    int n, const double2 *b, double2 *x, double tol, int inner, const int *rank_active = nullptr,
                     const LinkInterp &li = LinkInterp{}) {
     const long long V = c->g.V, fs = 12 * V;
     FullSolveReq q;
@@ -250,6 +259,8 @@ long long solve_all(psms_ctx *c, const double2 *U64, const float2 *U32, long lon
     q.U32 = U32;
     q.li32 = li;
     q.U64_bs = bs;
+    q.fx = fx;
+    q.fx_bs = fx_bs;
     q.tol = tol;
     q.inner_prec = inner;
     q.rank_active = rank_active;
@@ -269,12 +280,12 @@ SharedEnds outer_ends(psms_ctx *c, const double2 *U, const double2 *Up, int kind
 }
 
 // out = -1/2 H(in) with the given links over the whole lattice
-void hop_all(psms_ctx *c, const double2 *U64, long long bs, int n, const double2 *in, double2 *out) {
+void hop_all(psms_ctx *c, const int4 *fx, long long fx_bs, int n, const double2 *in, double2 *out) {
     const long long V = c->g.V, fs = 12 * V;
     HopCall h;
     h.prec = P64;
-    h.U = U64;
-    h.U_bs = bs;
+    h.fx = fx;
+    h.fx_bs = fx_bs;
     h.n_sys = n;
     h.p = -1;
     h.mode = HOP_ALL;
@@ -314,16 +325,18 @@ long long sub_chunk(psms_ctx *c, const double2 *U, const double2 *Up, int N, int
     int *status = (int *)scratch(c, "sub_status", sizeof(int) * nbh * n);
     long long tot = 0;
     std::vector<int> hit(nbh * n);
-    auto solve_ranks = [&](int lo, const double2 *U64, const float2 *U32, double2 *b, double2 *x) {
+    auto solve_ranks = [&](int lo, double2 *b, double2 *x) {
         BlockSolveReq q;
         q.rank_lo = lo;
         q.n_ranks = nbh;
         q.n_sys = n;
         q.b = View<double2>{b, V, 0, fs};
         q.x = View<double2>{x, V, 0, fs};
-        q.U64 = U64;
-        q.U32 = U32;
+        q.U64 = pr.a64;
+        q.U32 = pr.a32;
         q.U64_bs = pr.bs;
+        q.fx = pr.afx;
+        q.fx_bs = pr.fx_bs;
         q.tol = tol;
         q.inner_prec = inner;
         q.iters = iters;
@@ -341,8 +354,8 @@ long long sub_chunk(psms_ctx *c, const double2 *U, const double2 *Up, int N, int
     // inter-block hops stay inside the outer blocks
     HopCall h;
     h.prec = P64;
-    h.U = pr.a64;
-    h.U_bs = pr.bs;
+    h.fx = pr.afx;
+    h.fx_bs = pr.fx_bs;
     h.n_sys = n;
     h.p = -1;
     h.mode = HOP_INTER;
@@ -352,23 +365,23 @@ long long sub_chunk(psms_ctx *c, const double2 *U, const double2 *Up, int N, int
     h.in = View<void>{xi, V, 0, fs};
     h.out = View<void>{t1, V, 0, fs};
     hop_launch(c, h);
-    solve_ranks(nbh, pr.a64, pr.a32, t1, t2);  // D_ww^-1
+    solve_ranks(nbh, t1, t2);  // D_ww^-1
     h.rank_lo = 0;                              // D_bw on the black inner blocks
     h.in = View<void>{t2, V, 0, fs};
     h.out = View<void>{t1, V, 0, fs};
     hop_launch(c, h);
-    solve_ranks(0, pr.a64, pr.a32, t1, t2);  // D_bb^-1 (t2 keeps stale white values; P_b = 0 there)
+    solve_ranks(0, t1, t2);  // D_bb^-1 (t2 keeps stale white values; P_b = 0 there)
     sub_projected(c, outer::SUB, v, xi, t2, n);
     // w = (1 - P_b Q_b(U_{i+1}))^-1 v = v - P_b [D_O^-1 (0, D_wb v)]_black
     cuda_check(cudaMemsetAsync(t1, 0, sizeof(double2) * fs * n, c->stream), "sub memset");
-    h.U = pr.b64;
+    h.fx = pr.bfx;
     h.rank_lo = nbh;
     h.in = View<void>{v, V, 0, fs};
     h.out = View<void>{t1, V, 0, fs};
     hop_launch(c, h);
     LinkInterp li;
     if (inner != P64 && c->shared_links) li = link_interp(c, outer_ends(c, U, Up, 1, "sub"), N, i0, n, 1, mode, "sub");
-    tot += solve_all(c, pr.b64, pr.b32, pr.bs, n, t1, t2, tol, inner, nullptr, li);
+    tot += solve_all(c, pr.b64, pr.bfx, pr.fx_bs, pr.b32, pr.bs, n, t1, t2, tol, inner, nullptr, li);
     sub_projected(c, outer::SUB, w, v, t2, n);
     // per outer block |w|^2 - |xi|^2, summed over its inner blocks in rank order
     double *nw = (double *)scratch(c, "sub_nw", sizeof(double) * nr * n);
@@ -419,17 +432,17 @@ long long outer_global_chunk(psms_ctx *c, const double2 *U, const double2 *Up, i
     // masked links decouple the outer blocks and the right-hand sides vanish
     // on the other colour, so only that colour's inner blocks are iterated
     const int *white = outer_colour_ranks(c, 1), *black = outer_colour_ranks(c, 0);
-    hop_all(c, pc.a64, pc.bs, n, xi, t1);  // hops between outer blocks
+    hop_all(c, pc.afx, pc.fx_bs, n, xi, t1);  // hops between outer blocks
     keep_colour(c, t1, n, 1);               // D_wb xi
-    tot += solve_all(c, pm.a64, pm.a32, pm.bs, n, t1, t2, tol, inner, white, lim);  // D_ww^-1 (outer Dirichlet)
-    hop_all(c, pc.a64, pc.bs, n, t2, t1);
+    tot += solve_all(c, pm.a64, pm.afx, pm.fx_bs, pm.a32, pm.bs, n, t1, t2, tol, inner, white, lim);  // D_ww^-1 (outer Dirichlet)
+    hop_all(c, pc.afx, pc.fx_bs, n, t2, t1);
     keep_colour(c, t1, n, 0);  // D_bw
-    tot += solve_all(c, pm.a64, pm.a32, pm.bs, n, t1, t2, tol, inner, black, lim);  // D_bb^-1
+    tot += solve_all(c, pm.a64, pm.afx, pm.fx_bs, pm.a32, pm.bs, n, t1, t2, tol, inner, black, lim);  // D_bb^-1
     sub_projected(c, outer::OUTER, v, xi, t2, n);
     // w = (1 - P Q(U_{i+1}))^-1 v = v - P [D^-1 (0, D_wb v)]_black
-    hop_all(c, pc.b64, pc.bs, n, v, t1);
+    hop_all(c, pc.bfx, pc.fx_bs, n, v, t1);
     keep_colour(c, t1, n, 1);
-    tot += solve_all(c, pf.b64, pf.b32, pf.bs, n, t1, t2, tol, inner, nullptr, lif);
+    tot += solve_all(c, pf.b64, pf.bfx, pf.fx_bs, pf.b32, pf.bs, n, t1, t2, tol, inner, nullptr, lif);
     sub_projected(c, outer::OUTER, w, v, t2, n);
     double *nw = (double *)scratch(c, "og_nw", sizeof(double) * n);
     double *nx = (double *)scratch(c, "og_nx", sizeof(double) * n);

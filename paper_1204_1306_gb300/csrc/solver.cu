@@ -88,6 +88,8 @@ void block_solve(psms_ctx *c, const BlockSolveReq &q) {
     a.r64 = View<double2>{(double2 *)scratch(c, "bs_r64", full64 * q.n_sys), V, 0, 12 * V};
     a.U64 = q.U64;
     a.U64_bs = q.U64_bs;
+    a.fx = q.fx;
+    a.fx_bs = q.fx_bs;
     const bool in64 = (q.inner_prec == P64);
     const size_t esz = in64 ? sizeof(double2) : sizeof(float2);
     const long long per_sys = 24 * V + 7 * 12 * (long long)g.Vh;  // elements
@@ -392,7 +394,7 @@ __global__ void iters_bcg_kernel(const BCS *st, int *out, int n);
 template <class SV>
 static void inner_cg_full(psms_ctx *c, int n_sys, const void *Uin, long long U_bs, int prec, View<void> rhs,
                           View<void> e, const int *act_in, double delta, int maxit, int *iters_acc,
-                          const LinkInterp &li) {
+                          const LinkInterp &li, const int4 *fx, long long fx_bs) {
     using E = typename SV::elem;
     const Geom &g = c->g;
     const long long V = g.V, Vh = g.Vh;
@@ -420,6 +422,8 @@ static void inner_cg_full(psms_ctx *c, int n_sys, const void *Uin, long long U_b
     h.prec = prec;
     h.U = Uin;
     h.U_bs = U_bs;
+    h.fx = fx;
+    h.fx_bs = fx_bs;
     h.li = li;
     h.n_sys = n_sys;
     h.active = act_in;
@@ -709,7 +713,7 @@ __global__ void iters_bcg_kernel(const BCS *st, int *out, int n) {
 template <class SV>
 static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long long U_bs, int prec, View<void> rhs,
                                 View<void> e, const int *act_in, double delta, int maxit, int *iters_acc,
-                                const int *rank_active, const LinkInterp &li) {
+                                const int *rank_active, const LinkInterp &li, const int4 *fx, long long fx_bs) {
     using E = typename SV::elem;
     const Geom &g = c->g;
     const long long V = g.V, Vh = g.Vh;
@@ -739,6 +743,8 @@ static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long lo
     h.prec = prec;
     h.U = Uin;
     h.U_bs = U_bs;
+    h.fx = fx;
+    h.fx_bs = fx_bs;
     h.li = li;
     h.n_sys = n_sys;
     h.active = act_in;
@@ -941,6 +947,8 @@ void solve_full_batch(psms_ctx *c, const FullSolveReq &q, psms_solve_info *info)
         h.prec = P64;
         h.U = q.U64;
         h.U_bs = q.U64_bs;
+        h.fx = q.fx;
+        h.fx_bs = q.fx_bs;
         h.n_sys = n;
         if (outer > 0) {
             omap.clear();
@@ -989,10 +997,10 @@ void solve_full_batch(psms_ctx *c, const FullSolveReq &q, psms_solve_info *info)
             PSMS_LAUNCH_CHECK("scale_convert_kernel");
             if (bicg)
                 inner_bicgstab_full<Store<double>>(c, n, q.U64, q.U64_bs, P64, rin, ein, act, delta, q.maxit, iters,
-                                                   q.rank_active, LinkInterp{});
+                                                   q.rank_active, LinkInterp{}, q.fx, q.fx_bs);
             else
                 inner_cg_full<Store<double>>(c, n, q.U64, q.U64_bs, P64, rin, ein, act, delta, q.maxit, iters,
-                                             LinkInterp{});
+                                             LinkInterp{}, q.fx, q.fx_bs);
             accumulate_kernel<Store<double>, NT><<<grid, NT, 0, c->stream>>>(
                 View<double2>{(double2 *)q.x.p, q.x.cs, q.x.off, q.x.bs}, View<double2>{(double2 *)ein_p, V, 0, 12 * V},
                 rn, act, 0, V);
@@ -1003,9 +1011,10 @@ void solve_full_batch(psms_ctx *c, const FullSolveReq &q, psms_solve_info *info)
             PSMS_LAUNCH_CHECK("scale_convert_kernel");
             if (bicg)
                 inner_bicgstab_full<Store<float>>(c, n, q.U32, q.U64_bs, P32, rin, ein, act, delta, q.maxit, iters,
-                                                  q.rank_active, q.li32);
+                                                  q.rank_active, q.li32, nullptr, 0);
             else
-                inner_cg_full<Store<float>>(c, n, q.U32, q.U64_bs, P32, rin, ein, act, delta, q.maxit, iters, q.li32);
+                inner_cg_full<Store<float>>(c, n, q.U32, q.U64_bs, P32, rin, ein, act, delta, q.maxit, iters, q.li32,
+                                            nullptr, 0);
             accumulate_kernel<Store<float>, NT><<<grid, NT, 0, c->stream>>>(
                 View<double2>{(double2 *)q.x.p, q.x.cs, q.x.off, q.x.bs}, View<float2>{(float2 *)ein_p, V, 0, 12 * V},
                 rn, act, 0, V);
@@ -1016,10 +1025,10 @@ void solve_full_batch(psms_ctx *c, const FullSolveReq &q, psms_solve_info *info)
             PSMS_LAUNCH_CHECK("scale_convert_kernel");
             if (bicg)
                 inner_bicgstab_full<Store<__nv_bfloat16>>(c, n, q.U32, q.U64_bs, PB16, rin, ein, act, delta, q.maxit,
-                                                          iters, q.rank_active, q.li32);
+                                                          iters, q.rank_active, q.li32, nullptr, 0);
             else
                 inner_cg_full<Store<__nv_bfloat16>>(c, n, q.U32, q.U64_bs, PB16, rin, ein, act, delta, q.maxit,
-                                                    iters, q.li32);
+                                                    iters, q.li32, nullptr, 0);
             accumulate_kernel<Store<__nv_bfloat16>, NT><<<grid, NT, 0, c->stream>>>(
                 View<double2>{(double2 *)q.x.p, q.x.cs, q.x.off, q.x.bs},
                 View<__nv_bfloat162>{(__nv_bfloat162 *)ein_p, V, 0, 12 * V}, rn, act, 0, V);
@@ -1163,6 +1172,8 @@ extern "C" psms_status psms_block_solve_noalloc(psms_ctx *ctx, int field, int op
         a.r64 = View<double2>{r64, V, 0, 12 * V};
         a.U64 = ctx->U64[field];
         a.U64_bs = 0;
+        a.fx = nullptr;  // no room for a copy of the links
+        a.fx_bs = 0;
         a.Uin = ctx->U64[field];
         a.Uin_bs = 0;
         a.vin = vin;
@@ -1356,6 +1367,8 @@ psms_status psms_block_plan_create(const psms_block_problem *probs, int n_probs,
             a.r64 = View<double2>{(double2 *)r64, V, 0, 12 * V};
             a.U64 = c->U64[q.field];
             a.U64_bs = 0;
+            a.fx = links_fx(c, q.field);
+            a.fx_bs = 0;
             const bool in64 = inner_prec == P64;
             a.Uin = in64 ? (const void *)c->U64[q.field] : (const void *)links32(c, q.field);
             cuda_check(cudaStreamSynchronize(c->stream), "plan sync");
@@ -1446,13 +1459,14 @@ psms_status psms_block_plan_run(psms_block_plan *pl, void *stream, psms_solve_in
     if (!pl) return PSMS_EINVAL;
     try {
         cudaStream_t s = (cudaStream_t)stream;
-        // FP32 link copies must follow changes of the gauge fields
+        // link copies must follow changes of the gauge fields
         for (size_t p = 0; p < pl->probs.size(); ++p) {
             psms_ctx *c = pl->probs[p].ctx;
-            if (pl->inner == P32 && !c->u32_ok[pl->probs[p].field]) {
-                links32(c, pl->probs[p].field);
-                cuda_check(cudaStreamSynchronize(c->stream), "links sync");
-            }
+            const int f = pl->probs[p].field;
+            const bool need32 = pl->inner == P32 && !c->u32_ok[f], needfx = pl->h_args[p].fx && !c->ufx_ok[f];
+            if (need32) links32(c, f);
+            if (needfx) links_fx(c, f);
+            if (need32 || needfx) cuda_check(cudaStreamSynchronize(c->stream), "links sync");
         }
         cuda_check(cudaGraphLaunch(pl->exec, s), "graph launch");
         double h[3];

@@ -15,6 +15,10 @@ struct BlockSolveReq {
     const double2 *U64 = nullptr;
     const float2 *U32 = nullptr;
     long long U64_bs = 0;  // elements (complex) between the systems' link fields
+    // the FP64 links in fixed point (nullable; 16-byte elements between the
+    // systems): with them the FP64 links are read by FP64 inner iterations only
+    const int4 *fx = nullptr;
+    long long fx_bs = 0;
     double tol = 1e-13;
     int maxit = 100000;
     int inner_prec = P64;
@@ -34,6 +38,8 @@ struct FullSolveReq {
     const double2 *U64 = nullptr;
     const float2 *U32 = nullptr;
     long long U64_bs = 0;
+    const int4 *fx = nullptr;  // the FP64 links in fixed point (nullable)
+    long long fx_bs = 0;
     double tol = 1e-13;
     int maxit = 100000;
     int inner_prec = P64;
