@@ -1,0 +1,455 @@
+// Dirichlet block solver for blocks of 256 sites (4^4 and the other shapes of
+// that volume) with FP32 inner iterations: even-odd CGNR on Dhat^dag Dhat
+// inside the FP64 defect correction of block_solve.cuh, the whole solve of a
+// (block, system) by one CTA of 128 threads.
+//
+// What bounds it: the FP32 pipe.  A hop direction is 108 FP32 instructions on
+// 11 shared-memory loads; an iteration has four half hops.  So what the hops
+// touch lives on the SM: thread j owns odd site j and keeps its parts of res,
+// p and q in registers, the links inside the block (59 KB at 4^4) and the
+// vector that neighbours read (p, q or t; 12 KB) are in shared memory, and
+// three CTAs share an SM.  e and rho, used once an iteration, and the FP64
+// right-hand side, solution and residual of the defect correction are in
+// global memory (L2).
+//
+// FP64 has two lanes per SM here, a warp's FP64 instruction costs 16 clocks
+// of them, so the iterations have none: the norms are summed exactly in
+// integers (redux on two 25-bit limbs), the scalars are pairs of FP32 numbers,
+// and the true residual is taken in fixed point (fixed_hop.cuh), its spinors
+// converted once into the links' shared memory.
+#pragma once
+
+#include "fixed_hop.cuh"
+#include "kernels.hpp"
+#include "solver.hpp"
+
+namespace psms {
+
+constexpr int CG_NT = 128;
+constexpr int CG_XF = 12 * 128 + 16;  // 16-byte elements of a parity's fixed-point spinors (fixed.cuh)
+constexpr int CG_XS = 132;  // sites of an exchange row: 128, one zero site for hops that leave the block, padding
+
+// sum of a CTA's FP32 numbers as hi + lo
+struct ff {
+    float hi, lo;
+};
+
+__device__ __forceinline__ float pow2f(int k) {  // 2^k, 0 below the normal range, k <= 127
+    return k < -126 ? 0.0f : __int_as_float((k + 127) << 23);
+}
+
+// a / b to FP32 precision of the pairs
+__device__ __forceinline__ float ff_div(ff a, ff b) {
+    const float q = a.hi / b.hi;
+    const float r = fmaf(-q, b.hi, a.hi) + (a.lo - q * b.lo);
+    return q + r / b.hi;
+}
+
+// Sum over the CTA of t >= 0, exact for numbers down to 2^-26 of a warp's
+// largest (50 bits below it): mantissas on the warp's largest exponent, two
+// 25-bit limbs summed by redux, the four warps' sums as 64-bit integers.
+// slot: one of two, alternating (one barrier per sum).
+struct CgSums {
+    int v[2][CG_NT / 32][4];  // exponent, high, low limb sums
+};
+
+__device__ __forceinline__ ff cg_sum(float t, CgSums &sm, int &slot) {
+    const unsigned b = __float_as_uint(t) & 0x7FFFFFFFu;
+    const int e = (int)(b >> 23);
+    const int em = __reduce_max_sync(0xffffffffu, e);
+    const uint64_t m = e == 0 ? 0 : fx_shr((uint64_t)((b & 0x7FFFFFu) | 0x800000u) << 26, (uint32_t)(em - e));
+    const int hi = __reduce_add_sync(0xffffffffu, (int)(m >> 25)), lo = __reduce_add_sync(0xffffffffu, (int)(m & 0x1FFFFFFu));
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) *reinterpret_cast<int4 *>(sm.v[slot][w]) = make_int4(em, hi, lo, 0);
+    __syncthreads();
+    int E = 0;
+    int4 q[CG_NT / 32];
+#pragma unroll
+    for (int i = 0; i < CG_NT / 32; ++i) {
+        q[i] = *reinterpret_cast<const int4 *>(sm.v[slot][i]);
+        E = max(E, q[i].x);
+    }
+    slot ^= 1;
+    uint64_t s = 0;
+#pragma unroll
+    for (int i = 0; i < CG_NT / 32; ++i)
+        s += fx_shr(((uint64_t)(unsigned)q[i].y << 25) + (uint64_t)(unsigned)q[i].z, (uint32_t)(E - q[i].x));
+    // value = s 2^(E - 176), s < 2^57, as the exact sum of three floats
+    const float p2 = (float)(int)(s >> 48) * pow2f(E - 128), p1 = (float)(int)((s >> 24) & 0xFFFFFF) * pow2f(E - 152),
+                p0 = (float)(int)(s & 0xFFFFFF) * pow2f(E - 176);
+    const float a = p2 + p1, c = (p1 - (a - p2)) + p0;
+    ff r;
+    r.hi = a + c;
+    r.lo = c - (r.hi - a);
+    if (E == 255) r.hi = r.lo = __int_as_float(0x7FC00000);  // infinity or NaN among them
+    return r;
+}
+
+// FP64 sum over the CTA in a fixed order
+__device__ __forceinline__ double cg_sum64(double v, double *sh) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = sh[0];
+#pragma unroll
+    for (int i = 1; i < CG_NT / 32; ++i) t += sh[i];
+    return t;
+}
+
+// Links in shared memory: direction mu holds, per parity, the sites whose link
+// stays in the block (mu = 3: all), row by row of the FP32 field layout; at
+// most 864 links for the shapes of 256 sites.
+constexpr int CG_LINKS = 864;
+
+struct CgLinks {
+    int off[4];  // first link of direction mu
+    int n[4];    // links per parity
+    int sh[4];   // half index j -> j - (j >> sh) hs (sh = 31: j)
+    int hs[4];
+};
+
+__device__ __forceinline__ CgLinks cg_links(const Geom &g) {
+    CgLinks c;
+    int o = 0;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        const int h = g.lstride[mu] >> 1;  // 0 for mu = 3
+        c.hs[mu] = h;
+        c.sh[mu] = h ? 31 - __clz(h) + g.lsh[mu] : 31;
+        c.n[mu] = 128 - (h ? h << (7 - c.sh[mu]) : 0);
+        c.off[mu] = o;
+        o += 2 * c.n[mu];
+    }
+    return c;
+}
+
+// Neighbours of a thread's site of one parity inside the block: the eight
+// half indices (bytes of nb; 128, the zero site, for a hop that leaves) and
+// the positions of their links (16 bits each of lk[0], lk[1])
+struct CgSite {
+    uint64_t nb, lk[2];
+};
+
+__device__ __forceinline__ CgSite cg_site(const Geom &g, int p, int j) {
+    CgSite c;
+    c.nb = c.lk[0] = c.lk[1] = 0;
+    const CgLinks L = cg_links(g);
+    int y[4];
+    const int ll = local_lex(g, p, j, y);
+#pragma unroll
+    for (int d = 0; d < 8; ++d) {
+        const int mu = d >> 1, sg = (d & 1) ? -1 : 1;
+        const bool in = (unsigned)(y[mu] + sg) < (unsigned)g.l[mu];
+        const int n = in ? (ll + sg * g.lstride[mu]) >> 1 : 128;
+        c.nb |= (uint64_t)n << (8 * d);
+        // the link's site: this one forward, the neighbour backward (any
+        // valid link for a hop that leaves: its spinor is zero)
+        const int q = (d & 1) ? 1 - p : p, i = (d & 1) ? n : j;
+        const int l = in ? L.off[mu] + q * L.n[mu] + i - (i >> L.sh[mu]) * L.hs[mu] : L.off[mu];
+        c.lk[d >> 2] |= (uint64_t)l << (16 * (d & 3));
+    }
+    return c;
+}
+
+struct CgShared {
+    float4 links[4 * CG_LINKS];  // units of element pairs, [unit][link]; then the ninth elements
+    float2 links9[CG_LINKS];
+    float4 x[6 * CG_XS];         // the vector that neighbours read
+    CgSums sums;
+    double sh[CG_NT / 32];
+};
+
+__device__ __forceinline__ void cg_put(float4 *x, int j, const Spinor<float> &v) {
+#pragma unroll
+    for (int u = 0; u < 6; ++u) {
+        const cpx<float> a = v.c[(2 * u) / 3][(2 * u) % 3], b = v.c[(2 * u + 1) / 3][(2 * u + 1) % 3];
+        x[u * CG_XS + j] = make_float4(a.re, a.im, b.re, b.im);
+    }
+}
+
+// sum of the hops (s = sg: +1 D, -1 D^dagger) onto the thread's site
+__device__ __forceinline__ Spinor<float> cg_hop(const CgShared &sm, uint64_t nb, uint64_t lk0, uint64_t lk1, float sg) {
+    Spinor<float> acc;
+    zero(acc);
+#pragma unroll
+    for (int d = 0; d < 8; ++d) {
+        const int mu = d >> 1;
+        const bool fwd = (d & 1) == 0;
+        const int n = (int)(nb >> (8 * d)) & 255;
+        const int l = (int)((d < 4 ? lk0 : lk1) >> (16 * (d & 3))) & 0xFFFF;
+        Spinor<float> v;
+#pragma unroll
+        for (int u = 0; u < 6; ++u) {
+            const float4 w = sm.x[u * CG_XS + n];
+            v.c[(2 * u) / 3][(2 * u) % 3] = {w.x, w.y};
+            v.c[(2 * u + 1) / 3][(2 * u + 1) % 3] = {w.z, w.w};
+        }
+        const float t = fwd ? -sg : sg;
+        const Half<float> h = project(mu, t, v);
+        SU3<float> u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float4 w = sm.links[k * CG_LINKS + l];
+            u.e[(2 * k) / 3][(2 * k) % 3] = {w.x, w.y};
+            u.e[(2 * k + 1) / 3][(2 * k + 1) % 3] = {w.z, w.w};
+        }
+        const float2 w = sm.links9[l];
+        u.e[2][2] = {w.x, w.y};
+        reconstruct_add(mu, t, fwd ? su3_mul(u, h) : su3_dag_mul(u, h), acc);
+    }
+    return acc;
+}
+
+// a x + b y
+__device__ __forceinline__ Spinor<float> cg_axpby(float a, const Spinor<float> &x, float b, const Spinor<float> &y) {
+    Spinor<float> r;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            r.c[q][c] = {fmaf(a, x.c[q][c].re, b * y.c[q][c].re), fmaf(a, x.c[q][c].im, b * y.c[q][c].im)};
+    return r;
+}
+
+// x += a y
+__device__ __forceinline__ void cg_add(float a, const Spinor<float> &y, Spinor<float> &x) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            x.c[q][c].re = fmaf(a, y.c[q][c].re, x.c[q][c].re);
+            x.c[q][c].im = fmaf(a, y.c[q][c].im, x.c[q][c].im);
+        }
+}
+
+__device__ __forceinline__ float cg_norm(const Spinor<float> &x) {
+    float t = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) t = fmaf(x.c[q][c].re, x.c[q][c].re, fmaf(x.c[q][c].im, x.c[q][c].im, t));
+    return t;
+}
+
+// The whole solve of item (block rl of the launch, system k).  The hop is one
+// copy of code, used by every step of a small state machine (several inlined
+// copies overflow the instruction cache).
+template <class Args>
+__device__ void block_cg_item(const Args &a, int rl, int k, CgShared &sm) {
+    const Geom &g = a.g;
+    const int j = threadIdx.x, r = a.rank_lo + rl;
+    const long long out_i = (long long)k * a.n_ranks + rl;
+    const BlockInfo &bi = a.binfo[r];
+    const long long V = g.V, Vh = g.Vh;
+    const long long site[2] = {(long long)r * g.Vbh + j, Vh + (long long)r * g.Vbh + j};
+    const double2 *b = a.b.p + k * a.b.bs - a.b.off;
+    double2 *x = a.x.p + k * a.x.bs - a.x.off;
+    double2 *r64 = a.r64.p + k * a.r64.bs - a.r64.off;
+    // FP32 vectors of the system in global memory: the even half of the inner
+    // right-hand side (full layout), then e (full layout) and rho (odd half)
+    float2 *rhs_e = (float2 *)a.vin + k * a.vin_bs;
+    float2 *ev = rhs_e + 12 * V, *rhov = rhs_e + 24 * V - 2 * Vh;  // (rho: odd site s at unit u Vh + s - Vh)
+    bool skip = (a.sys_active && !a.sys_active[k]) || (a.block_active && !a.block_active[bi.lex]);
+    double bn = 0;
+    if (!skip) {
+        for (int p = 0; p < 2; ++p)
+            for (int q = 0; q < 12; ++q) {
+                const double2 v = b[q * a.b.cs + site[p]];
+                x[q * a.x.cs + site[p]] = make_double2(0, 0);
+                bn = fma(v.x, v.x, fma(v.y, v.y, bn));
+            }
+        bn = cg_sum64(bn, sm.sh);
+        skip = bn == 0.0;
+    }
+    if (skip) {
+        if (j == 0) {
+            a.iters[out_i] = 0;
+            a.resid[out_i] = 0;
+            a.status[out_i] = 0;
+            if (a.xnorm2) a.xnorm2[out_i] = 0;
+        }
+        return;
+    }
+    if (j < 6) sm.x[j * CG_XS + 128] = make_float4(0, 0, 0, 0);
+    const CgSite st_e = cg_site(g, 0, j), st_o = cg_site(g, 1, j);
+    const float A = (float)a.A, c4 = (float)(-1.0 / (4.0 * a.A)), h2A = (float)(0.5 / a.A), iA = (float)(1.0 / a.A);
+    const float delta2 = (float)(a.delta * a.delta);
+    int total_it = 0, status = 0, slot = 0;
+    double rel = 0, rn = bn;
+    for (int outer = 0;; ++outer) {
+        // FP64 true residual r64 = b - D_b x (r64 = b on the first step)
+        if (outer > 0) {
+            // x in fixed point takes the place of the links in shared memory
+            longlong2 *xs = reinterpret_cast<longlong2 *>(sm.links);
+            rn = 0;
+            __syncthreads();
+#pragma unroll 1
+            for (int p = 0; p < 2; ++p) {
+                int64_t v[12][2];
+                const int e = fx_load_spinor(x + site[p], a.x.cs, v);
+                longlong2 *o = xs + p * CG_XF;
+#pragma unroll
+                for (int c = 0; c < 12; ++c) o[c * 128 + j] = make_longlong2(v[c][0], v[c][1]);
+                reinterpret_cast<uint16_t *>(o + 12 * 128)[j] = (uint16_t)e;
+            }
+            __syncthreads();
+#pragma unroll 1
+            for (int p = 0; p < 2; ++p) {
+                const FxHop h{x, a.x.cs, 0, a.fx + k * a.fx_bs, HOP_INTRA, 0, xs + (1 - p) * CG_XF, 128,
+                              site[1 - p] - j};
+                double2 hx[12];
+                fx_site<false>(h, g, bi, r, p, j, 0.5, hx);
+                for (int q = 0; q < 12; ++q) {
+                    const double2 bv = b[q * a.b.cs + site[p]], xv = x[q * a.x.cs + site[p]];
+                    const double2 v = make_double2(fma(-a.A, xv.x, bv.x + hx[q].x), fma(-a.A, xv.y, bv.y + hx[q].y));
+                    r64[q * a.r64.cs + site[p]] = v;
+                    rn = fma(v.x, v.x, fma(v.y, v.y, rn));
+                }
+            }
+            rn = cg_sum64(rn, sm.sh);
+        }
+        rel = sqrt(rn / bn);
+        if (rel <= a.tol) break;
+        if (outer >= a.max_outer || total_it >= a.maxit) {
+            status = 1;
+            break;
+        }
+        const double2 *src = outer ? r64 : b;
+        const long long scs = outer ? a.r64.cs : a.b.cs;
+        const double scale = 1.0 / sqrt(rn);
+        __syncthreads();
+        // links of the block
+        {
+            const float2 *U = (const float2 *)a.Uin + k * a.Uin_bs;
+            const CgLinks L = cg_links(g);
+#pragma unroll 1
+            for (int t = 0; t < 8; ++t) {
+                const int mu = t >> 1, q = t & 1;
+                int y[4];
+                local_lex(g, q, j, y);
+                if (mu < 3 && y[mu] == g.l[mu] - 1) continue;
+                const int l = L.off[mu] + q * L.n[mu] + j - (j >> L.sh[mu]) * L.hs[mu];
+                const float2 *gb = U + (long long)mu * 9 * V;
+                const float4 *g4 = reinterpret_cast<const float4 *>(gb);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) sm.links[u * CG_LINKS + l] = __ldg(g4 + u * V + site[q]);
+                sm.links9[l] = __ldg(gb + 8 * V + site[q]);
+            }
+        }
+        // inner rhs = r64 / |r64| in FP32: even half to the exchange buffer
+        // (and kept in global memory for the end), odd half in q
+        Spinor<float> res, pp, q;
+        for (int c = 0; c < 12; ++c) {
+            const double2 v = src[c * scs + site[0]];
+            q.c[c / 3][c % 3] = {(float)(v.x * scale), (float)(v.y * scale)};
+        }
+        store_spinor<Store<float>>(rhs_e, V, site[0], q);
+        cg_put(sm.x, j, q);
+        for (int c = 0; c < 12; ++c) {
+            const double2 w = src[c * scs + site[1]];
+            q.c[c / 3][c % 3] = {(float)(w.x * scale), (float)(w.y * scale)};
+        }
+        zero(res);
+        zero(pp);
+        store_spinor<Store<float>>(ev, V, site[1], res);  // e = 0
+        __syncthreads();
+        ff rr = {0, 0};
+        float target = 0, alpha = 0;
+        int it = 0;
+        // steps: 0 bhat = rhs_o + H_o(rhs_e)/(2A) (= rho, kept in q); 1, 2 res =
+        // Dhat^dag rho; 3, 4 q = Dhat p and the updates of e, rho; 5, 6
+        // Dhat^dag q and the updates of res, p; 7 e_e = (rhs_e + H_e(e)/2)/A
+#pragma unroll 1
+        for (int step = 0;;) {
+            const bool odd = (step & 1) == 0;  // output parity (steps 0, 2, 4, 6)
+            const Spinor<float> acc = cg_hop(sm, odd ? st_o.nb : st_e.nb, odd ? st_o.lk[0] : st_e.lk[0],
+                                             odd ? st_o.lk[1] : st_e.lk[1],
+                                             step == 1 || step == 2 || step == 5 || step == 6 ? -1.0f : 1.0f);
+            if (step == 0) {
+                cg_add(h2A, acc, q);
+                store_spinor<Store<float>>(rhov, Vh, site[1], q);
+                const ff bb = cg_sum(cg_norm(q), sm.sums, slot);
+                target = bb.hi * delta2;
+                step = bb.hi > 0 ? 1 : 7;  // (a zero right-hand side: e = 0)
+                if (step == 7) q = res;
+                cg_put(sm.x, j, q);
+            } else if (odd == false && step != 7) {  // 1, 3, 5: the vector on even sites
+                __syncthreads();
+                cg_put(sm.x, j, acc);
+                ++step;
+            } else if (step == 2) {
+                res = cg_axpby(A, q, c4, acc);
+                pp = res;
+                rr = cg_sum(cg_norm(res), sm.sums, slot);
+                const bool stop = total_it >= a.maxit;
+                if (stop) zero(q);
+                cg_put(sm.x, j, stop ? q : pp);
+                step = stop ? 7 : 3;
+            } else if (step == 4) {
+                q = cg_axpby(A, pp, c4, acc);
+                Spinor<float> rho = load_spinor<Store<float>>(rhov, Vh, site[1]);
+                Spinor<float> e = load_spinor<Store<float>>(ev, V, site[1]);
+                const ff qq = cg_sum(cg_norm(q), sm.sums, slot);
+                alpha = ff_div(rr, qq);
+                cg_add(alpha, pp, e);
+                cg_add(-alpha, q, rho);
+                store_spinor<Store<float>>(ev, V, site[1], e);
+                store_spinor<Store<float>>(rhov, Vh, site[1], rho);
+                const ff rhorho = cg_sum(cg_norm(rho), sm.sums, slot);
+                ++it;
+                // converged, broken down (NaN included)
+                const bool stop = !(rhorho.hi > target) || !(qq.hi > 0);
+                cg_put(sm.x, j, stop ? e : q);
+                step = stop ? 7 : 5;
+            } else if (step == 6) {
+                cg_add(-alpha, cg_axpby(A, q, c4, acc), res);
+                const ff rn2 = cg_sum(cg_norm(res), sm.sums, slot);
+                const float beta = ff_div(rn2, rr);
+                rr = rn2;
+                pp = cg_axpby(beta, pp, 1.0f, res);
+                const bool stop = total_it + it >= a.maxit;
+                if (stop) q = load_spinor<Store<float>>(ev, V, site[1]);
+                cg_put(sm.x, j, stop ? q : pp);
+                step = stop ? 7 : 3;
+            } else {
+                // the solution of the inner system, added to x in FP64
+                const Spinor<float> e = load_spinor<Store<float>>(ev, V, site[1]);
+                Spinor<float> ee = load_spinor<Store<float>>(rhs_e, V, site[0]);
+                ee = cg_axpby(iA, ee, h2A, acc);
+                const double unscale = sqrt(rn);
+                for (int c = 0; c < 12; ++c) {
+                    double2 v = x[c * a.x.cs + site[0]];
+                    v.x = fma(unscale, (double)ee.c[c / 3][c % 3].re, v.x);
+                    v.y = fma(unscale, (double)ee.c[c / 3][c % 3].im, v.y);
+                    x[c * a.x.cs + site[0]] = v;
+                    double2 w = x[c * a.x.cs + site[1]];
+                    w.x = fma(unscale, (double)e.c[c / 3][c % 3].re, w.x);
+                    w.y = fma(unscale, (double)e.c[c / 3][c % 3].im, w.y);
+                    x[c * a.x.cs + site[1]] = w;
+                }
+                break;
+            }
+            __syncthreads();
+        }
+        total_it += it;
+    }
+    double xn = 0;
+    if (a.xnorm2) {
+        for (int p = 0; p < 2; ++p)
+            for (int q = 0; q < 12; ++q) {
+                const double2 v = x[q * a.x.cs + site[p]];
+                xn = fma(v.x, v.x, fma(v.y, v.y, xn));
+            }
+        xn = cg_sum64(xn, sm.sh);
+    }
+    if (j == 0) {
+        a.iters[out_i] = total_it;
+        a.resid[out_i] = rel;
+        a.status[out_i] = status;
+        if (a.xnorm2) a.xnorm2[out_i] = xn;
+    }
+}
+
+}  // namespace psms

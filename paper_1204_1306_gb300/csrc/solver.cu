@@ -16,6 +16,7 @@
 //    inner iterations; per-system scalars live on the device; the host only
 //    polls convergence flags every few iterations.
 #include "bicgstab.cuh"
+#include "block_cg.cuh"
 #include "block_solve.cuh"
 #include "kernels.hpp"
 #include "solver.hpp"
@@ -73,6 +74,22 @@ static void launch_block_variant(psms_ctx *c, const BlockSolveArgs &a, int n_ran
     }
 }
 
+// one CTA per (block, system): blocks of 256 sites, FP32 inner CGNR
+__global__ void __launch_bounds__(CG_NT, 3) block_cg_kernel(const BlockSolveArgs a) {
+    extern __shared__ __align__(16) unsigned char cg_smem[];
+    block_cg_item(a, blockIdx.x, blockIdx.y, *reinterpret_cast<CgShared *>(cg_smem));
+}
+
+// the solver of block_cg.cuh runs these solves
+static bool block_cg_fits(const Geom &g, int inner_prec, const int4 *fx) {
+    return inner_prec == P32 && g.Vbh == CG_NT && fx;
+}
+
+static void block_cg_prepare() {
+    cuda_check(cudaFuncSetAttribute(block_cg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CgShared)),
+               "block solver shared memory");
+}
+
 void block_solve(psms_ctx *c, const BlockSolveReq &q) {
     const Geom &g = c->g;
     BlockSolveArgs a;
@@ -107,6 +124,14 @@ void block_solve(psms_ctx *c, const BlockSolveReq &q) {
     a.resid = q.resid;
     a.xnorm2 = q.xnorm2;
     a.status = q.status;
+    if (c->forced_block_variant < 0 && c->block_krylov == 0 && block_cg_fits(g, q.inner_prec, q.fx)) {
+        block_cg_prepare();
+        const int slot = c->prof ? prof_block_begin(c) : -1;
+        block_cg_kernel<<<dim3(q.n_ranks, q.n_sys), CG_NT, sizeof(CgShared), c->stream>>>(a);
+        PSMS_LAUNCH_CHECK("block_cg_kernel");
+        if (slot >= 0) prof_block_end(c, slot);
+        return;
+    }
     // Variants (cluster size CL, min CTAs per SM, hop form): one block solved
     // by CL CTAs of a thread-block cluster; hop form 1 calls one out-of-line
     // copy of the hop instead of inlining it at every call site, form 2 is
