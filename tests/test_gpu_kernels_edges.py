@@ -1,0 +1,168 @@
+"""Sizes and inputs at which the fixed-point hops, the 256-site block solver
+and the blocked LU can go wrong, against the oracle, the FP64 form of the same
+operator or torch's dense LU."""
+import numpy as np
+import pytest
+import torch
+
+import paper_1204_1306_gb300 as ps
+from oracle import dirac, estimator, gauge, lattice
+from oracle.gamma import GAMMA
+from tests import seeded
+from tests.gpu_util import canonical, native, rel_err
+
+pytestmark = pytest.mark.gpu
+
+
+def _ctx(dims, block, seed=11, kappa=0.15, eps=0.4):
+    ctx = ps.psms_create(dims, block, kappa, 1)
+    ps.psms_gauge_init(ctx, 0, eps, seed)
+    return ctx, gauge.generate_links(dims, eps, seed)
+
+
+def _apply(ctx, nat, op, graph=False):
+    """D psi; graph: under stream capture, where the FP64 form of the hops runs."""
+    out = torch.zeros_like(nat)
+    if not graph:
+        ps.psms_dw_apply(ctx, 0, op, nat, out, ps.PREC_F64)
+        torch.cuda.synchronize()
+        return out.view(torch.float64)
+    ps.psms_autotune(ctx, False)  # no timing runs inside the capture
+    s = torch.cuda.Stream()
+    ps.psms_set_stream(ctx, s)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        ps.psms_dw_apply(ctx, 0, op, nat, out, ps.PREC_F64)
+    ps.psms_set_stream(ctx, None)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    return out.view(torch.float64)
+
+
+# (below and above the split into directions; V/2 not a multiple of a CTA; odd block counts)
+@pytest.mark.parametrize("dims,block", [((4, 4, 4, 4), (2, 2, 2, 2)), ((6, 4, 4, 2), (2, 2, 2, 2)),
+                                        ((12, 12, 12, 12), (4, 4, 4, 4)), ((16, 8, 16, 12), (8, 2, 4, 4))])
+@pytest.mark.parametrize("op", [ps.OP_FULL, ps.OP_BLOCKS, 1])
+def test_fixed_point_hops_against_the_fp64_form(dims, block, op):
+    ctx, _ = _ctx(dims, block)
+    nat = native(ctx, seeded.spinor(dims, 3))
+    a, b = _apply(ctx, nat, op), _apply(ctx, nat, op, graph=True)
+    # each site is a sum of 192 products; both forms round to a few 2^-53 of its largest terms
+    assert float((a - b).abs().max() / b.abs().max()) < 64 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("dims,block", [((4, 4, 4, 4), (2, 2, 2, 2)), ((16, 16, 16, 8), (4, 4, 4, 4))])
+@pytest.mark.parametrize("scale", [2.0 ** -1000, 2.0 ** -850, 2.0 ** 850, 2.0 ** 1000])
+def test_hops_at_the_ends_of_the_fp64_range(dims, block, scale):
+    ctx, _ = _ctx(dims, block)
+    nat = native(ctx, seeded.spinor(dims, 4))
+    ref = _apply(ctx, nat, ps.OP_FULL)
+    big = nat.clone()
+    big.view(torch.float64).mul_(scale)  # a power of two: exact
+    got = _apply(ctx, big, ps.OP_FULL)
+    assert float((got / scale - ref).abs().max() / ref.abs().max()) < 64 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("dims,block", [((4, 4, 4, 4), (2, 2, 2, 2)), ((16, 16, 16, 8), (4, 4, 4, 4))])
+def test_non_finite_spinors_spread_as_in_fp64(dims, block, bad):
+    ctx, _ = _ctx(dims, block)
+    nat = native(ctx, seeded.spinor(dims, 5))
+    nat.view(torch.float64)[2 * 77 + 1] = bad
+    a, b = _apply(ctx, nat, ps.OP_FULL), _apply(ctx, nat, ps.OP_FULL, graph=True)
+    fin = torch.isfinite(b)
+    assert 24 < int((~fin).sum()) <= 9 * 24
+    assert torch.equal(fin, torch.isfinite(a))
+    assert float((a[fin] - b[fin]).abs().max()) < 64 * 2.0 ** -53 * float(b[fin].abs().max())
+
+
+def test_copies_of_a_field_follow_its_changes():
+    dims, block = (8, 8, 8, 8), (4, 4, 4, 4)
+    ctx, _ = _ctx(dims, block)
+    nat = native(ctx, seeded.spinor(dims, 6))
+    first = _apply(ctx, nat, ps.OP_FULL).clone()
+    ps.psms_gauge_sweep(ctx, 0, ps.ACTIVE_ALL, 1, 0, 5.3, 3, 0)
+    a, b = _apply(ctx, nat, ps.OP_FULL), _apply(ctx, nat, ps.OP_FULL, graph=True)
+    assert float((a - b).abs().max() / b.abs().max()) < 64 * 2.0 ** -53
+    assert float((a - first).abs().max()) > 1e-3
+
+
+# every way to cut 256 sites that the link layout of the block solver treats apart, odd block counts among them
+@pytest.mark.parametrize("dims,block", [((4, 4, 4, 4), (4, 4, 4, 4)), ((8, 4, 4, 2), (8, 4, 4, 2)),
+                                        ((4, 4, 12, 8), (4, 4, 2, 8)), ((16, 4, 4, 4), (16, 4, 2, 2)),
+                                        ((2, 2, 4, 32), (2, 2, 2, 32)), ((32, 4, 2, 4), (32, 2, 2, 2)),
+                                        ((12, 4, 4, 4), (4, 4, 4, 4))])
+@pytest.mark.parametrize("krylov", [None, ps.SOLVER_CGNR, ps.SOLVER_BICGSTAB])
+def test_block_solver_shapes(dims, block, krylov):
+    assert int(np.prod(block)) == 256
+    ctx, U = _ctx(dims, block, kappa=0.156, eps=0.5)
+    if krylov is not None:
+        ps.psms_block_krylov(ctx, krylov)
+    geom = lattice.Geometry(dims, block)
+    b = seeded.spinor(dims, 7)
+    nat = native(ctx, b)
+    x = torch.zeros_like(nat)
+    info = ps.psms_solve(ctx, 0, ps.OP_BLOCKS, nat, x, 1e-13, 20000, ps.PREC_F32)
+    assert info["true_residual"] <= 1e-13
+    got = canonical(ctx, x)
+    r = b - dirac.apply_D(U, got, 0.156, geom, mode="block")
+    assert np.sqrt(np.sum(np.abs(r) ** 2) / np.sum(np.abs(b) ** 2)) < 2e-13
+    last = geom.n_blocks - 1
+    ref = estimator.solve_blocks(U, b, geom, 0.156, [last], 1e-14)
+    assert rel_err(dirac.extract_block(got, geom, last), dirac.extract_block(ref, geom, last)) < 1e-11
+
+
+def test_block_solver_right_hand_sides():
+    """A zero block, a block with an even half only, and the iteration cap."""
+    dims, block = (8, 4, 4, 4), (4, 4, 4, 4)
+    ctx, U = _ctx(dims, block, kappa=0.156, eps=0.5)
+    geom = lattice.Geometry(dims, block)
+    b = seeded.spinor(dims, 8)
+    b[:4] = 0
+    b[4:][geom.parity[4:] == 1] = 0
+    nat = native(ctx, b)
+    x = torch.zeros_like(nat)
+    info = ps.psms_solve(ctx, 0, ps.OP_BLOCKS, nat, x, 1e-13, 20000, ps.PREC_F32)
+    got = canonical(ctx, x)
+    assert info["true_residual"] <= 1e-13 and np.abs(got[:4]).max() == 0.0
+    r = b - dirac.apply_D(U, got, 0.156, geom, mode="block")
+    assert np.sqrt(np.sum(np.abs(r) ** 2) / np.sum(np.abs(b) ** 2)) < 2e-13
+    with pytest.raises(ps.PsmsError) as e:
+        ps.psms_solve(ctx, 0, ps.OP_BLOCKS, nat, x, 1e-13, 3, ps.PREC_F32)
+    assert e.value.status == 4  # PSMS_ENOCONV
+
+
+# 16 sites (one sub-panel row per thread), 64, 256, and 512 sites (the tall panels)
+@pytest.mark.parametrize("dims,block", [((4, 4, 4, 2), (2, 2, 2, 2)), ((4, 4, 4, 4), (4, 4, 2, 2)),
+                                        ((4, 4, 4, 8), (4, 4, 4, 4)), ((8, 4, 4, 4), (8, 4, 4, 4))])
+def test_lu_sizes_against_torch(dims, block):
+    kappa = 0.15
+    ctx, U = _ctx(dims, block, kappa=kappa)
+    geom = lattice.Geometry(dims, block)
+    got = ps.psms_block_logdet(ctx, 0)
+    for b in sorted({0, geom.n_blocks - 1}):
+        ref = _dense_logdet(dirac.extract_block(U, geom, b), block, kappa)
+        assert abs(got[b] - ref) < 1e-11 * abs(ref)
+
+
+def _dense_logdet(Ub, block, kappa):
+    """ln |det D_b| from torch's LU of A - D_oe D_eo / A, the hops written into a dense matrix."""
+    A = 1.0 / (2.0 * kappa)
+    n = int(np.prod(block))
+    u = torch.from_numpy(np.ascontiguousarray(Ub)).cuda()
+    D = torch.zeros(n, 4, 3, n, 4, 3, dtype=torch.complex128, device="cuda")
+    g = torch.arange(n, device="cuda").reshape(block)
+    for mu in range(4):
+        x, y = g.narrow(mu, 0, block[mu] - 1).reshape(-1), g.narrow(mu, 1, block[mu] - 1).reshape(-1)
+        w = u[..., mu, :, :].reshape(n, 3, 3)[x]
+        gm = torch.from_numpy(np.asarray(GAMMA[mu], dtype=np.complex128)).cuda()
+        one = torch.eye(4, dtype=torch.complex128, device="cuda")
+        for t, src, dst, m in ((-1.0, y, x, w), (1.0, x, y, w.conj().transpose(-1, -2))):
+            D[dst, :, :, src, :, :] += -0.5 * (one + t * gm)[None, :, None, :, None] * m[:, None, :, None, :]
+    par = torch.from_numpy((np.indices(block).sum(0) % 2).reshape(-1)).cuda()
+    o, e = torch.nonzero(par == 1).reshape(-1), torch.nonzero(par == 0).reshape(-1)
+    D = D.reshape(n, 12, n, 12)
+    oe, eo = D[o][:, :, e].reshape(6 * n, 6 * n), D[e][:, :, o].reshape(6 * n, 6 * n)
+    M = A * torch.eye(6 * n, dtype=torch.complex128, device="cuda") - (oe @ eo) / A
+    return 6 * n * np.log(A) + torch.linalg.slogdet(M).logabsdet.item()
