@@ -31,7 +31,8 @@ long long &launch_counter() {
     return n;
 }
 
-void *scratch(psms_ctx *c, const std::string &name, size_t bytes) {
+static cudaError_t scratch_get(psms_ctx *c, const std::string &name, size_t bytes, void **out) {
+    *out = nullptr;
     if (bytes == 0) bytes = 16;
     DevBuf &b = c->scratch[name];
     if (b.bytes < bytes) {
@@ -41,10 +42,29 @@ void *scratch(psms_ctx *c, const std::string &name, size_t bytes) {
             b.p = nullptr;
             b.bytes = 0;
         }
-        cuda_check(cudaMalloc(&b.p, bytes), ("scratch alloc " + name).c_str());
+        const cudaError_t e = cudaMalloc(&b.p, bytes);
+        if (e != cudaSuccess) {
+            b.p = nullptr;
+            return e;
+        }
         b.bytes = bytes;
     }
-    return b.p;
+    *out = b.p;
+    return cudaSuccess;
+}
+
+void *scratch(psms_ctx *c, const std::string &name, size_t bytes) {
+    void *p;
+    cuda_check(scratch_get(c, name, bytes, &p), ("scratch alloc " + name).c_str());
+    return p;
+}
+
+void *scratch_try(psms_ctx *c, const std::string &name, size_t bytes) {
+    void *p;
+    const cudaError_t e = scratch_get(c, name, bytes, &p);
+    if (e != cudaErrorMemoryAllocation) cuda_check(e, ("scratch alloc " + name).c_str());
+    else cudaGetLastError();  // cleared: the caller does without
+    return p;
 }
 
 void check_field(psms_ctx *c, int f) {
@@ -61,6 +81,16 @@ float2 *links32(psms_ctx *c, int f) {
     return c->U32[f];
 }
 
+void fx_wait(psms_ctx *c) {
+    if (c->fx_ev && c->fx_stream != c->stream) cuda_check(cudaStreamWaitEvent(c->stream, c->fx_ev, 0), "stream order");
+}
+
+void fx_mark(psms_ctx *c) {
+    if (!c->fx_ev) cuda_check(cudaEventCreateWithFlags(&c->fx_ev, cudaEventDisableTiming), "event create");
+    cuda_check(cudaEventRecord(c->fx_ev, c->stream), "event record");
+    c->fx_stream = c->stream;
+}
+
 const int4 *links_fx(psms_ctx *c, int f) {
     check_field(c, f);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -71,8 +101,10 @@ const int4 *links_fx(psms_ctx *c, int f) {
         c->Ufx[f] = nullptr;
         return nullptr;
     }
+    fx_wait(c);
     if (!c->ufx_ok[f]) {
         links_to_fx(c, c->U64[f], 0, c->Ufx[f], 1);
+        fx_mark(c);
         c->ufx_ok[f] = 1;
     }
     return c->Ufx[f];
@@ -259,6 +291,7 @@ static void free_ctx(psms_ctx *c) {
         if (kv.second.p) cudaFree(kv.second.p);
     for (auto e : c->ev_pool) cudaEventDestroy(e);
     for (auto e : c->ev_pool_b) cudaEventDestroy(e);
+    if (c->fx_ev) cudaEventDestroy(c->fx_ev);
     if (c->d_prof_sites) cudaFree(c->d_prof_sites);
     if (c->d_binfo) cudaFree(c->d_binfo);
     if (c->mlp && c->mlp_free) c->mlp_free(c->mlp);

@@ -49,6 +49,10 @@ struct psms_ctx {
     std::vector<int> u32_ok;
     std::vector<int4 *> Ufx;      // fixed-point copies (fixed.cuh), valid when ufx_ok
     std::vector<int> ufx_ok;
+    // last use of the fixed-point copies' scratch, or their last conversion:
+    // calls on another stream wait for it (psms_dw_apply does not synchronise)
+    cudaEvent_t fx_ev = nullptr;
+    cudaStream_t fx_stream = nullptr;
     std::vector<psms::BlockInfo> h_binfo;
     psms::BlockInfo *d_binfo = nullptr;
     cudaStream_t stream = nullptr;
@@ -98,6 +102,8 @@ namespace psms {
 
 // grow-only named scratch buffer
 void *scratch(psms_ctx *c, const std::string &name, size_t bytes);
+// the same; null when there is no room
+void *scratch_try(psms_ctx *c, const std::string &name, size_t bytes);
 // FP32 copy of a gauge slot (converted on first use after a change)
 float2 *links32(psms_ctx *c, int field);
 // fixed-point copy of a gauge slot, made on first use after a change; null
@@ -105,6 +111,9 @@ float2 *links32(psms_ctx *c, int field);
 // has to read the slot itself, which may change before the graph runs):
 // the caller then uses the FP64 links
 const int4 *links_fx(psms_ctx *c, int field);
+// order this stream's use of the fixed-point copies after another's (fx_ev)
+void fx_wait(psms_ctx *c);
+void fx_mark(psms_ctx *c);
 inline void touch_field(psms_ctx *c, int f) { c->u32_ok[f] = c->ufx_ok[f] = 0; }
 void check_field(psms_ctx *c, int f);
 

@@ -823,12 +823,27 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     }
     const int nct = hop_ctas(c, h);
     const int nsys = h.sys_map ? h.n_map : h.n_sys;
-    const bool fixed = std::is_same<S, Store<double>>::value && h.fx != nullptr;
+    if (nct == 0 || nsys == 0) return 0;
+    // FP64 hops in fixed point (fixed.cuh).  Few output sites (below four
+    // warps per scheduler over the chip), or a few blocks of a large lattice:
+    // the directions of a site go to eight warps, which convert what they
+    // read; else a pass converts the input first (no room for its copy: the
+    // FP64 kernel)
+    bool fixed = std::is_same<S, Store<double>>::value && h.fx != nullptr;
+    const long long per = (h.p < 0 ? 2LL : 1LL) * a.n_ranks * c->g.Vbh;
+    const bool fx_split = !h.partial && (per * nsys <= FX_SPLIT_SITES || 8LL * a.n_ranks <= c->g.nblocks);
+    if (fixed && !fx_split) {
+        a.fxs_bs = fx_spinors(a.in.cs);
+        a.fxs = (longlong2 *)scratch_try(c, "hop_fx", sizeof(longlong2) * (size_t)a.fxs_bs * h.n_sys);
+        if (!a.fxs) {
+            if (!h.U) fail(PSMS_ENOMEM, "hop: no room for the input in fixed point");
+            fixed = false;
+        }
+    }
     if (fixed) {
         a.U = h.fx;
         a.U_bs = h.fx_bs;
     }
-    if (nct == 0 || nsys == 0) return 0;
     a.nct = nct;
     // shared-endpoint links: the systems of a launch run side by side (CTA
     // index = cta * nsys + system), so each endpoint link leaves HBM once
@@ -851,26 +866,19 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     }
     if constexpr (std::is_same<S, Store<double>>::value) {
         if (fixed) {
-            // FP64 hops in fixed point (fixed.cuh).  Few output sites (below
-            // four warps per scheduler over the chip), or a few blocks of a
-            // large lattice: the directions of a site go to eight warps, which
-            // convert what they read; else a pass converts the input first
-            const long long per = (h.p < 0 ? 2LL : 1LL) * a.n_ranks * c->g.Vbh;
-            if (!h.partial && (per * nsys <= FX_SPLIT_SITES || 8LL * a.n_ranks <= c->g.nblocks)) {
+            if (fx_split) {
                 const auto fn = h.dag ? hop_fx_split_kernel<true> : hop_fx_split_kernel<false>;
                 cuda_check(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)sizeof(FxSplitShared)),
                            "hop shared memory");
                 fn<<<dim3((unsigned)((per + 31) / 32), nsys), 256, sizeof(FxSplitShared), c->stream>>>(a);
             } else {
-                const long long fs = fx_spinors(a.in.cs);
-                longlong2 *x = (longlong2 *)scratch(c, "hop_fx", sizeof(longlong2) * (size_t)fs * h.n_sys);
-                spinor_fx_kernel<<<dim3((unsigned)((a.in.cs + 255) / 256), nsys), 256, 0, c->stream>>>(a.in, x, fs, h.sys_map,
-                                                                                                   h.active);
+                fx_wait(c);
+                spinor_fx_kernel<<<dim3((unsigned)((a.in.cs + 255) / 256), nsys), 256, 0, c->stream>>>(
+                    a.in, const_cast<longlong2 *>(a.fxs), a.fxs_bs, h.sys_map, h.active);
                 PSMS_LAUNCH_CHECK("spinor_fx_kernel");
-                a.fxs = x;
-                a.fxs_bs = fs;
-                (h.dag ? hop_fx_kernel<HOP_NT, 3, true> : hop_fx_kernel<HOP_NT, 3, false>)<<<grid, HOP_NT, 0, c->stream>>>(a);
+                (h.dag ? hop_fx_kernel<HOP_NT, 4, true> : hop_fx_kernel<HOP_NT, 4, false>)<<<grid, HOP_NT, 0, c->stream>>>(a);
+                fx_mark(c);
             }
             PSMS_LAUNCH_CHECK("hop_fx_kernel");
             if (slot >= 0) prof_end(c, slot, bytes);

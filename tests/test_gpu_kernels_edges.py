@@ -52,6 +52,25 @@ def test_fixed_point_hops_against_the_fp64_form(dims, block, op):
     assert float((a - b).abs().max() / b.abs().max()) < 64 * 2.0 ** -53
 
 
+def test_hops_alternating_between_streams():
+    dims = (16, 16, 16, 16)  # the form that keeps the input in scratch
+    ctx, _ = _ctx(dims, (4, 4, 4, 4))
+    nats = [native(ctx, seeded.spinor(dims, k)) for k in range(4)]
+    refs = [_apply(ctx, nat, ps.OP_FULL) for nat in nats]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    outs = [[torch.zeros_like(nat) for nat in nats] for _ in range(8)]
+    torch.cuda.synchronize()
+    for row in outs:
+        for k, nat in enumerate(nats):
+            ps.psms_set_stream(ctx, streams[k % 2])
+            ps.psms_dw_apply(ctx, 0, ps.OP_FULL, nat, row[k], ps.PREC_F64)
+    ps.psms_set_stream(ctx, None)
+    torch.cuda.synchronize()
+    for row in outs:
+        for out, ref in zip(row, refs):
+            assert torch.equal(out.view(torch.float64), ref)
+
+
 @pytest.mark.parametrize("dims,block", [((4, 4, 4, 4), (2, 2, 2, 2)), ((16, 16, 16, 8), (4, 4, 4, 4))])
 @pytest.mark.parametrize("scale", [2.0 ** -1000, 2.0 ** -850, 2.0 ** 850, 2.0 ** 1000])
 def test_hops_at_the_ends_of_the_fp64_range(dims, block, scale):
