@@ -98,27 +98,47 @@ __device__ __forceinline__ SU3<typename SL::R> hop_link(const HopArgs<E> &a, con
 template <class E>
 __device__ __forceinline__ bool hop_site(const HopArgs<E> &a, const Geom &g, long long t, long long total, int &p,
                                          int &r, int &j) {
+    bool work = t < total;
     p = r = j = 0;
-    if (t >= total) return false;
-    // both parities: block-major order (block, parity, site) so that the two
-    // endpoints of a block's links are processed close in time and each link
-    // is fetched from HBM about once per launch
-    const int both = a.p < 0 ? 1 : 0;
-    r = a.rank_lo + (int)(t >> (g.vbh_sh + both));
-    p = both ? (int)((t >> g.vbh_sh) & 1) : a.p;
-    j = (int)(t & (g.Vbh - 1));
-    if (a.n_ranks == g.nblocks && g.coloured) {
-        // whole lattice: walk the blocks in lexicographic order (colours
-        // interleaved), so that the faces a block reads from its neighbours
-        // were loaded by CTAs that ran just before and are still in L2
-        int B[4], rem = r;
-        for (int m = 3; m >= 0; --m) {
-            B[m] = rem % g.nb[m];
-            rem /= g.nb[m];
+    if (work) {
+        // both parities: block-major order (block, parity, site) so that the
+        // two endpoints of a block's links are processed close in time and
+        // each link is fetched from HBM about once per launch
+        if (a.p < 0) {
+            r = a.rank_lo + (int)(t >> (g.vbh_sh + 1));
+            p = (int)((t >> g.vbh_sh) & 1);
+            j = (int)(t & (g.Vbh - 1));
+            if (a.n_ranks == g.nblocks) {
+                // whole lattice: walk the blocks in lexicographic order, so
+                // that a block's neighbours (opposite colour) are processed
+                // soon after it and face data is still in L2
+                int B[4], rem = r;
+                for (int m = 3; m >= 0; --m) {
+                    B[m] = rem % g.nb[m];
+                    rem /= g.nb[m];
+                }
+                r = rank_of_lex(g, r, B);
+            }
+        } else {
+            p = a.p;
+            r = a.rank_lo + (int)(t >> g.vbh_sh);
+            j = (int)(t & (g.Vbh - 1));
+            if (a.n_ranks == g.nblocks && g.coloured) {
+                // whole lattice, one parity: walk the blocks in lexicographic
+                // order (colours interleaved), so that the faces a block
+                // reads from its neighbours were loaded by CTAs that ran
+                // just before and are still in L2
+                int B[4], rem = r;
+                for (int m = 3; m >= 0; --m) {
+                    B[m] = rem % g.nb[m];
+                    rem /= g.nb[m];
+                }
+                r = rank_of_lex(g, r, B);
+            }
         }
-        r = rank_of_lex(g, r, B);
+        work = !a.rank_active || a.rank_active[r];
     }
-    return !a.rank_active || a.rank_active[r];
+    return work;
 }
 
 template <int NT>
@@ -143,15 +163,20 @@ __device__ __forceinline__ void hop_dirs(const HopArgs<E> &a, const Geom &g, con
                                          const typename SL::elem *U, typename SL::R sg,
                                          Spinor<typename SL::R> &acc) {
     using R = typename SL::R;
-    long long snb[8];
-    int bsg[8];
+    // (below 2^31 sites: 32-bit indices keep the eight neighbours in registers)
+    const int off = (int)a.in.off;
+    int snb[8], bsg[8];
 #pragma unroll
-    for (int d = D0; d < D1; ++d) neighbour(g, bi, r, p, y, ll, d >> 1, (d & 1) ? -1 : 1, HOP_ALL, snb[d], bsg[d]);
+    for (int d = D0; d < D1; ++d) {
+        long long sn;
+        neighbour(g, bi, r, p, y, ll, d >> 1, (d & 1) ? -1 : 1, HOP_ALL, sn, bsg[d]);
+        snb[d] = (int)sn;
+    }
 #pragma unroll
     for (int d = D0; d < D1; ++d) {
         const int mu = d >> 1;
         const bool fwd = (d & 1) == 0;
-        Spinor<R> v = load_spinor_ro<S>(in, a.in.cs, snb[d] - a.in.off);
+        Spinor<R> v = load_spinor_ro<S>(in, a.in.cs, snb[d] - off);
         const R tt = fwd ? -sg : sg;
         Half<R> h = project(mu, tt, v);
         if (mu == 0) {
@@ -162,7 +187,7 @@ __device__ __forceinline__ void hop_dirs(const HopArgs<E> &a, const Geom &g, con
 #pragma unroll
                 for (int c = 0; c < 3; ++c) h.c[q][c] = bsr * h.c[q][c];
         }
-        SU3<R> u = hop_link<SL, LI>(a, U, k, mu, fwd ? s : snb[d]);
+        SU3<R> u = hop_link<SL, LI>(a, U, k, mu, fwd ? s : (long long)snb[d]);
         reconstruct_add(mu, tt, fwd ? su3_mul(u, h) : su3_dag_mul(u, h), acc);
     }
 }
@@ -226,7 +251,9 @@ __device__ __forceinline__ void hop_stage(const HopArgs<E> &a, const double sum[
 // no divergence); the second half's partial spinors join the first's
 // through shared memory and the first half finishes the site -- half the
 // per-thread state, twice the threads in flight.
-template <class S, class SL, int NT, int MINB, int ALL, int LI = 0, int SPLIT = 0>
+// DOT = 1: with the reduction of a BiCGStab half iteration (a form of its own:
+// its seven sums would cost the plain operator registers).
+template <class S, class SL, int NT, int MINB, int ALL, int LI = 0, int SPLIT = 0, int DOT = 0>
 __global__ void __launch_bounds__(NT, MINB) hop_kernel(const HopArgs<typename S::elem> a) {
     using R = typename SL::R;
     using E = typename S::elem;
@@ -356,7 +383,7 @@ __global__ void __launch_bounds__(NT, MINB) hop_kernel(const HopArgs<typename S:
                 for (int c = 0; c < 3; ++c) o.c[q][c] = o.c[q][c] + ca * v.c[q][c];
         }
         store_spinor<S>(a.out.p + k * a.out.bs, a.out.cs, s - a.out.off, o);
-        if (a.dot) {
+        if constexpr (DOT) {
             const Spinor<R> x = load_spinor<S>(a.dx.p + k * a.dx.bs, a.dx.cs, s - a.dx.off);
             Spinor<R> yv;
             if (a.dot == 2) yv = load_spinor<S>(a.y.p + k * a.y.bs, a.y.cs, s - a.y.off);
@@ -373,7 +400,7 @@ __global__ void __launch_bounds__(NT, MINB) hop_kernel(const HopArgs<typename S:
         double tot = block_sum<NT>(nrm, sh);
         if (threadIdx.x == 0) a.partial[(long long)k * a.nct + bx] = tot;
     }
-    if (a.dot) {
+    if constexpr (DOT) {
         __shared__ double shd[BCG_SUMS][NT / 32];
         hop_stage<NT>(a, dsum, shd, k, bx);
     }
@@ -760,6 +787,37 @@ __global__ void __launch_bounds__(NT, MINB) hop_staged_kernel(const HopArgs<type
 static constexpr int HOP_NT = 128;
 constexpr long long FX_SPLIT_SITES = 152 * 128;  // output sites of all systems
 
+// The FP32 forms, by the number psms_hop_variant takes.  part: general form,
+// register caps 2, 6, 7, 8 CTAs/SM.  whole (whole lattice): the same, the
+// branch-free form with caps 4 to 7, two threads per site (8, 9), staged forms
+// (10 to 13: blocks of 2 x 128 sites only).
+// li (whole lattice, links shared by the endpoints): caps 2 to 8, general and
+// branch-free forms, flagged or unconditional U1 reads, two threads per site
+// (13, 14).
+template <class S, class SL, int D>
+struct HopVars {
+    using KFn = void (*)(const HopArgs<typename S::elem>);
+    static constexpr int N = HOP_NT, W = 2 * HOP_NT;
+    static constexpr KFn part[] = {hop_kernel<S, SL, N, 2, 0, 0, 0, D>, hop_kernel<S, SL, N, 6, 0, 0, 0, D>,
+                                   hop_kernel<S, SL, N, 7, 0, 0, 0, D>, hop_kernel<S, SL, N, 8, 0, 0, 0, D>};
+    static constexpr KFn whole[] = {part[0], part[1], part[2], part[3],
+                                    hop_kernel<S, SL, N, 4, 1, 0, 0, D>, hop_kernel<S, SL, N, 5, 1, 0, 0, D>,
+                                    hop_kernel<S, SL, N, 6, 1, 0, 0, D>, hop_kernel<S, SL, N, 7, 1, 0, 0, D>,
+                                    hop_kernel<S, SL, W, 3, 1, 0, 1, D>, hop_kernel<S, SL, W, 4, 1, 0, 1, D>,
+                                    hop_staged_kernel<S, SL, N, 4>, hop_staged_kernel<S, SL, N, 6>,
+                                    hop_staged_kernel<S, SL, N, 4, 1>, hop_staged_kernel<S, SL, N, 6, 1>};
+    static constexpr int whole_nt[] = {N, N, N, N, N, N, N, N, W, W, N, N, N, N};
+    static constexpr KFn li[] = {hop_kernel<S, SL, N, 2, 0, 1, 0, D>, hop_kernel<S, SL, N, 4, 0, 1, 0, D>,
+                                 hop_kernel<S, SL, N, 2, 1, 1, 0, D>, hop_kernel<S, SL, N, 3, 1, 1, 0, D>,
+                                 hop_kernel<S, SL, N, 4, 1, 1, 0, D>, hop_kernel<S, SL, N, 5, 1, 1, 0, D>,
+                                 hop_kernel<S, SL, N, 6, 0, 1, 0, D>, hop_kernel<S, SL, N, 8, 0, 1, 0, D>,
+                                 hop_kernel<S, SL, N, 6, 1, 1, 0, D>, hop_kernel<S, SL, N, 4, 0, 2, 0, D>,
+                                 hop_kernel<S, SL, N, 6, 0, 2, 0, D>, hop_kernel<S, SL, N, 4, 1, 2, 0, D>,
+                                 hop_kernel<S, SL, N, 6, 1, 2, 0, D>, hop_kernel<S, SL, W, 2, 1, 1, 1, D>,
+                                 hop_kernel<S, SL, W, 3, 1, 1, 1, D>};
+    static constexpr int li_nt[] = {N, N, N, N, N, N, N, N, N, N, N, N, N, W, W};
+};
+
 int hop_ctas(psms_ctx *c, const HopCall &h) {
     const int nr = h.n_ranks < 0 ? c->g.nblocks : h.n_ranks;
     const long long total = (h.p < 0 ? 2LL : 1LL) * nr * c->g.Vbh;
@@ -892,8 +950,6 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     // y2, U only), so the extra tuning launches leave the result unchanged.
     using KFn = void (*)(const HopArgs<E>);
     constexpr bool f32 = sizeof(typename SL::R) == 4;
-    // FP32 links: register caps 2, 6, 7, 8 CTAs/SM; for the whole lattice
-    // (HOP_ALL) the branch-free specialisation with caps 4, 5, 6, 7 besides
     const bool all = h.mode == HOP_ALL;
     // the staged kernel: whole lattice, 128 sites of each parity per block
     const bool staged = all && a.n_ranks == c->g.nblocks && h.rank_lo == 0 && c->g.Vbh == HOP_NT;
@@ -901,34 +957,14 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     const int *thr = nullptr;  // threads per CTA of each variant (null: all HOP_NT)
     int nvar;
     if constexpr (f32) {
-        static const KFn v32[] = {hop_kernel<S, SL, HOP_NT, 2, 0>, hop_kernel<S, SL, HOP_NT, 6, 0>,
-                                  hop_kernel<S, SL, HOP_NT, 7, 0>, hop_kernel<S, SL, HOP_NT, 8, 0>};
-        static const KFn v32all[] = {hop_kernel<S, SL, HOP_NT, 2, 0>, hop_kernel<S, SL, HOP_NT, 6, 0>,
-                                     hop_kernel<S, SL, HOP_NT, 7, 0>, hop_kernel<S, SL, HOP_NT, 8, 0>,
-                                     hop_kernel<S, SL, HOP_NT, 4, 1>, hop_kernel<S, SL, HOP_NT, 5, 1>,
-                                     hop_kernel<S, SL, HOP_NT, 6, 1>, hop_kernel<S, SL, HOP_NT, 7, 1>,
-                                     hop_kernel<S, SL, 2 * HOP_NT, 3, 1, 0, 1>, hop_kernel<S, SL, 2 * HOP_NT, 4, 1, 0, 1>,
-                                     hop_staged_kernel<S, SL, HOP_NT, 4>, hop_staged_kernel<S, SL, HOP_NT, 6>,
-                                     hop_staged_kernel<S, SL, HOP_NT, 4, 1>, hop_staged_kernel<S, SL, HOP_NT, 6, 1>};
-        static const int t32all[] = {HOP_NT, HOP_NT, HOP_NT, HOP_NT, HOP_NT, HOP_NT, HOP_NT,
-                                     HOP_NT, 2 * HOP_NT, 2 * HOP_NT, HOP_NT, HOP_NT, HOP_NT, HOP_NT};
-        // shared-endpoint links (whole lattice): register caps 2-8 CTAs/SM,
-        // general and branch-free forms, flagged or unconditional U1 reads
-        static const KFn v32li[] = {hop_kernel<S, SL, HOP_NT, 2, 0, 1>, hop_kernel<S, SL, HOP_NT, 4, 0, 1>,
-                                    hop_kernel<S, SL, HOP_NT, 2, 1, 1>, hop_kernel<S, SL, HOP_NT, 3, 1, 1>,
-                                    hop_kernel<S, SL, HOP_NT, 4, 1, 1>, hop_kernel<S, SL, HOP_NT, 5, 1, 1>,
-                                    hop_kernel<S, SL, HOP_NT, 6, 0, 1>, hop_kernel<S, SL, HOP_NT, 8, 0, 1>,
-                                    hop_kernel<S, SL, HOP_NT, 6, 1, 1>, hop_kernel<S, SL, HOP_NT, 4, 0, 2>,
-                                    hop_kernel<S, SL, HOP_NT, 6, 0, 2>, hop_kernel<S, SL, HOP_NT, 4, 1, 2>,
-                                    hop_kernel<S, SL, HOP_NT, 6, 1, 2>,
-                                    hop_kernel<S, SL, 2 * HOP_NT, 2, 1, 1, 1>, hop_kernel<S, SL, 2 * HOP_NT, 3, 1, 1, 1>};
-        static const int t32li[] = {HOP_NT, HOP_NT, HOP_NT, HOP_NT, HOP_NT, HOP_NT, HOP_NT, HOP_NT,
-                                    HOP_NT, HOP_NT, HOP_NT, HOP_NT, HOP_NT, 2 * HOP_NT, 2 * HOP_NT};
+        using V = HopVars<S, SL, 0>;
+        vars = shared_links ? V::li : (all ? V::whole : V::part);
+        thr = shared_links ? V::li_nt : (all ? V::whole_nt : nullptr);
+        if constexpr (std::is_same<S, Store<float>>::value) {
+            using D = HopVars<S, SL, 1>;
+            if (a.dot) vars = shared_links ? D::li : (all ? D::whole : D::part);
+        }
         if (shared_links && !all) fail(PSMS_EINVAL, "hop_launch: shared-endpoint links on whole-lattice hops only");
-        vars = shared_links ? v32li : (all ? v32all : v32);
-        thr = shared_links ? t32li : (all ? t32all : nullptr);
-        // two-threads-per-site forms: v32all entries 8, 9 and v32li 13, 14;
-        // staged forms: v32all 10 to 13 (blocks of 2 x 128 sites only)
         nvar = shared_links ? 15 : (all ? (staged ? 14 : 10) : 4);
     } else {
         // FP64 (ALU bound): the general form, and for the whole lattice the
@@ -968,7 +1004,7 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     }
     int v = (choice >= 0 && choice < nvar) ? choice : (f32 ? 1 : 0);
     if (c->forced_hop_variant >= 0) v = c->forced_hop_variant % nvar;
-    // the staged kernels (v32all entries 10 to 13) carry no fused reduction
+    // the staged kernels (10 to 13) carry no fused reduction
     if (a.dot && !shared_links && all && v >= 10) v = 6;
     vars[v]<<<grid, thr ? thr[v] : HOP_NT, 0, c->stream>>>(a);
     PSMS_LAUNCH_CHECK("hop_kernel");
