@@ -294,6 +294,7 @@ static void free_ctx(psms_ctx *c) {
     if (c->fx_ev) cudaEventDestroy(c->fx_ev);
     if (c->d_prof_sites) cudaFree(c->d_prof_sites);
     if (c->d_binfo) cudaFree(c->d_binfo);
+    if (c->d_gauss) cudaFree(c->d_gauss);
     if (c->mlp && c->mlp_free) c->mlp_free(c->mlp);
     delete c;
 }
@@ -365,6 +366,7 @@ psms_status psms_create(const psms_lattice_desc *desc, psms_ctx **out) {
             unit_links_kernel<<<(unsigned)((n + 255) / 256), 256>>>(c->U64[f], c->g.V);
             PSMS_LAUNCH_CHECK("unit links");
         }
+        noise_tables(c);
         cuda_check(cudaDeviceSynchronize(), "create sync");
     } catch (const Error &e) {
         psms_status st = e.st;

@@ -55,6 +55,7 @@ struct psms_ctx {
     cudaStream_t fx_stream = nullptr;
     std::vector<psms::BlockInfo> h_binfo;
     psms::BlockInfo *d_binfo = nullptr;
+    void *d_gauss = nullptr;  // tables of the noise (gauss.cuh)
     cudaStream_t stream = nullptr;
     std::string err;
     std::map<std::string, psms::DevBuf> scratch;

@@ -14,6 +14,7 @@
 // i), and all blocks of a level are solved by one persistent launch.
 #include "estimator.hpp"
 #include "fixed.cuh"
+#include "gauss.cuh"
 #include "interp_plan.hpp"
 #include "gauge.hpp"
 #include "solver.hpp"
@@ -55,36 +56,62 @@ __device__ __forceinline__ void apply_P(const Geom &g, int r, const int y[4], Sp
         for (int b = 0; b < 3; ++b) v.c[a][b] = 0.5 * v.c[a][b];
 }
 
-__global__ void noise_kernel(Geom g, const BlockInfo *binfo, double2 *out, long long bs, uint64_t seed,
-                             uint64_t counter, uint64_t level, int proj, int i0) {
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.V) return;
+constexpr int NOISE_NT = 128;
+
+// One site of one system per thread (gauss.cuh says what bounds it); the tables
+// are copied to shared memory, where lanes look up different entries.
+__global__ void __launch_bounds__(NOISE_NT) noise_kernel(Geom g, const BlockInfo *binfo, const GaussTables *tables,
+                                                         double2 *out, long long bs, uint64_t seed, uint64_t counter,
+                                                         uint64_t level, int proj, int i0) {
+    __shared__ GaussTables T;
+    {
+        const uint64_t *src = reinterpret_cast<const uint64_t *>(tables);
+        uint64_t *dst = reinterpret_cast<uint64_t *>(&T);
+        for (int t = threadIdx.x; t < (int)(sizeof(GaussTables) / 8); t += NOISE_NT) dst[t] = __ldg(src + t);
+    }
+    __syncthreads();
     const uint64_t i = blockIdx.y;
-    int p, r, j, y[4], x[4];
-    decode(g, binfo, s, p, r, j, y, x);
-    const uint64_t lex = (uint64_t)lex_index(g, x);
     const uint64_t stream = (level << 32) | (uint64_t)(i0 + i);
-    Spinor<double> v;
-    for (int jj = 0; jj < 6; ++jj) {
-        uni4 u = uniforms(seed, TAG_NOISE, counter, stream, lex, (uint64_t)jj);
-        for (int m = 0; m < 2; ++m) {
-            const double rad = sqrt(-log(u.u[2 * m]));
-            // e^{2 pi i u_b}: one sincospi call (exact argument reduction)
-            double sn, cs;
-            sincospi(2.0 * u.u[2 * m + 1], &sn, &cs);
-            const int comp = 2 * jj + m;
-            v.c[comp / 3][comp % 3] = {rad * cs, rad * sn};
+    for (long long s = (long long)blockIdx.x * NOISE_NT + threadIdx.x; s < g.V; s += (long long)gridDim.x * NOISE_NT) {
+        int p, r, j, y[4], x[4];
+        decode(g, binfo, s, p, r, j, y, x);
+        const uint64_t lex = (uint64_t)lex_index(g, x);
+        Spinor<double> v;
+#pragma unroll 1
+        for (int jj = 0; jj < 6; ++jj) {
+            const u64x4 w = philox(counter, stream, lex, (uint64_t)jj, seed, TAG_NOISE);
+            double2 z[2];
+            gauss_pair(T, w.w[0], w.w[1], z[0].x, z[0].y);
+            gauss_pair(T, w.w[2], w.w[3], z[1].x, z[1].y);
+            // (stored at once: the projection, if any, reads them back)
+            out[i * bs + (2 * jj) * g.V + s] = z[0];
+            out[i * bs + (2 * jj + 1) * g.V + s] = z[1];
+        }
+        if (proj) {
+            v = load_spinor<Store<double>>(out + i * bs, g.V, s);
+            apply_P(g, r, y, v);
+            store_spinor<Store<double>>(out + i * bs, g.V, s, v);
         }
     }
-    if (proj) apply_P(g, r, y, v);
-    store_spinor<Store<double>>(out + i * bs, g.V, s, v);
+}
+
+// made with the context, so that a noise call may be captured
+void noise_tables(psms_ctx *c) {
+    static const GaussTables h = [] {
+        GaussTables t;
+        gauss_tables(t);
+        return t;
+    }();
+    cuda_check(cudaMalloc(&c->d_gauss, sizeof(h)), "noise tables");
+    cuda_check(cudaMemcpy(c->d_gauss, &h, sizeof(h), cudaMemcpyHostToDevice), "noise tables");
 }
 
 void noise(psms_ctx *c, double2 *out, int n, uint64_t seed, uint64_t counter, int level, int proj, int i0) {
-    const int NT = 128;
-    dim3 grid((unsigned)((c->g.V + NT - 1) / NT), n);
-    noise_kernel<<<grid, NT, 0, c->stream>>>(c->g, c->d_binfo, out, 12 * c->g.V, seed, counter, (uint64_t)level, proj,
-                                             i0);
+    // about eight CTAs per SM over all systems, so that a CTA's copy of the
+    // tables serves several sites
+    const long long nb = (c->g.V + NOISE_NT - 1) / NOISE_NT, want = (152 * 8 + n - 1) / n;
+    noise_kernel<<<dim3((unsigned)std::min(nb, want), n), NOISE_NT, 0, c->stream>>>(
+        c->g, c->d_binfo, (const GaussTables *)c->d_gauss, out, 12 * c->g.V, seed, counter, (uint64_t)level, proj, i0);
     PSMS_LAUNCH_CHECK("noise");
 }
 

@@ -11,6 +11,7 @@ namespace psms {
 // equal sizes (the last one at most one smaller)
 int chunk_size(psms_ctx *c, int N, double bytes_per_site);
 // noise fields xi_i (i = 0..n-1) for `level`, FP64 full layout, optional P projection
+void noise_tables(psms_ctx *c);  // c->d_gauss
 void noise(psms_ctx *c, double2 *out, int n, uint64_t seed, uint64_t counter, int level, int proj, int i0);
 // d_delta[b * N + i] (b = lexicographic block index); returns total inner iterations
 long long block_level(psms_ctx *c, const double2 *U, const double2 *Up, int N, int mode, uint64_t seed,

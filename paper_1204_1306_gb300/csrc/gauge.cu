@@ -433,8 +433,11 @@ static ActiveList active_list(psms_ctx *c, int all) {
     const auto it = c->scratch.find(name);
     const bool have = it != c->scratch.end() && it->second.p;
     int *d = (int *)scratch(c, name, sizeof(int) * (h.empty() ? 1 : h.size()));
-    if (!have && !h.empty())
-        cuda_check(cudaMemcpy(d, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice), "active list");
+    if (!have && !h.empty()) {
+        cuda_check(cudaMemcpyAsync(d, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, c->stream),
+                   "active list");
+        cuda_check(cudaStreamSynchronize(c->stream), "active list");
+    }
     a.d = d;
     return a;
 }
