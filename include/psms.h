@@ -263,8 +263,8 @@ psms_status psms_dw_apply(psms_ctx *ctx, int field, int op, const void *in_dev, 
 
 /* Solve op(U_field) x = b to |b - op x| <= tol |b| in FP64 (true residual),
  * with inner Krylov iterations on the even-odd operator in inner_prec inside
- * FP64 defect correction: BiCGStab (whole lattice, default) or CGNR (blocks,
- * default), see psms_full_solver / psms_block_krylov.  b, x: native FP64
+ * FP64 defect correction: BiCGStab or CGNR, see psms_full_solver /
+ * psms_block_krylov.  b, x: native FP64
  * buffers.  PSMS_ENOCONV if maxit inner iterations do not reach tol;
  * PSMS_EINVAL for a non-finite b. */
 psms_status psms_solve(psms_ctx *ctx, int field, int op, const void *b_dev, void *x_dev, double tol,
@@ -470,9 +470,11 @@ psms_status psms_inner_reduction(psms_ctx *ctx, double delta);
  * The FP64 true residuals use the FP64 interpolated fields either way, so
  * both reach the same tolerance.  PSMS_EINVAL for another value. */
 psms_status psms_shared_links(psms_ctx *ctx, int on);
-/* Inner Krylov method of the Dirichlet block solves (default CGNR; the
- * autotuner then chooses among that method's variants only, so every tuned
- * choice gives identical results).  PSMS_EINVAL for another kind. */
+/* Inner Krylov method of the Dirichlet block solves (the autotuner then
+ * chooses among that method's variants only, so every tuned choice gives
+ * identical results).  Unless called, blocks of 256 sites with FP32 inner
+ * iterations use BiCGStab and fall back to CGNR per block where it stalls,
+ * all others CGNR.  PSMS_EINVAL for another kind. */
 psms_status psms_block_krylov(psms_ctx *ctx, int kind);
 
 /* Largest number of interpolation steps (systems) batched into one launch

@@ -1,14 +1,18 @@
 // Dirichlet block solver for blocks of 256 sites (4^4 and the other shapes of
-// that volume) with FP32 inner iterations: even-odd CGNR on Dhat^dag Dhat
-// inside the FP64 defect correction of block_solve.cuh, the whole solve of a
-// (block, system) by one CTA of 128 threads.
+// that volume) with FP32 inner iterations on the even-odd operator Dhat inside
+// the FP64 defect correction of block_solve.cuh, the whole solve of a (block,
+// system) by one CTA of 128 threads.  The inner method is BiCGStab unless the
+// context asks for CGNR: a 1e-6 reduction takes 10 iterations of two Dhat
+// against 24 of Dhat and Dhat^dag (4^4 blocks, beta 5.3, kappa 0.156).  An
+// item whose BiCGStab breaks down or fails to reduce the true residual drops
+// that correction and goes on with CGNR.
 //
-// What bounds it: the FP32 pipe.  A hop direction is 108 FP32 instructions on
-// 11 shared-memory loads; an iteration has four half hops.  So what the hops
-// touch lives on the SM: thread j owns odd site j and keeps its parts of res,
-// p and q in registers, the links inside the block (59 KB at 4^4) and the
-// vector that neighbours read (p, q or t; 12 KB) are in shared memory, and
-// three CTAs share an SM.  e and rho, used once an iteration, and the FP64
+// What bounds it: the FP32 pipe and shared memory (a hop direction is 108 FP32
+// instructions on 11 shared-memory loads; an iteration has four half hops).
+// So what the hops touch lives on the SM: thread j owns odd site j and keeps
+// its parts of three vectors in registers, the links inside the block (59 KB
+// at 4^4) and the vector that neighbours read (12 KB) are in shared memory,
+// and three CTAs share an SM.  Vectors used once an iteration, and the FP64
 // right-hand side, solution and residual of the defect correction are in
 // global memory (L2).
 //
@@ -45,44 +49,77 @@ __device__ __forceinline__ float ff_div(ff a, ff b) {
     return q + r / b.hi;
 }
 
-// Sum over the CTA of t >= 0, exact for numbers down to 2^-26 of a warp's
-// largest (50 bits below it): mantissas on the warp's largest exponent, two
-// 25-bit limbs summed by redux, the four warps' sums as 64-bit integers.
-// slot: one of two, alternating (one barrier per sum).
+// Sums over the CTA of N FP32 numbers per thread, exact for numbers down to
+// 2^-26 of a warp's largest (50 bits below it): signed mantissas on the warp's
+// largest exponent, two 25-bit limbs summed by redux, the four warps' sums as
+// 64-bit integers, value i by lane i.  slot: one of two, alternating (one
+// barrier per call).
+constexpr int CG_SUMS = 7;
+
 struct CgSums {
-    int v[2][CG_NT / 32][4];  // exponent, high, low limb sums
+    int4 v[2][CG_NT / 32][CG_SUMS];  // exponent, high, low limb sums
 };
 
-__device__ __forceinline__ ff cg_sum(float t, CgSums &sm, int &slot) {
-    const unsigned b = __float_as_uint(t) & 0x7FFFFFFFu;
-    const int e = (int)(b >> 23);
-    const int em = __reduce_max_sync(0xffffffffu, e);
-    const uint64_t m = e == 0 ? 0 : fx_shr((uint64_t)((b & 0x7FFFFFu) | 0x800000u) << 26, (uint32_t)(em - e));
-    const int hi = __reduce_add_sync(0xffffffffu, (int)(m >> 25)), lo = __reduce_add_sync(0xffffffffu, (int)(m & 0x1FFFFFFu));
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) *reinterpret_cast<int4 *>(sm.v[slot][w]) = make_int4(em, hi, lo, 0);
-    __syncthreads();
-    int E = 0;
-    int4 q[CG_NT / 32];
+template <int N>
+__device__ __forceinline__ void cg_sum(const float *t, ff *out, CgSums &sm, int &slot) {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < CG_NT / 32; ++i) {
-        q[i] = *reinterpret_cast<const int4 *>(sm.v[slot][i]);
-        E = max(E, q[i].x);
+    for (int i = 0; i < N; ++i) {
+        const unsigned b = __float_as_uint(t[i]);
+        const int e = (int)(b >> 23) & 255;
+        const int em = __reduce_max_sync(0xffffffffu, e);
+        const int64_t m =
+            e == 0 ? 0 : (int64_t)fx_shr((uint64_t)((b & 0x7FFFFFu) | 0x800000u) << 26, (uint32_t)(em - e));
+        const int64_t q = (int)b < 0 ? -m : m;
+        const int hi = __reduce_add_sync(0xffffffffu, (int)(q >> 25)),
+                  lo = __reduce_add_sync(0xffffffffu, (int)(q & 0x1FFFFFF));
+        if (l == i) sm.v[slot][w][i] = make_int4(em, hi, lo, 0);
+    }
+    __syncthreads();
+    float rh = 0, rl = 0;
+    if (l < N) {
+        int E = 0;
+        int4 q[CG_NT / 32];
+#pragma unroll
+        for (int i = 0; i < CG_NT / 32; ++i) {
+            q[i] = sm.v[slot][i][l];
+            E = max(E, q[i].x);
+        }
+        int64_t s = 0;
+#pragma unroll
+        for (int i = 0; i < CG_NT / 32; ++i) {
+            const int sh = min(E - q[i].x, 63);
+            s += (((int64_t)q[i].y << 25) + (int64_t)q[i].z) >> sh;
+        }
+        // value = s 2^(E - 176), |s| < 2^57, as the exact sum of three floats
+        const uint64_t a = s < 0 ? (uint64_t)-s : (uint64_t)s;
+        const float p2 = (float)(int)(a >> 48) * pow2f(E - 128), p1 = (float)(int)((a >> 24) & 0xFFFFFF) * pow2f(E - 152),
+                    p0 = (float)(int)(a & 0xFFFFFF) * pow2f(E - 176);
+        const float x = p2 + p1, c = (p1 - (x - p2)) + p0;
+        rh = x + c;
+        rl = c - (rh - x);
+        if (s < 0) rh = -rh, rl = -rl;
+        if (E == 255) rh = rl = __int_as_float(0x7FC00000);  // infinity or NaN among them
     }
     slot ^= 1;
-    uint64_t s = 0;
 #pragma unroll
-    for (int i = 0; i < CG_NT / 32; ++i)
-        s += fx_shr(((uint64_t)(unsigned)q[i].y << 25) + (uint64_t)(unsigned)q[i].z, (uint32_t)(E - q[i].x));
-    // value = s 2^(E - 176), s < 2^57, as the exact sum of three floats
-    const float p2 = (float)(int)(s >> 48) * pow2f(E - 128), p1 = (float)(int)((s >> 24) & 0xFFFFFF) * pow2f(E - 152),
-                p0 = (float)(int)(s & 0xFFFFFF) * pow2f(E - 176);
-    const float a = p2 + p1, c = (p1 - (a - p2)) + p0;
+    for (int i = 0; i < N; ++i) {
+        out[i].hi = __shfl_sync(0xffffffffu, rh, i);
+        out[i].lo = __shfl_sync(0xffffffffu, rl, i);
+    }
+}
+
+__device__ __forceinline__ ff cg_sum1(float t, CgSums &sm, int &slot) {
     ff r;
-    r.hi = a + c;
-    r.lo = c - (r.hi - a);
-    if (E == 255) r.hi = r.lo = __int_as_float(0x7FC00000);  // infinity or NaN among them
+    cg_sum<1>(&t, &r, sm, slot);
     return r;
+}
+
+// complex quotient, scaled against overflow of the squares
+__device__ __forceinline__ cpx<float> cg_div(cpx<float> a, cpx<float> b) {
+    const float m = fmaxf(fabsf(b.re), fabsf(b.im)), i = 1.0f / m;
+    const float x = b.re * i, y = b.im * i, d = 1.0f / (x * x + y * y);
+    return {(a.re * x + a.im * y) * d * i, (a.im * x - a.re * y) * d * i};
 }
 
 // FP64 sum over the CTA in a fixed order
@@ -233,11 +270,32 @@ __device__ __forceinline__ float cg_norm(const Spinor<float> &x) {
     return t;
 }
 
+// x += a y, complex a
+__device__ __forceinline__ void cg_cadd(cpx<float> a, const Spinor<float> &y, Spinor<float> &x) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x.c[q][c] = cfma(a, y.c[q][c], x.c[q][c]);
+}
+
+// sum of conj(x) y
+__device__ __forceinline__ void cg_dot(const Spinor<float> &x, const Spinor<float> &y, float *t) {
+    t[0] = t[1] = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const cpx<float> a = x.c[q][c], b = y.c[q][c];
+            t[0] = fmaf(a.re, b.re, fmaf(a.im, b.im, t[0]));
+            t[1] = fmaf(a.re, b.im, fmaf(-a.im, b.re, t[1]));
+        }
+}
+
 // The whole solve of item (block rl of the launch, system k).  The hop is one
 // copy of code, used by every step of a small state machine (several inlined
 // copies overflow the instruction cache).
 template <class Args>
-__device__ void block_cg_item(const Args &a, int rl, int k, CgShared &sm) {
+__device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared &sm) {
     const Geom &g = a.g;
     const int j = threadIdx.x, r = a.rank_lo + rl;
     const long long out_i = (long long)k * a.n_ranks + rl;
@@ -248,7 +306,7 @@ __device__ void block_cg_item(const Args &a, int rl, int k, CgShared &sm) {
     double2 *x = a.x.p + k * a.x.bs - a.x.off;
     double2 *r64 = a.r64.p + k * a.r64.bs - a.r64.off;
     // FP32 vectors of the system in global memory: the even half of the inner
-    // right-hand side (full layout), then e (full layout) and rho (odd half)
+    // right-hand side (full layout), then e (full layout) and rho or rh (odd half)
     float2 *rhs_e = (float2 *)a.vin + k * a.vin_bs;
     float2 *ev = rhs_e + 12 * V, *rhov = rhs_e + 24 * V - 2 * Vh;  // (rho: odd site s at unit u Vh + s - Vh)
     bool skip = (a.sys_active && !a.sys_active[k]) || (a.block_active && !a.block_active[bi.lex]);
@@ -277,7 +335,7 @@ __device__ void block_cg_item(const Args &a, int rl, int k, CgShared &sm) {
     const float A = (float)a.A, c4 = (float)(-1.0 / (4.0 * a.A)), h2A = (float)(0.5 / a.A), iA = (float)(1.0 / a.A);
     const float delta2 = (float)(a.delta * a.delta);
     int total_it = 0, status = 0, slot = 0;
-    double rel = 0, rn = bn;
+    double rel = 0, rn = bn, rn_old = 0;
     for (int outer = 0;; ++outer) {
         // FP64 true residual r64 = b - D_b x (r64 = b on the first step)
         if (outer > 0) {
@@ -340,6 +398,8 @@ __device__ void block_cg_item(const Args &a, int rl, int k, CgShared &sm) {
         }
         // inner rhs = r64 / |r64| in FP32: even half to the exchange buffer
         // (and kept in global memory for the end), odd half in q
+        if (bicg && outer > 0 && !(rn <= 0.25 * rn_old)) bicg = false;  // no use here: CGNR from now on
+        rn_old = rn;
         Spinor<float> res, pp, q;
         for (int c = 0; c < 12; ++c) {
             const double2 v = src[c * scs + site[0]];
@@ -357,47 +417,54 @@ __device__ void block_cg_item(const Args &a, int rl, int k, CgShared &sm) {
         __syncthreads();
         ff rr = {0, 0};
         float target = 0, alpha = 0;
+        cpx<float> rho = {0, 0}, al = {0, 0};
         int it = 0;
-        // steps: 0 bhat = rhs_o + H_o(rhs_e)/(2A) (= rho, kept in q); 1, 2 res =
-        // Dhat^dag rho; 3, 4 q = Dhat p and the updates of e, rho; 5, 6
-        // Dhat^dag q and the updates of res, p; 7 e_e = (rhs_e + H_e(e)/2)/A
+        // steps: 0 bhat = rhs_o + H_o(rhs_e)/(2A) (kept in q).
+        // CGNR (rho = bhat): 1, 2 res = Dhat^dag rho; 3, 4 q = Dhat p and the
+        // updates of e, rho; 5, 6 Dhat^dag q and the updates of res, p.
+        // BiCGStab (rh = bhat, r = res, v = q): 8, 9 v = Dhat p, s = r - alpha v;
+        // 10, 11 t = Dhat s and the updates of e, r, p.
+        // 7 e_e = (rhs_e + H_e(e)/2)/A
 #pragma unroll 1
         for (int step = 0;;) {
-            const bool odd = (step & 1) == 0;  // output parity (steps 0, 2, 4, 6)
+            const bool odd = step < 8 ? (step & 1) == 0 : (step & 1) == 1;  // output parity
             const Spinor<float> acc = cg_hop(sm, odd ? st_o.nb : st_e.nb, odd ? st_o.lk[0] : st_e.lk[0],
                                              odd ? st_o.lk[1] : st_e.lk[1],
                                              step == 1 || step == 2 || step == 5 || step == 6 ? -1.0f : 1.0f);
             if (step == 0) {
                 cg_add(h2A, acc, q);
                 store_spinor<Store<float>>(rhov, Vh, site[1], q);
-                const ff bb = cg_sum(cg_norm(q), sm.sums, slot);
+                const ff bb = cg_sum1(cg_norm(q), sm.sums, slot);
                 target = bb.hi * delta2;
-                step = bb.hi > 0 ? 1 : 7;  // (a zero right-hand side: e = 0)
+                step = !(bb.hi > 0) || total_it >= a.maxit ? 7 : bicg ? 8 : 1;  // (a zero right-hand side: e = 0)
                 if (step == 7) q = res;
+                if (step == 8) {
+                    res = q;
+                    pp = q;
+                    rho = {bb.hi, 0};
+                }
                 cg_put(sm.x, j, q);
-            } else if (odd == false && step != 7) {  // 1, 3, 5: the vector on even sites
+            } else if (odd == false && step != 7) {  // 1, 3, 5, 8, 10: the vector on even sites
                 __syncthreads();
                 cg_put(sm.x, j, acc);
                 ++step;
             } else if (step == 2) {
                 res = cg_axpby(A, q, c4, acc);
                 pp = res;
-                rr = cg_sum(cg_norm(res), sm.sums, slot);
-                const bool stop = total_it >= a.maxit;
-                if (stop) zero(q);
-                cg_put(sm.x, j, stop ? q : pp);
-                step = stop ? 7 : 3;
+                rr = cg_sum1(cg_norm(res), sm.sums, slot);
+                cg_put(sm.x, j, pp);
+                step = 3;
             } else if (step == 4) {
                 q = cg_axpby(A, pp, c4, acc);
-                Spinor<float> rho = load_spinor<Store<float>>(rhov, Vh, site[1]);
+                Spinor<float> rhoc = load_spinor<Store<float>>(rhov, Vh, site[1]);
                 Spinor<float> e = load_spinor<Store<float>>(ev, V, site[1]);
-                const ff qq = cg_sum(cg_norm(q), sm.sums, slot);
+                const ff qq = cg_sum1(cg_norm(q), sm.sums, slot);
                 alpha = ff_div(rr, qq);
                 cg_add(alpha, pp, e);
-                cg_add(-alpha, q, rho);
+                cg_add(-alpha, q, rhoc);
                 store_spinor<Store<float>>(ev, V, site[1], e);
-                store_spinor<Store<float>>(rhov, Vh, site[1], rho);
-                const ff rhorho = cg_sum(cg_norm(rho), sm.sums, slot);
+                store_spinor<Store<float>>(rhov, Vh, site[1], rhoc);
+                const ff rhorho = cg_sum1(cg_norm(rhoc), sm.sums, slot);
                 ++it;
                 // converged, broken down (NaN included)
                 const bool stop = !(rhorho.hi > target) || !(qq.hi > 0);
@@ -405,7 +472,7 @@ __device__ void block_cg_item(const Args &a, int rl, int k, CgShared &sm) {
                 step = stop ? 7 : 5;
             } else if (step == 6) {
                 cg_add(-alpha, cg_axpby(A, q, c4, acc), res);
-                const ff rn2 = cg_sum(cg_norm(res), sm.sums, slot);
+                const ff rn2 = cg_sum1(cg_norm(res), sm.sums, slot);
                 const float beta = ff_div(rn2, rr);
                 rr = rn2;
                 pp = cg_axpby(beta, pp, 1.0f, res);
@@ -413,6 +480,65 @@ __device__ void block_cg_item(const Args &a, int rl, int k, CgShared &sm) {
                 if (stop) q = load_spinor<Store<float>>(ev, V, site[1]);
                 cg_put(sm.x, j, stop ? q : pp);
                 step = stop ? 7 : 3;
+            } else if (step == 9) {
+                q = cg_axpby(A, pp, c4, acc);
+                float t[2];
+                cg_dot(load_spinor<Store<float>>(rhov, Vh, site[1]), q, t);
+                ff d[2];
+                cg_sum<2>(t, d, sm.sums, slot);
+                if (!(fabsf(d[0].hi) + fabsf(d[1].hi) > 0)) {  // breakdown (NaN included): the correction so far
+                    bicg = false;
+                    q = load_spinor<Store<float>>(ev, V, site[1]);
+                    cg_put(sm.x, j, q);
+                    step = 7;
+                } else {
+                    al = cg_div(rho, {d[0].hi, d[1].hi});
+                    cg_cadd({-al.re, -al.im}, q, res);  // s
+                    cg_put(sm.x, j, res);
+                    step = 10;
+                }
+            } else if (step == 11) {
+                const Spinor<float> t = cg_axpby(A, res, c4, acc);
+                float u[7];
+                cg_dot(t, res, u);
+                u[2] = cg_norm(t);
+                const Spinor<float> rh = load_spinor<Store<float>>(rhov, Vh, site[1]);
+                cg_dot(rh, t, u + 3);
+                cg_dot(rh, res, u + 5);
+                Spinor<float> e = load_spinor<Store<float>>(ev, V, site[1]);
+                ff d[7];
+                cg_sum<7>(u, d, sm.sums, slot);
+                const float itt = d[2].hi > 0 ? 1.0f / d[2].hi : 0.0f;
+                const cpx<float> om = {d[0].hi * itt, d[1].hi * itt};
+                const cpx<float> w = cmul(om, cpx<float>{d[3].hi, d[4].hi});
+                const cpx<float> rho1 = {d[5].hi - w.re, d[6].hi - w.im};
+                const bool stalled = !(fabsf(om.re) + fabsf(om.im) > 0) || !(fabsf(rho1.re) + fabsf(rho1.im) > 0);
+                cg_cadd(al, pp, e);
+                cg_cadd(om, res, e);
+                store_spinor<Store<float>>(ev, V, site[1], e);
+                cg_cadd({-om.re, -om.im}, q, pp);    // p - omega v
+                cg_cadd({-om.re, -om.im}, t, res);   // r
+                const ff r2 = cg_sum1(cg_norm(res), sm.sums, slot);
+                ++it;
+                if (!(r2.hi > target) || stalled || total_it + it >= a.maxit) {
+                    if (!(r2.hi <= target)) bicg = false;  // stalled, NaN or out of iterations
+                    q = e;
+                    if (!(r2.hi * delta2 < target)) {  // no better than e = 0
+                        zero(q);
+                        store_spinor<Store<float>>(ev, V, site[1], q);
+                    }
+                    cg_put(sm.x, j, q);
+                    step = 7;
+                } else {
+                    const cpx<float> be = cmul(cg_div(rho1, rho), cg_div(al, om));
+                    rho = rho1;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) pp.c[b][c] = cfma(be, pp.c[b][c], res.c[b][c]);
+                    cg_put(sm.x, j, pp);
+                    step = 8;
+                }
             } else {
                 // the solution of the inner system, added to x in FP64
                 const Spinor<float> e = load_spinor<Store<float>>(ev, V, site[1]);

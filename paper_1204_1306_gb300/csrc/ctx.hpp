@@ -77,7 +77,10 @@ struct psms_ctx {
     double inner_delta = 0;       // inner relative reduction of whole-lattice solves (0: defaults)
     int shared_links = 1;         // estimators' whole-lattice FP32 solves: shared-endpoint links
     int full_solver = 1;          // inner Krylov method of whole-lattice solves: 0 CGNR, 1 BiCGStab
-    int block_krylov = 0;         // inner Krylov method of block solves: 0 CGNR, 1 BiCGStab
+    // inner Krylov method of block solves: 0 CGNR, 1 BiCGStab, -1 (not set):
+    // BiCGStab with CGNR as its fallback where the solver has one (block_cg.cuh),
+    // CGNR elsewhere
+    int block_krylov = -1;
     int outer[4] = {0, 0, 0, 0};  // outer blocks of the recursive decomposition (0: none)
     int max_chunk = 0;            // cap on systems per estimator launch (0: from the memory estimate)
     // per-block records of the last filter step (psms_filter_record); empty

@@ -74,10 +74,10 @@ static void launch_block_variant(psms_ctx *c, const BlockSolveArgs &a, int n_ran
     }
 }
 
-// one CTA per (block, system): blocks of 256 sites, FP32 inner CGNR
-__global__ void __launch_bounds__(CG_NT, 3) block_cg_kernel(const BlockSolveArgs a) {
+// one CTA per (block, system): blocks of 256 sites, FP32 inner iterations
+__global__ void __launch_bounds__(CG_NT, 3) block_cg_kernel(const BlockSolveArgs a, bool bicg) {
     extern __shared__ __align__(16) unsigned char cg_smem[];
-    block_cg_item(a, blockIdx.x, blockIdx.y, *reinterpret_cast<CgShared *>(cg_smem));
+    block_cg_item(a, blockIdx.x, blockIdx.y, bicg, *reinterpret_cast<CgShared *>(cg_smem));
 }
 
 // the solver of block_cg.cuh runs these solves
@@ -124,10 +124,10 @@ void block_solve(psms_ctx *c, const BlockSolveReq &q) {
     a.resid = q.resid;
     a.xnorm2 = q.xnorm2;
     a.status = q.status;
-    if (c->forced_block_variant < 0 && c->block_krylov == 0 && block_cg_fits(g, q.inner_prec, q.fx)) {
+    if (c->forced_block_variant < 0 && block_cg_fits(g, q.inner_prec, q.fx)) {
         block_cg_prepare();
         const int slot = c->prof ? prof_block_begin(c) : -1;
-        block_cg_kernel<<<dim3(q.n_ranks, q.n_sys), CG_NT, sizeof(CgShared), c->stream>>>(a);
+        block_cg_kernel<<<dim3(q.n_ranks, q.n_sys), CG_NT, sizeof(CgShared), c->stream>>>(a, c->block_krylov != 0);
         PSMS_LAUNCH_CHECK("block_cg_kernel");
         if (slot >= 0) prof_block_end(c, slot);
         return;
@@ -163,7 +163,8 @@ void block_solve(psms_ctx *c, const BlockSolveReq &q) {
     // the autotuner chooses among the variants of the context's Krylov
     // method only, so that every tuned choice gives the same bits
     auto method = [&](int v) { return (vars[v].hv >> 2) & 1; };
-    const long long key = ((long long)q.inner_prec << 40) | ((long long)c->block_krylov << 36) |
+    const int krylov = c->block_krylov == PSMS_SOLVER_BICGSTAB ? 1 : 0;
+    const long long key = ((long long)q.inner_prec << 40) | ((long long)krylov << 36) |
                           ((long long)g.Vbh << 8) | (q.n_sys > 1 ? 1 : 0);
     auto it = c->block_variant.find(key);
     int choice = it == c->block_variant.end() ? -1 : it->second;
@@ -174,7 +175,7 @@ void block_solve(psms_ctx *c, const BlockSolveReq &q) {
         cuda_check(cudaEventCreate(&e1), "tune event");
         float best = 1e30f;
         for (int v = 0; v < nvar; ++v) {
-            if (!admissible(v) || method(v) != c->block_krylov) continue;
+            if (!admissible(v) || method(v) != krylov) continue;
             cuda_check(cudaEventRecord(e0, c->stream), "tune record");
             launch(v);
             cuda_check(cudaEventRecord(e1, c->stream), "tune record");
@@ -189,7 +190,7 @@ void block_solve(psms_ctx *c, const BlockSolveReq &q) {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
     }
-    if (choice < 0) choice = c->block_krylov ? 15 : 0;
+    if (choice < 0) choice = krylov ? 15 : 0;
     if (c->forced_block_variant < 0) c->block_variant[key] = choice;
     const int slot = c->prof ? prof_block_begin(c) : -1;
     launch(choice);
@@ -1245,7 +1246,22 @@ struct MultiArgs {
 };
 
 // Persistent CTAs take items from an atomic counter until the list is empty;
-// no CTA waits for another.
+// no CTA waits for another.  Blocks of 256 sites of every lattice with FP32
+// inner iterations: the solver of block_cg.cuh (item.w: its BiCGStab).
+__global__ void __launch_bounds__(CG_NT, 3) block_cg_multi_kernel(const MultiArgs m) {
+    extern __shared__ __align__(16) unsigned char cg_smem[];
+    __shared__ int item;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) item = atomicAdd(m.counter, 1);
+        __syncthreads();
+        const int it = item;
+        if (it >= m.n_items) return;
+        const int4 w = m.items[it];
+        block_cg_item(m.probs[w.x], w.y, w.z, w.w != 0, *reinterpret_cast<CgShared *>(cg_smem));
+    }
+}
+
 template <class SV, class SL, int NT>
 __global__ void __launch_bounds__(NT) block_solve_multi_kernel(const MultiArgs m) {
     __shared__ double sh[NT / 32 + 1];
@@ -1289,6 +1305,7 @@ struct psms_block_plan {
     double *d_summary = nullptr;
     int n_items = 0;
     int inner = 0;
+    bool cg = false;  // every problem runs the solver of block_cg.cuh
     int ctas = 0, order = 0;
     double tuned_ms = 0;
     cudaStream_t stream = nullptr;
@@ -1309,22 +1326,23 @@ static void plan_alloc(psms_block_plan *pl, void **p, size_t bytes) {
 static std::vector<int4> make_items(const psms_block_plan *pl, int order) {
     std::vector<int4> it;
     const int np = (int)pl->probs.size();
+    auto bicg = [&](int p) { return pl->probs[p].ctx->block_krylov != 0 ? 1 : 0; };
     if (order == 0) {
         for (int p = 0; p < np; ++p)
             for (int k = 0; k < pl->probs[p].n_rhs; ++k)
-                for (int r = 0; r < pl->h_args[p].n_ranks; ++r) it.push_back(make_int4(p, r, k, 0));
+                for (int r = 0; r < pl->h_args[p].n_ranks; ++r) it.push_back(make_int4(p, r, k, bicg(p)));
     } else if (order == 1) {
         int kmax = 0;
         for (auto &q : pl->probs) kmax = std::max(kmax, q.n_rhs);
         for (int k = 0; k < kmax; ++k)
             for (int p = 0; p < np; ++p)
                 if (k < pl->probs[p].n_rhs)
-                    for (int r = 0; r < pl->h_args[p].n_ranks; ++r) it.push_back(make_int4(p, r, k, 0));
+                    for (int r = 0; r < pl->h_args[p].n_ranks; ++r) it.push_back(make_int4(p, r, k, bicg(p)));
     } else {
         std::vector<std::vector<int4>> per(np);
         for (int p = 0; p < np; ++p)
             for (int k = 0; k < pl->probs[p].n_rhs; ++k)
-                for (int r = 0; r < pl->h_args[p].n_ranks; ++r) per[p].push_back(make_int4(p, r, k, 0));
+                for (int r = 0; r < pl->h_args[p].n_ranks; ++r) per[p].push_back(make_int4(p, r, k, bicg(p)));
         size_t mx = 0;
         for (auto &v : per) mx = std::max(mx, v.size());
         for (size_t i = 0; i < mx; ++i)
@@ -1338,7 +1356,9 @@ static void plan_launch(psms_block_plan *pl, cudaStream_t s, int ctas) {
     MultiArgs m{pl->d_args, pl->d_items, pl->n_items, pl->d_counter};
     cuda_check(cudaMemsetAsync(pl->d_counter, 0, sizeof(int), s), "plan counter");
     const int NT = 128;
-    if (pl->inner == P64)
+    if (pl->cg)
+        block_cg_multi_kernel<<<ctas, CG_NT, sizeof(CgShared), s>>>(m);
+    else if (pl->inner == P64)
         block_solve_multi_kernel<Store<double>, Store<double>, NT><<<ctas, NT, 0, s>>>(m);
     else
         block_solve_multi_kernel<Store<float>, Store<float>, NT><<<ctas, NT, 0, s>>>(m);
@@ -1422,6 +1442,13 @@ psms_status psms_block_plan_create(const psms_block_problem *probs, int n_probs,
             pl->n_per.push_back(n_out);
             pl->n_items += n_out;
         }
+        pl->cg = true;
+        for (int p = 0; p < n_probs; ++p)
+            pl->cg = pl->cg && block_cg_fits(probs[p].ctx->g, inner_prec, pl->h_args[p].fx);
+        if (pl->cg)
+            cuda_check(cudaFuncSetAttribute(block_cg_multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)sizeof(CgShared)),
+                       "block solver shared memory");
         plan_alloc(pl, (void **)&pl->d_args, sizeof(BlockSolveArgs) * n_probs);
         plan_alloc(pl, (void **)&pl->d_nper, sizeof(int) * n_probs);
         plan_alloc(pl, (void **)&pl->d_items, sizeof(int4) * pl->n_items);
