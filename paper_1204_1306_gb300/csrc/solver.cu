@@ -842,7 +842,7 @@ static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long lo
         h.dot = HopDot{};
     };
     int it = 0;
-    int chunk = 8;
+    const int chunk = 4;  // iterations between host checks: an iteration launched too many costs more than a check
     std::vector<int> hflags(n_sys), hmap;
     h.active = flags;
     // systems still iterating, refreshed at every host check: later launches
@@ -895,7 +895,6 @@ static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long lo
             map = d_map;
         }
         n_act = (int)hmap.size();
-        chunk = std::min(chunk * 2, 64);
     }
     h.sys_map = nullptr;
     h.n_map = 0;
