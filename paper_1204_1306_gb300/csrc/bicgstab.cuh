@@ -5,6 +5,8 @@
 // kernels of the solver and by Wilson hops that fuse their dot products.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace psms {
@@ -80,6 +82,44 @@ __device__ __forceinline__ double wsum(const double *v) {
     for (; o > 0; o >>= 1) r[0] += __shfl_xor_sync(0xffffffffu, r[0], o);
     return r[0];
 }
+// The same of FP32 numbers, without the FP64 pipe: signed mantissas on the
+// largest exponent of the warp's numbers (57 bits below it), summed as 64-bit
+// integers, so the error is below that of FP64 sums.
+template <int P>
+__device__ __forceinline__ double wsum(const float *v) {
+    const int l = threadIdx.x & 31;
+    int64_t r[P];
+    unsigned em[P], top = 0;
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        const unsigned b = __float_as_uint(v[i]), e = (b >> 23) & 255u;
+        em[i] = max(__reduce_max_sync(0xffffffffu, e), 1u);
+        top = max(top, em[i]);
+        const unsigned m = (b & 0x7FFFFFu) | (e ? 0x800000u : 0u), sh = em[i] - max(e, 1u);
+        const int64_t x = (int64_t)(((uint64_t)m << 33) >> min(sh, 63u));
+        r[i] = (int)b < 0 ? -x : x;
+    }
+    if (top == 255u) {  // infinity or NaN
+        double d[P];
+#pragma unroll
+        for (int i = 0; i < P; ++i) d[i] = (double)v[i];
+        return wsum<P>(d);
+    }
+    int o = 16;
+#pragma unroll
+    for (int m = P; m > 1; m >>= 1, o >>= 1) {
+        const bool up = l & o;
+#pragma unroll
+        for (int i = 0; i < m / 2; ++i) {
+            const int64_t keep = up ? r[i + m / 2] : r[i], give = up ? r[i] : r[i + m / 2];
+            r[i] = keep + __shfl_xor_sync(0xffffffffu, (long long)give, o);
+            em[i] = up ? em[i + m / 2] : em[i];
+        }
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) r[0] += __shfl_xor_sync(0xffffffffu, (long long)r[0], o);
+    return (double)r[0] * __hiloint2double((int)(em[0] + 1023u - 183u) << 20, 0);  // 2^(em - 127 - 23 - 33)
+}
 template <int P>
 __device__ __forceinline__ int wsum_index(int l) {  // the leading bits of the lane number
     return P == 1 ? 0 : P == 2 ? l >> 4 : P == 4 ? l >> 3 : l >> 2;
@@ -90,8 +130,8 @@ __device__ __forceinline__ int wsum_index(int l) {  // the leading bits of the l
 // order and applies the scalar stage, so the result does not depend on
 // which CTA finishes last.  part: BCG_SUMS arrays of part_n doubles; the sums
 // [LO, HI) are taken.  Ends at a barrier.
-template <int NT, int LO, int HI>
-__device__ __forceinline__ void bcg_partials_and_stage(BCS *st, const double in[BCG_SUMS], double *part,
+template <int NT, int LO, int HI, class T>
+__device__ __forceinline__ void bcg_partials_and_stage(BCS *st, const T in[BCG_SUMS], double *part,
                                                        long long part_n, unsigned int *counters, int stage, int maxit,
                                                        int *flags, double (*sh)[NT / 32], int k, int cta, int nct) {
     const long long slot = (long long)k * nct + cta;
@@ -99,10 +139,10 @@ __device__ __forceinline__ void bcg_partials_and_stage(BCS *st, const double in[
     constexpr int N = HI - LO, P = N > 4 ? 8 : N > 2 ? 4 : N;
     const int l = threadIdx.x & 31, wi = wsum_index<P>(l);
     const bool lead = l == wi * (32 / P) && wi < N;
-    auto warp_sums = [&](const double *v) {
-        double x[P];
+    auto warp_sums = [&](const auto *v) {
+        std::decay_t<decltype(*v)> x[P];
 #pragma unroll
-        for (int a = 0; a < P; ++a) x[a] = a < N ? v[LO + a] : 0.0;
+        for (int a = 0; a < P; ++a) x[a] = a < N ? v[LO + a] : 0;
         const double t = wsum<P>(x);
         if (lead) sh[LO + wi][threadIdx.x >> 5] = t;
     };

@@ -80,7 +80,10 @@ __global__ void __launch_bounds__(CG_NT, 3) block_cg_kernel(const BlockSolveArgs
     block_cg_item(a, blockIdx.x, blockIdx.y, bicg, *reinterpret_cast<CgShared *>(cg_smem));
 }
 
-// the solver of block_cg.cuh runs these solves
+// The solver of block_cg.cuh runs these solves: one CTA holds 128 sites of each
+// parity, two to three times faster than the general kernel at any number of
+// blocks (block_cg.cuh); other sizes, FP64 inner iterations and solves without
+// fixed-point links have the general one.
 static bool block_cg_fits(const Geom &g, int inner_prec, const int4 *fx) {
     return inner_prec == P32 && g.Vbh == CG_NT && fx;
 }
@@ -635,7 +638,7 @@ __global__ void __launch_bounds__(NT) bcg_dot_stage_kernel(BCS *st, View<typenam
     __shared__ double sh[BCG_SUMS][NT / 32];
     const int k = map ? map[blockIdx.y] : (int)blockIdx.y;
     if (!st[k].active) return;
-    double sum[BCG_SUMS] = {};
+    R sum[BCG_SUMS] = {};
     const long long i = (long long)blockIdx.x * NT + threadIdx.x;
     if (i < n && (!rank_active || rank_active[(int)(i >> vbh_sh)])) {
         const long long sx = s_lo + i;
@@ -663,16 +666,16 @@ __global__ void __launch_bounds__(NT) bcg_dot_stage_kernel(BCS *st, View<typenam
                     zr += h.re * y.re + h.im * y.im;
                     zi += h.re * y.im - h.im * y.re;
                 }
-            sum[0] = (double)yr;
-            sum[1] = (double)yi;
-            sum[2] = (double)aa;
-            sum[3] = (double)xr;
-            sum[4] = (double)xi;
-            sum[5] = (double)zr;
-            sum[6] = (double)zi;
+            sum[0] = yr;
+            sum[1] = yi;
+            sum[2] = aa;
+            sum[3] = xr;
+            sum[4] = xi;
+            sum[5] = zr;
+            sum[6] = zi;
         } else {
-            sum[0] = (double)xr;
-            sum[1] = (double)xi;
+            sum[0] = xr;
+            sum[1] = xi;
         }
     }
     bcg_partials_and_stage<NT, 0, BCG_SUMS>(st, sum, part, part_n, counters, stage, maxit, flags, sh, k,
@@ -681,9 +684,9 @@ __global__ void __launch_bounds__(NT) bcg_dot_stage_kernel(BCS *st, View<typenam
 
 // x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), then
 // |r|^2 and stage 2.  Eight passes over memory bound it; a thread takes its
-// site unit by unit, which keeps it at few registers and the SMs full (whole
-// spinors at once: 12 % occupancy and 60 us for 12 systems at 16^4), with one
-// FP64 reduction per site (one per unit: 71 us).
+// site unit by unit, which keeps it at few registers and the SMs full (42 us for
+// 12 systems at 16^4, 7.2 TB/s, part of it from L2; whole spinors at once: 12 %
+// occupancy and 60 us), with one reduction per site (one per unit: 71 us).
 template <class S, int NT>
 __global__ void __launch_bounds__(NT) bcg_update_stage_kernel(BCS *st, View<typename S::elem> x,
                                                               View<typename S::elem> p, View<typename S::elem> r,
@@ -697,7 +700,7 @@ __global__ void __launch_bounds__(NT) bcg_update_stage_kernel(BCS *st, View<type
     __shared__ double sh[BCG_SUMS][NT / 32];
     const int k = map ? map[blockIdx.y] : (int)blockIdx.y;
     if (!st[k].active) return;
-    double sum[BCG_SUMS] = {};
+    R sum[BCG_SUMS] = {};
     const long long i = (long long)blockIdx.x * NT + threadIdx.x;
     if (i < n && (!rank_active || rank_active[(int)(i >> vbh_sh)])) {
         const double2 a = st[k].alpha, o = st[k].omega, b = st[k].beta;
@@ -725,7 +728,7 @@ __global__ void __launch_bounds__(NT) bcg_update_stage_kernel(BCS *st, View<type
             store_unit<S>(at(r), sv);
             store_unit<S>(at(p), pv);
         }
-        sum[2] = (double)aa;
+        sum[2] = aa;
     }
     bcg_partials_and_stage<NT, 2, 3>(st, sum, part, part_n, counters, 2, maxit, flags, sh, k, (int)blockIdx.x,
                                      (int)gridDim.x);
