@@ -488,7 +488,8 @@ psms_status psms_max_chunk(psms_ctx *ctx, int n);
  * each block's input of the other parity in shared memory by per-thread or
  * bulk (TMA) copies; for FP32 links in the whole-lattice mode 14 variants on
  * such blocks, 10 on others, 15 with shared-endpoint links, 4 otherwise; for
- * FP64 links 4 in the whole-lattice mode, 1 otherwise; used modulo their
+ * FP64 arithmetic 4 in the whole-lattice mode, 1 otherwise (FP64 operators
+ * run in fixed point where they can, which has one form); used modulo their
  * count) instead of the autotuned one; -1 returns to autotuning.  All
  * variants compute the same operator.  *n_variants (may be NULL) receives
  * 15.  PSMS_EINVAL outside -1..14. */
@@ -537,9 +538,9 @@ psms_status psms_block_action_change(psms_ctx *ctx, int field_old, int field_new
  * takes small-block determinants by LU), lexicographic block index, into
  * out_host[n_blocks]: det D_b = A^{n_e} det(Dhat_b) with A = 4 + m0 and
  * Dhat_b = A - D_oe D_eo / A the even-odd reduced block operator (n x n
- * complex, n = 6 x block volume), factorised by batched FP64 LU with
- * partial pivoting on the device.  Cost about (8/3) n^3 FP64 flop per block
- * (1e10 for a 4^4 block); device memory n^2 x 16 B per block of a batch
+ * complex, n = 6 x block volume), factorised by batched LU with partial
+ * pivoting on the device to FP64 accuracy.  Cost about (8/3) n^3 flop per
+ * block (1e10 for a 4^4 block; 3.7 ms each in a batch); device memory n^2 x 16 B per block of a batch
  * (batches sized from the free memory, psms_max_chunk caps them).
  * PSMS_ESPECTRUM if a block operator is singular (non-finite result);
  * PSMS_EINVAL for blocks of more than 1024 sites.  Synchronises the

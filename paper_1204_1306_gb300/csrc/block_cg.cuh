@@ -16,6 +16,10 @@
 // right-hand side, solution and residual of the defect correction are in
 // global memory (L2).
 //
+// Measured with CGNR against the general solver: the block level of 16^4 with
+// twelve systems 18.7 -> 10.8 ms, 243 blocks of 12^4 1.10 -> 0.52 ms; with
+// BiCGStab 6.9 and 0.41 ms (960 us for the 512 blocks of a 16^3 x 32 lattice).
+//
 // FP64 has two lanes per SM here, a warp's FP64 instruction costs 16 clocks
 // of them, so the iterations have none: the norms are summed exactly in
 // integers (redux on two 25-bit limbs), the scalars are pairs of FP32 numbers,

@@ -353,7 +353,9 @@ __global__ void __launch_bounds__(64) lu_solve_kernel(double2 *Mall, int n, int 
 // HI = sum hi hi <= 2^62, MID = sum (hi lo + lo hi) < 2^63 exact in 64 bits
 // for w <= 32.  One conversion and one FP64 multiply-add per real number
 // remain.  12 integer instead of 4 FP64 instructions per complex multiply-add,
-// at 32 times the rate.
+// at 32 times the rate.  16 blocks of 4^4: 135 -> 42 ms of updates (the whole
+// determinant 181 -> 58 ms) with 256 threads of 4 x 2 outputs; 128 threads of
+// 4 x 4 take 82 ms in all, panels of 32 columns 73.
 struct LuLimbs {
     int hi, lo;
 };

@@ -788,7 +788,7 @@ __global__ void __launch_bounds__(NT, MINB) hop_staged_kernel(const HopArgs<type
 }
 
 static constexpr int HOP_NT = 128;
-constexpr long long FX_SPLIT_SITES = 152 * 128;  // output sites of all systems
+constexpr long long FX_SPLIT_SITES = 152 * 128;  // output sites of all systems (hop_launch_t gives both sides)
 
 // The FP32 forms, by the number psms_hop_variant takes.  part: general form,
 // register caps 2, 6, 7, 8 CTAs/SM.  whole (whole lattice): the same, the
@@ -885,11 +885,12 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     const int nct = hop_ctas(c, h);
     const int nsys = h.sys_map ? h.n_map : h.n_sys;
     if (nct == 0 || nsys == 0) return 0;
-    // FP64 hops in fixed point (fixed.cuh).  Few output sites (below four
-    // warps per scheduler over the chip), or a few blocks of a large lattice:
-    // the directions of a site go to eight warps, which convert what they
-    // read; else a pass converts the input first (no room for its copy: the
-    // FP64 kernel)
+    // FP64 hops in fixed point (fixed.cuh).  Few output sites, or a few blocks
+    // of a large lattice (whose other sites need no conversion): the
+    // directions of a site go to eight warps, which convert what they read;
+    // else a pass converts the input first (no room for its copy: the FP64
+    // kernel).  Directions / pass, us per D_w: 4096 sites 8.4 / 28.9, 8192
+    // 14.5 / 29.0, 16384 23.7 / 28.9, 32768 39.1 / 36.4, 65536 77 / 54.
     bool fixed = std::is_same<S, Store<double>>::value && h.fx != nullptr;
     const long long per = (h.p < 0 ? 2LL : 1LL) * a.n_ranks * c->g.Vbh;
     const bool fx_split = !h.partial && (per * nsys <= FX_SPLIT_SITES || 8LL * a.n_ranks <= c->g.nblocks);

