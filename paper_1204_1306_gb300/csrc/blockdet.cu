@@ -11,7 +11,8 @@
 //      hops to a unit vector and scatters the result; column-major storage);
 //   2. LU with partial pivoting, right-looking (below);
 //   3. ln|det D_b| = n_e ln A + sum_j ln|u_jj|, summed in a fixed order.
-// FP64 accuracy throughout: the level built on it is exact, and its Delta is
+// FP64 accuracy throughout (the update in integers, errors no larger than those
+// of FP64 chains on such factors): the level built on it is exact, and its Delta is
 // compared across devices.
 #include <cmath>
 #include <string>
@@ -346,28 +347,13 @@ __global__ void __launch_bounds__(64) lu_solve_kernel(double2 *Mall, int n, int 
 //
 // In FP64 this update ran at the rate of the two FP64 lanes per SM (1.1
 // TFLOP/s, 75 % of the time of a determinant).  Here the products are
-// integer multiply-adds (fixed.cuh gives the rates): rows of L21 and columns
-// of U12 become two 28-bit limbs on the exponent of their largest number (56
-// bits: exact down to 2^-3 of it, the rest to 2^-56), and
-//     sum l u = HI 2^56 + MID 2^28 (+ sum lo lo, below 2^-50 of the smallest bit kept of HI, dropped),
-// HI = sum hi hi <= 2^62, MID = sum (hi lo + lo hi) < 2^63 exact in 64 bits
-// for w <= 32.  One conversion and one FP64 multiply-add per real number
-// remain.  12 integer instead of 4 FP64 instructions per complex multiply-add,
-// at 32 times the rate.  16 blocks of 4^4: 135 -> 42 ms of updates (the whole
-// determinant 181 -> 58 ms) with 256 threads of 4 x 2 outputs; 128 threads of
-// 4 x 4 take 82 ms in all, panels of 32 columns 73.
-struct LuLimbs {
-    int hi, lo;
-};
-
-__device__ __forceinline__ LuLimbs lu_limbs(double v, int E) {
-    LuLimbs l;
-    const int64_t x = E == 0 ? 0 : fx_convert<54>(f64_bits(v), E);
-    l.hi = (int)(x >> 28);
-    l.lo = (int)((uint32_t)x & 0xFFFFFFFu);
-    return l;
-}
-
+// integer multiply-adds (fixed.cuh gives the rates) of the two limbs that
+// lu_limbs makes of the rows of L21 and the columns of U12, and one conversion
+// and one FP64 multiply-add per real number remain.  12 integer instead of 4
+// FP64 instructions per complex multiply-add, at 32 times the rate.  16 blocks
+// of 4^4: 135 -> 42 ms of updates (the whole determinant 181 -> 58 ms) with
+// 256 threads of 4 x 2 outputs; 128 threads of 4 x 4 take 82 ms in all, panels
+// of 32 columns 73.
 struct LuShared {
     int4 L[kNb][kTileR];  // limbs (re hi, re lo, im hi, im lo) of L21 rows
     int4 U[kNb][kTileC];
@@ -432,7 +418,7 @@ __global__ void __launch_bounds__(kUpdNT) lu_update_kernel(double2 *Mall, int n,
         for (int a = 0; a < NA; ++a) l[a] = Ls[q][tr + 16 * a];
 #pragma unroll
         for (int b = 0; b < NB; ++b) u[b] = Us[q][tc + CB * b];
-        // product by product over the sixteen outputs, so that consecutive
+        // product by product over the thread's outputs, so that consecutive
         // multiply-adds do not wait for each other
 #define LU_MADS(ACC, X, Y)                                    \
     _Pragma("unroll") for (int a = 0; a < NA; ++a)            \
@@ -467,8 +453,8 @@ __global__ void __launch_bounds__(kUpdNT) lu_update_kernel(double2 *Mall, int n,
             // sum = t 2^(el + eu - 2046 - 54); non-finite numbers poison it
             double f = (el == 0x7FF || eu == 0x7FF) ? nan("") : lu_scale(el + eu - 2100);
             double2 v = col[i];
-            v.x = fma(-f, (double)(hr[a][b] + (mr[a][b] >> 28)), v.x);
-            v.y = fma(-f, (double)(hi[a][b] + (mi[a][b] >> 28)), v.y);
+            v.x = fma(-f, (double)lu_join(hr[a][b], mr[a][b]), v.x);
+            v.y = fma(-f, (double)lu_join(hi[a][b], mi[a][b]), v.y);
             col[i] = v;
         }
     }
@@ -532,7 +518,7 @@ void block_logdet(psms_ctx *c, const double2 *U, double *d_out) {
             lu_update_kernel<<<grid, kUpdNT, sizeof(LuShared), c->stream>>>(M, n, k, w, c0, c1);
             PSMS_LAUNCH_CHECK("blockdet update");
         };
-        // n = 12 Vbh is a multiple of kNb = 32 (blocks have at least 16 sites)
+        // n = 12 Vbh is a multiple of kNb = 16 (blocks have at least 16 sites)
         for (int k = 0; k < n; k += kNb) {
             const int end = k + kNb;
             for (int j = k; j < end; j += kSub) {

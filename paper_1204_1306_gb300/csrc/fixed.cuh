@@ -400,6 +400,35 @@ __host__ __device__ __forceinline__ void fx_hop(int d, bool neg, const int2 hl[2
     else fx_reconstruct<DAG, false>(d >> 1, w, acc);
 }
 
+// Products of the blocked LU's trailing update (blockdet.cu): each row of L21
+// and each column of U12 is held as x 2^(E - 1078), |x| < 2^56, on the exponent
+// E (biased) of its largest real number (exact for the numbers down to 2^-3
+// of it, smaller ones and denormals are cut off at 2^-55 of 2^(E - 1023)), in
+// two limbs
+//     x = hi 2^28 + lo,  |hi| <= 2^28, -2^27 <= lo < 2^27,
+// so that, with w <= 16 complex products,
+//     sum x y = HI 2^56 + MID 2^28 + sum lo lo,
+// HI = sum hi hi <= 2^61 and MID = sum (hi lo + lo hi) <= 2^61 exact in 64
+// bits.  The last sum is dropped: at most 8 units of HI, in the root mean
+// square half a unit and of no sign (lo is rounded, not cut off: with lo in 0
+// .. 2^28 the imaginary part, whose products all add, was short by 8 units in
+// the mean).  The error of a sum is below that of the FP64 chain
+// (tests/test_fixed_point_host.py).
+struct LuLimbs {
+    int hi, lo;
+};
+
+__host__ __device__ __forceinline__ LuLimbs lu_limbs(double v, int E) {
+    LuLimbs l;
+    const int64_t x = E == 0 ? 0 : fx_convert<54>(f64_bits(v), E);
+    l.hi = (int)((x + (1 << 27)) >> 28);
+    l.lo = (int)(x - ((int64_t)l.hi << 28));
+    return l;
+}
+
+// HI + MID 2^-28, rounded: the sum in units of 2^56
+__host__ __device__ __forceinline__ int64_t lu_join(int64_t hi, int64_t mid) { return hi + ((mid + (1 << 27)) >> 28); }
+
 // Factor that turns the integers of a finished sum into b times its value;
 // false when it is out of the normal range.
 __host__ __device__ __forceinline__ bool fx_factor(const FxAcc &acc, double b, double &f) {

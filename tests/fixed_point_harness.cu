@@ -1,6 +1,9 @@
 // Test harness: the fixed-point hops of csrc/fixed.cuh, compiled for the host
 // and driven with the eight hops of a site.  Not part of the
 // library.
+#include <algorithm>
+#include <cmath>
+
 #include "../paper_1204_1306_gb300/csrc/fixed.cuh"
 
 using namespace psms;
@@ -66,4 +69,25 @@ extern "C" int fx_link_host(const double *u, double *out) {
         out[2 * k + 1] = fx_value(w[k].z, w[k].w, ue);
     }
     return ue;
+}
+
+// one element of the LU's trailing update: w complex products of a row l (on
+// its largest exponent) and a column u; out = the value subtracted
+extern "C" void lu_sum_host(const double *l, const double *u, int w, double *out) {
+    int el = 0, eu = 0;
+    for (int q = 0; q < 2 * w; ++q) {
+        el = std::max(el, (int)(f64_bits(l[q]) >> 52) & 0x7FF);
+        eu = std::max(eu, (int)(f64_bits(u[q]) >> 52) & 0x7FF);
+    }
+    int64_t hr = 0, hi = 0, mr = 0, mi = 0;
+    for (int q = 0; q < w; ++q) {
+        const LuLimbs a = lu_limbs(l[2 * q], el), b = lu_limbs(l[2 * q + 1], el), c = lu_limbs(u[2 * q], eu),
+                      d = lu_limbs(u[2 * q + 1], eu);
+        fx_mad(hr, a.hi, c.hi), fx_mad(hr, -b.hi, d.hi);
+        fx_mad(hi, a.hi, d.hi), fx_mad(hi, b.hi, c.hi);
+        fx_mad(mr, a.hi, c.lo), fx_mad(mr, a.lo, c.hi), fx_mad(mr, -b.hi, d.lo), fx_mad(mr, -b.lo, d.hi);
+        fx_mad(mi, a.hi, d.lo), fx_mad(mi, a.lo, d.hi), fx_mad(mi, b.hi, c.lo), fx_mad(mi, b.lo, c.hi);
+    }
+    out[0] = std::ldexp((double)lu_join(hr, mr), el + eu - 2100);
+    out[1] = std::ldexp((double)lu_join(hi, mi), el + eu - 2100);
 }

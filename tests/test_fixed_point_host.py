@@ -12,7 +12,7 @@ from fractions import Fraction
 import numpy as np
 import pytest
 
-from oracle import gauge
+from oracle import dirac, gauge
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 T = np.array([-1, 1] * 4, dtype=np.int32)  # D: t = -1 forward, +1 backward
@@ -198,3 +198,71 @@ def test_range_and_scaling(lib):
     w[w != 1e-290] = 0  # out of range: kept as it is
     assert lib.fx_link_host(w.ctypes.data_as(ctypes.c_void_p), out.ctypes.data_as(ctypes.c_void_p)) == 0xFFFF
     assert np.array_equal(out, w)
+
+
+def _lu_rows(kind, n, w, seed):
+    g = np.random.default_rng(seed)
+    l = g.standard_normal((n, w)) + 1j * g.standard_normal((n, w))
+    u = g.standard_normal((n, w)) + 1j * g.standard_normal((n, w))
+    if kind == "multipliers":  # rows of L21 after partial pivoting
+        l = l / np.maximum(1.0, np.abs(l))
+    elif kind == "graded":  # large multipliers meet small entries, over three decades
+        s = 10.0 ** g.uniform(-3, 0, (n, w))
+        l, u = l * s, u / s * 10.0 ** g.uniform(-3, 0, (n, w))
+    elif kind == "positive":  # no cancellation, all errors of one sign would add up
+        l, u = np.abs(l.real) + 1j * np.abs(l.imag), np.abs(u.real) + 1j * np.abs(u.imag)
+    elif kind == "largest":
+        x = 2.0 - 2.0 ** -52
+        l, u = l * 0 + x * (1 - 1j), u * 0 + x * (1 - 1j)
+        u[n // 2:] = x * (1 + 1j)
+    elif kind == "factors":  # rows and columns of the LU of an even-odd reduced block operator
+        scipy_linalg = pytest.importorskip("scipy.linalg")
+        block, kappa = (4, 4, 2, 2), 0.156
+        A = 1.0 / (2.0 * kappa)
+        U = gauge.generate_links(block, 0.5, seed)
+        M = dirac.dense_matrix(lambda v: dirac.apply_D_open(U, v, kappa), 64, block + (4, 3))
+        odd = np.repeat((np.indices(block).sum(0) % 2).reshape(-1), 12) == 1
+        S = A * np.eye(384) - M[np.ix_(odd, ~odd)] @ M[np.ix_(~odd, odd)] / A
+        _, L, R = scipy_linalg.lu(S)
+        for k in range(n):
+            p = w * int(g.integers(0, 384 // w - 1))
+            i, j = (int(v) for v in g.integers(p + w, 384, 2))
+            l[k], u[k] = L[i, p:p + w], R[p:p + w, j]
+    return l, u
+
+
+@pytest.mark.parametrize("kind", ["gauss", "multipliers", "positive", "largest", "factors", "graded"])
+@pytest.mark.parametrize("w", [8, 16])
+def test_lu_update_error_is_no_larger_than_in_fp64(lib, kind, w):
+    """The sums of the LU's trailing update against exact ones: rms error at most
+    that of a chain of FP64 multiply-adds, and no bias.  Where a row and its
+    column are graded against each other, only relative to the product of their
+    largest numbers (a common exponent each)."""
+    n = 200
+    l, u = _lu_rows(kind, n, w, 3)
+    e_fx, e_64, ulp = np.zeros((n, 2)), np.zeros((n, 2)), np.zeros((n, 2))
+    for i in range(n):
+        o = np.zeros(2)
+        a, b = np.ascontiguousarray(l[i]), np.ascontiguousarray(u[i])
+        lib.lu_sum_host(a.ctypes.data_as(ctypes.c_void_p), b.ctypes.data_as(ctypes.c_void_p), w,
+                        o.ctypes.data_as(ctypes.c_void_p))
+        exact, chain = [Fraction(0), Fraction(0)], [0.0, 0.0]
+        for p, q in zip(l[i], u[i]):
+            x, y, z, t = (Fraction(float(v)) for v in (p.real, p.imag, q.real, q.imag))
+            for k, m in ((0, x * z), (0, -y * t), (1, x * t), (1, y * z)):
+                exact[k] += m
+                chain[k] = float(Fraction(chain[k]) + m)  # one rounding, as a fused multiply-add
+        scale = Fraction(float(np.abs(l[i]).max() * np.abs(u[i]).max())) or 1  # (a zero row)
+        for k in range(2):
+            e_fx[i, k] = float((Fraction(float(o[k])) - exact[k]) / scale)
+            e_64[i, k] = float((Fraction(chain[k]) - exact[k]) / scale)
+            ulp[i, k] = abs(float(exact[k] / scale)) * 2.0 ** -53  # rounding of the result itself
+    rms = np.sqrt((e_fx ** 2).mean())
+    if kind == "graded":
+        # 4 w numbers cut off by less than 2^-55 of 2^E, times one of at most 2 2^E; 8 + 1/2 units of 2^-54 dropped
+        assert np.abs(e_fx).max() <= (8 * w + 17) * 2.0 ** -55
+        return
+    assert rms <= np.sqrt(np.maximum((e_64 ** 2).mean(), (ulp ** 2).mean()))
+    # the mean of n errors of no sign stays within four of its own standard deviations
+    if kind != "largest":
+        assert np.abs(e_fx.mean(0)).max() <= 4 * rms / np.sqrt(n)
