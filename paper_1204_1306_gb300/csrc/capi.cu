@@ -91,11 +91,15 @@ void fx_mark(psms_ctx *c) {
     c->fx_stream = c->stream;
 }
 
-const int4 *links_fx(psms_ctx *c, int f) {
-    check_field(c, f);
+bool capturing(psms_ctx *c) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cuda_check(cudaStreamIsCapturing(c->stream, &cap), "capture status");
-    if (cap != cudaStreamCaptureStatusNone) return nullptr;
+    return cap != cudaStreamCaptureStatusNone;
+}
+
+const int4 *links_fx(psms_ctx *c, int f) {
+    check_field(c, f);
+    if (capturing(c)) return nullptr;
     if (!c->Ufx[f] && cudaMalloc(&c->Ufx[f], sizeof(int4) * (size_t)fx_field(c->g.V)) != cudaSuccess) {
         cudaGetLastError();
         c->Ufx[f] = nullptr;

@@ -110,6 +110,9 @@ void *scratch(psms_ctx *c, const std::string &name, size_t bytes);
 void *scratch_try(psms_ctx *c, const std::string &name, size_t bytes);
 // FP32 copy of a gauge slot (converted on first use after a change)
 float2 *links32(psms_ctx *c, int field);
+// whether the context's stream is being captured: no timing, no conversion
+// that a later call would rely on
+bool capturing(psms_ctx *c);
 // fixed-point copy of a gauge slot, made on first use after a change; null
 // when there is no memory for it, or while the stream is captured (a graph
 // has to read the slot itself, which may change before the graph runs):

@@ -981,8 +981,8 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     }
     int &choice = c->hop_variant[h.prec][h.p < 0 ? 1 : 0][all ? 1 : 0][shared_links ? 1 : 0];
     // (launches with a fused reduction are not used for tuning: they advance
-    // the solver's scalars)
-    if (choice < 0 && c->autotune && nvar > 1 && slot < 0 && c->forced_hop_variant < 0 && !a.dot) {
+    // the solver's scalars; nor are captured ones, which cannot be timed)
+    if (choice < 0 && c->autotune && nvar > 1 && slot < 0 && c->forced_hop_variant < 0 && !a.dot && !capturing(c)) {
         cudaEvent_t e0, e1;
         cuda_check(cudaEventCreate(&e0), "tune event");
         cuda_check(cudaEventCreate(&e1), "tune event");

@@ -52,6 +52,41 @@ def test_fixed_point_hops_against_the_fp64_form(dims, block, op):
     assert float((a - b).abs().max() / b.abs().max()) < 64 * 2.0 ** -53
 
 
+@pytest.mark.parametrize("prec,tol,warm", [(ps.PREC_F64, 64 * 2.0 ** -53, True), (ps.PREC_F64, 64 * 2.0 ** -53, False),
+                                           (ps.PREC_F32, 0.0, True), (ps.PREC_BF16, 0.0, True)])
+def test_capture_with_the_default_settings(prec, tol, warm):
+    """An operator call is captured with autotuning on, after a warm-up call and
+    without one (FP64: the captured call runs another form than the warm-up; the
+    other precisions allocate their links in the warm-up)."""
+    dims = (8, 8, 8, 8)
+    ctx, _ = _ctx(dims, (4, 4, 4, 4))
+    nat = native(ctx, seeded.spinor(dims, 9), prec)
+    typ = {ps.PREC_F64: torch.float64, ps.PREC_F32: torch.float32, ps.PREC_BF16: torch.bfloat16}[prec]
+    out = torch.zeros_like(nat)
+
+    def call():
+        ps.psms_dw_apply(ctx, 0, ps.OP_FULL, nat, out, prec)
+
+    if warm:
+        call()
+        torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    ps.psms_set_stream(ctx, s)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        call()
+    ps.psms_set_stream(ctx, None)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    got = out.view(typ).double()
+    call()
+    torch.cuda.synchronize()
+    ref = out.view(typ).double()
+    assert float(ref.abs().max()) > 0.1
+    assert float((got - ref).abs().max()) <= tol * float(ref.abs().max())
+
+
 def test_hops_alternating_between_streams():
     dims = (16, 16, 16, 16)  # the form that keeps the input in scratch
     ctx, _ = _ctx(dims, (4, 4, 4, 4))
