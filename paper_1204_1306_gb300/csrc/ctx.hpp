@@ -37,6 +37,12 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
+// sites of the links that a sweep updates (gauge.cu: active_list)
+struct ActiveList {
+    const int *d = nullptr;  // device (context scratch), the eight lists back to back
+    int off[4][2], n[4][2];
+};
+
 }  // namespace psms
 
 struct psms_ctx {
@@ -55,6 +61,7 @@ struct psms_ctx {
     cudaStream_t fx_stream = nullptr;
     std::vector<psms::BlockInfo> h_binfo;
     psms::BlockInfo *d_binfo = nullptr;
+    psms::ActiveList active[2];  // of the blocks, of all links
     void *d_gauss = nullptr;  // tables of the noise (gauss.cuh)
     cudaStream_t stream = nullptr;
     std::string err;

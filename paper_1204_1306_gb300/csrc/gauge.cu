@@ -407,15 +407,13 @@ __global__ void __launch_bounds__(128) reunit_active_kernel(Geom g, double2 *U, 
 }
 
 // Active sites of every (mu, parity): indices within a block's half, block
-// after block alike.  Built once per context and active set.
-struct ActiveList {
-    const int *d = nullptr;  // device, the eight lists back to back
-    int off[4][2], n[4][2];
-};
-
-static ActiveList active_list(psms_ctx *c, int all) {
+// after block alike.  Made once per context and active set (the host's walk
+// over a block costs 8 tests per pair of sites: 0.2 s when one block is a
+// lattice of 32^3 x 64).
+static const ActiveList &active_list(psms_ctx *c, int all) {
     const Geom &g = c->g;
-    ActiveList a;
+    ActiveList &a = c->active[all];
+    if (a.d) return a;
     std::vector<int> h;
     for (int mu = 0; mu < 4; ++mu)
         for (int p = 0; p < 2; ++p) {
@@ -431,16 +429,12 @@ static ActiveList active_list(psms_ctx *c, int all) {
             }
             a.n[mu][p] = (int)h.size() - a.off[mu][p];
         }
-    const std::string name = all ? "act_all" : "act_blocks";
-    const auto it = c->scratch.find(name);
-    const bool have = it != c->scratch.end() && it->second.p;
-    int *d = (int *)scratch(c, name, sizeof(int) * (h.empty() ? 1 : h.size()));
-    if (!have && !h.empty()) {
+    int *d = (int *)scratch(c, all ? "act_all" : "act_blocks", sizeof(int) * (h.empty() ? 1 : h.size()));
+    if (!h.empty())
         cuda_check(cudaMemcpyAsync(d, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, c->stream),
                    "active list");
-        cuda_check(cudaStreamSynchronize(c->stream), "active list");
-    }
-    a.d = d;
+    cuda_check(cudaStreamSynchronize(c->stream), "active list");
+    a.d = d;  // (complete: a call on another stream finds it)
     return a;
 }
 
@@ -458,7 +452,7 @@ int gauge_sweep(psms_ctx *c, double2 *U, int active_set, int n_iter, int n_or, d
     for (int col = 0; col < ncol; ++col)
         for (int mu = 0; mu < 4; ++mu)
             for (int p = 0; p < 2; ++p) subs.push_back({mu, p, ncol == 2 ? col : -1});
-    const ActiveList act = active_list(c, all);
+    const ActiveList &act = active_list(c, all);
     int *failed = (int *)scratch(c, "hb_failed", sizeof(int));
     cuda_check(cudaMemsetAsync(failed, 0, sizeof(int), c->stream), "hb memset");
     auto sweep = [&](int kind, bool rev, uint64_t sid) {

@@ -1,6 +1,8 @@
 """Sizes and inputs at which the fixed-point hops, the 256-site block solver
 and the blocked LU can go wrong, against the oracle, the FP64 form of the same
 operator or torch's dense LU."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -9,7 +11,7 @@ import paper_1204_1306_gb300 as ps
 from oracle import dirac, estimator, gauge, lattice
 from oracle.gamma import GAMMA
 from tests import seeded
-from tests.gpu_util import canonical, native, rel_err
+from tests.gpu_util import canonical, get_links, native, rel_err, set_links
 
 pytestmark = pytest.mark.gpu
 
@@ -185,6 +187,33 @@ def test_block_solver_right_hand_sides():
     with pytest.raises(ps.PsmsError) as e:
         ps.psms_solve(ctx, 0, ps.OP_BLOCKS, nat, x, 1e-13, 3, ps.PREC_F32)
     assert e.value.status == 4  # PSMS_ENOCONV
+
+
+def test_sweep_lists_are_made_once():
+    """Both active sets in turn give what a fresh context gives, and a later call
+    does not walk over the block on the host again (one block of 2^20 sites)."""
+    dims, block = (8, 8, 4, 4), (4, 4, 4, 4)
+    ctx, _ = _ctx(dims, block)
+    for k, active in enumerate((ps.ACTIVE_ALL, ps.ACTIVE_BLOCKS, ps.ACTIVE_ALL, ps.ACTIVE_BLOCKS)):
+        fresh, _ = _ctx(dims, block)
+        set_links(fresh, 0, get_links(ctx, 0))
+        for c in (ctx, fresh):
+            ps.psms_gauge_sweep(c, 0, active, 1, 1, 5.3, 3, 10 * k)
+        assert np.array_equal(get_links(ctx, 0), get_links(fresh, 0))
+
+    def calls(n):
+        ctx = ps.psms_create((32, 32, 32, 32), (32, 32, 32, 32), 0.15, 1)
+        t = []
+        for _ in range(n):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            ps.psms_gauge_sweep(ctx, 0, ps.ACTIVE_BLOCKS, 0, 0, 5.3, 3, 0)  # no updates: the lists and the projection
+            t.append(time.perf_counter() - t0)
+        return t
+
+    calls(1)
+    first, *later = calls(6)
+    assert min(later) < 0.5 * first
 
 
 # 16 sites (one sub-panel row per thread), 64, 256, and 512 sites (the tall panels)
