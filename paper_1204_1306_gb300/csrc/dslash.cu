@@ -456,7 +456,9 @@ static __device__ __noinline__ double hop_f64_site(const HopArgs<double2> &a, co
 // the loop over directions is kept rolled: unrolled, its code misses the
 // instruction cache and it is 2.4 times slower).  D_w of 32^3 x 64: 3340 us with
 // FP64 arithmetic, 1332 us at three CTAs per SM, 1166 us at four (1.7 TB/s).
-template <int NT, int MINB, bool DAG>
+// CONV: without room for the converted input, each site is converted by the
+// threads that read it.
+template <int NT, int MINB, bool DAG, bool CONV>
 __global__ void __launch_bounds__(NT, MINB) hop_fx_kernel(const HopArgs<double2> a) {
     __shared__ double sh[NT / 32];
     const int ks = (int)blockIdx.y, bx = (int)blockIdx.x;
@@ -480,11 +482,11 @@ __global__ void __launch_bounds__(NT, MINB) hop_fx_kernel(const HopArgs<double2>
         const int ll = local_lex(g, p, j, y);
         const BlockInfo &bi = a.binfo[r];
         const FxHop h{a.in.p + k * a.in.bs, a.in.cs, a.in.off, (const int4 *)a.U + k * a.U_bs, a.mode, a.dag,
-                      a.fxs + k * a.fxs_bs, a.in.cs, a.in.off};
+                      CONV ? nullptr : a.fxs + k * a.fxs_bs, a.in.cs, a.in.off};
         FxAcc acc;
         fx_zero(acc);
         double f;
-        if (fx_dirs<false, DAG>(h, g, bi, r, p, y, ll, s, acc) && fx_factor(acc, a.b, f)) {
+        if (fx_dirs<CONV, DAG>(h, g, bi, r, p, y, ll, s, acc) && fx_factor(acc, a.b, f)) {
             const double2 *yv = a.y.p ? a.y.p + k * a.y.bs + s - a.y.off : nullptr;
             const double2 *y2v = a.y2.p ? a.y2.p + k * a.y2.bs + s - a.y2.off : nullptr;
             double2 *o = a.out.p + k * a.out.bs + s - a.out.off;
@@ -888,19 +890,16 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     // FP64 hops in fixed point (fixed.cuh).  Few output sites, or a few blocks
     // of a large lattice (whose other sites need no conversion): the
     // directions of a site go to eight warps, which convert what they read;
-    // else a pass converts the input first (no room for its copy: the FP64
-    // kernel).  Directions / pass, us per D_w: 4096 sites 8.4 / 28.9, 8192
-    // 14.5 / 29.0, 16384 23.7 / 28.9, 32768 39.1 / 36.4, 65536 77 / 54.
-    bool fixed = std::is_same<S, Store<double>>::value && h.fx != nullptr;
+    // else a pass converts the input first (no room for its copy: converted as
+    // it is read, which needs no memory).  Directions / pass, us per D_w: 4096
+    // sites 8.4 / 28.9, 8192 14.5 / 29.0, 16384 23.7 / 28.9, 32768 39.1 / 36.4,
+    // 65536 77 / 54.
+    const bool fixed = std::is_same<S, Store<double>>::value && h.fx != nullptr;
     const long long per = (h.p < 0 ? 2LL : 1LL) * a.n_ranks * c->g.Vbh;
     const bool fx_split = !h.partial && (per * nsys <= FX_SPLIT_SITES || 8LL * a.n_ranks <= c->g.nblocks);
     if (fixed && !fx_split) {
         a.fxs_bs = fx_spinors(a.in.cs);
         a.fxs = (longlong2 *)scratch_try(c, "hop_fx", sizeof(longlong2) * (size_t)a.fxs_bs * h.n_sys);
-        if (!a.fxs) {
-            if (!h.U) fail(PSMS_ENOMEM, "hop: no room for the input in fixed point");
-            fixed = false;
-        }
     }
     if (fixed) {
         a.U = h.fx;
@@ -934,13 +933,17 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
                                                 (int)sizeof(FxSplitShared)),
                            "hop shared memory");
                 fn<<<dim3((unsigned)((per + 31) / 32), nsys), 256, sizeof(FxSplitShared), c->stream>>>(a);
-            } else {
+            } else if (a.fxs) {
                 fx_wait(c);
                 spinor_fx_kernel<<<dim3((unsigned)((a.in.cs + 255) / 256), nsys), 256, 0, c->stream>>>(
                     a.in, const_cast<longlong2 *>(a.fxs), a.fxs_bs, h.sys_map, h.active);
                 PSMS_LAUNCH_CHECK("spinor_fx_kernel");
-                (h.dag ? hop_fx_kernel<HOP_NT, 4, true> : hop_fx_kernel<HOP_NT, 4, false>)<<<grid, HOP_NT, 0, c->stream>>>(a);
+                const auto fn = h.dag ? hop_fx_kernel<HOP_NT, 4, true, false> : hop_fx_kernel<HOP_NT, 4, false, false>;
+                fn<<<grid, HOP_NT, 0, c->stream>>>(a);
                 fx_mark(c);
+            } else {
+                const auto fn = h.dag ? hop_fx_kernel<HOP_NT, 4, true, true> : hop_fx_kernel<HOP_NT, 4, false, true>;
+                fn<<<grid, HOP_NT, 0, c->stream>>>(a);
             }
             PSMS_LAUNCH_CHECK("hop_fx_kernel");
             if (slot >= 0) prof_end(c, slot, bytes);

@@ -89,6 +89,33 @@ def test_capture_with_the_default_settings(prec, tol, warm):
     assert float((got - ref).abs().max()) <= tol * float(ref.abs().max())
 
 
+def test_hops_without_room_for_the_converted_input():
+    """All but 256 MB of the device is held, so that the 407 MB copy of the input
+    does not fit: the sites are converted as they are read, to the same bits."""
+    dims = (64, 32, 32, 32)
+    ctx = ps.psms_create(dims, (4, 4, 4, 4), 0.15, 1)
+    ps.psms_gauge_init(ctx, 0, 0.4, 11)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    nat = torch.randn(int(np.prod(dims)) * 24, dtype=torch.float64, device="cuda", generator=g)
+    out = torch.zeros_like(nat)
+    ps.psms_dw_apply(ctx, 0, 3, nat, out, ps.PREC_F64)  # one block: makes the copy of the links, not of the input
+    torch.cuda.synchronize()
+    held = ps.psms_scratch_bytes(ctx)
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (256 << 20), dtype=torch.uint8, device="cuda")
+    ps.psms_dw_apply(ctx, 0, ps.OP_FULL, nat, out, ps.PREC_F64)
+    torch.cuda.synchronize()
+    assert ps.psms_scratch_bytes(ctx) == held
+    got = out.cpu()
+    del fill
+    torch.cuda.empty_cache()
+    ps.psms_dw_apply(ctx, 0, ps.OP_FULL, nat, out, ps.PREC_F64)
+    torch.cuda.synchronize()
+    assert ps.psms_scratch_bytes(ctx) > held
+    assert torch.equal(out.cpu(), got)
+
+
 def test_hops_alternating_between_streams():
     dims = (16, 16, 16, 16)  # the form that keeps the input in scratch
     ctx, _ = _ctx(dims, (4, 4, 4, 4))
