@@ -81,14 +81,23 @@ float2 *links32(psms_ctx *c, int f) {
     return c->U32[f];
 }
 
+// a stream's number, never given twice (a handle is: the work of a destroyed
+// stream may still run when its handle is handed out again)
+static unsigned long long stream_id(cudaStream_t s) {
+    unsigned long long id = 0;
+    cuda_check(cudaStreamGetId(s, &id), "stream id");
+    return id;
+}
+
 void fx_wait(psms_ctx *c) {
-    if (c->fx_ev && c->fx_stream != c->stream) cuda_check(cudaStreamWaitEvent(c->stream, c->fx_ev, 0), "stream order");
+    if (c->fx_ev && c->fx_stream != stream_id(c->stream))
+        cuda_check(cudaStreamWaitEvent(c->stream, c->fx_ev, 0), "stream order");
 }
 
 void fx_mark(psms_ctx *c) {
     if (!c->fx_ev) cuda_check(cudaEventCreateWithFlags(&c->fx_ev, cudaEventDisableTiming), "event create");
     cuda_check(cudaEventRecord(c->fx_ev, c->stream), "event record");
-    c->fx_stream = c->stream;
+    c->fx_stream = stream_id(c->stream);
 }
 
 bool capturing(psms_ctx *c) {

@@ -58,7 +58,7 @@ struct psms_ctx {
     // last use of the fixed-point copies' scratch, or their last conversion:
     // calls on another stream wait for it (psms_dw_apply does not synchronise)
     cudaEvent_t fx_ev = nullptr;
-    cudaStream_t fx_stream = nullptr;
+    unsigned long long fx_stream = 0;  // the stream's number (capi.cu: stream_id)
     std::vector<psms::BlockInfo> h_binfo;
     psms::BlockInfo *d_binfo = nullptr;
     psms::ActiveList active[2];  // of the blocks, of all links

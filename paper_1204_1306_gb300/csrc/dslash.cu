@@ -898,6 +898,7 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     const long long per = (h.p < 0 ? 2LL : 1LL) * a.n_ranks * c->g.Vbh;
     const bool fx_split = !h.partial && (per * nsys <= FX_SPLIT_SITES || 8LL * a.n_ranks <= c->g.nblocks);
     if (fixed && !fx_split) {
+        fx_wait(c);  // (first: a smaller copy in use on another stream may be given back here)
         a.fxs_bs = fx_spinors(a.in.cs);
         a.fxs = (longlong2 *)scratch_try(c, "hop_fx", sizeof(longlong2) * (size_t)a.fxs_bs * h.n_sys);
     }
@@ -934,7 +935,6 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
                            "hop shared memory");
                 fn<<<dim3((unsigned)((per + 31) / 32), nsys), 256, sizeof(FxSplitShared), c->stream>>>(a);
             } else if (a.fxs) {
-                fx_wait(c);
                 spinor_fx_kernel<<<dim3((unsigned)((a.in.cs + 255) / 256), nsys), 256, 0, c->stream>>>(
                     a.in, const_cast<longlong2 *>(a.fxs), a.fxs_bs, h.sys_map, h.active);
                 PSMS_LAUNCH_CHECK("spinor_fx_kernel");

@@ -1,6 +1,7 @@
 """Sizes and inputs at which the fixed-point hops, the 256-site block solver
 and the blocked LU can go wrong, against the oracle, the FP64 form of the same
 operator or torch's dense LU."""
+import ctypes
 import time
 
 import numpy as np
@@ -133,6 +134,28 @@ def test_hops_alternating_between_streams():
     for row in outs:
         for out, ref in zip(row, refs):
             assert torch.equal(out.view(torch.float64), ref)
+
+
+def test_hops_on_streams_that_are_destroyed_at_once():
+    """A stream destroyed with a hop in flight, and the next one, which may get
+    the same handle: the second call waits for the first one's scratch."""
+    dims = (16, 16, 16, 16)
+    ctx, _ = _ctx(dims, (4, 4, 4, 4))
+    nats = [native(ctx, seeded.spinor(dims, k)) for k in range(2)]
+    refs = [_apply(ctx, nat, ps.OP_FULL) for nat in nats]
+    outs = [torch.zeros_like(nats[k % 2]) for k in range(16)]
+    torch.cuda.synchronize()
+    rt = torch.cuda.cudart()
+    for k, out in enumerate(outs):
+        h = ctypes.c_void_p()
+        assert int(rt.cudaStreamCreate(ctypes.addressof(h))) == 0
+        ps.psms_set_stream(ctx, h.value)
+        ps.psms_dw_apply(ctx, 0, ps.OP_FULL, nats[k % 2], out, ps.PREC_F64)
+        assert int(rt.cudaStreamDestroy(h.value)) == 0
+    ps.psms_set_stream(ctx, None)
+    torch.cuda.synchronize()
+    for k, out in enumerate(outs):
+        assert torch.equal(out.view(torch.float64), refs[k % 2])
 
 
 @pytest.mark.parametrize("dims,block", [((4, 4, 4, 4), (2, 2, 2, 2)), ((16, 16, 16, 8), (4, 4, 4, 4))])
