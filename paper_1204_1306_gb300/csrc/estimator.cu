@@ -310,7 +310,7 @@ static long long block_level_chunk(psms_ctx *c, const double2 *U, const double2 
 
 long long block_level(psms_ctx *c, const double2 *U, const double2 *Up, int N, int mode, uint64_t seed,
                       uint64_t counter, double tol, int inner, double *d_delta, const int *d_mask) {
-    const int ch = chunk_size(c, N, inner == P64 ? 2600.0 : 2100.0);
+    const int ch = chunk_size(c, N, level_bytes(LV_BLOCK, inner == P64, c->shared_links));
     long long tot = 0;
     for (int i0 = 0; i0 < N; i0 += ch)
         tot += block_level_chunk(c, U, Up, N, i0, std::min(ch, N - i0), mode, seed, counter, tol, inner, d_delta,
@@ -503,7 +503,7 @@ static long long global_level_chunk(psms_ctx *c, const double2 *U, const double2
 long long global_level(psms_ctx *c, const double2 *U, const double2 *Up, int N, int mode, uint64_t seed,
                        uint64_t counter, double tol, int inner, double *d_delta) {
     if (!c->g.coloured) fail(PSMS_EINVAL, "the Schur complement needs an even number of blocks in every direction");
-    const int ch = chunk_size(c, N, inner == P64 ? 4600.0 : 3700.0);
+    const int ch = chunk_size(c, N, level_bytes(LV_GLOBAL, inner == P64, c->shared_links));
     std::vector<double> h(N);
     long long tot = 0;
     for (int i0 = 0; i0 < N; i0 += ch)

@@ -23,6 +23,7 @@
 #include "estimator.hpp"
 #include "fixed.cuh"
 #include "gauge.hpp"
+#include "interp_plan.hpp"
 #include "outer.cuh"
 #include "outer.hpp"
 #include "solver.hpp"
@@ -168,8 +169,11 @@ void sub_projected(psms_ctx *c, int mode, double2 *out, const double2 *y, double
 }
 
 // interpolated link fields U_{i0} .. U_{i0+n} (or U, U' when independent),
-// masked by `kind` (0 none, 1 crossing links zeroed, 2 only crossing kept),
-// FP64 and, when asked, their FP32 copies
+// masked by `kind` (0 none, 1 crossing links zeroed, 2 only crossing kept):
+// fixed-point copies (the FP64 hops and true residuals) and, when asked, the
+// FP64 or FP32 ones (inner iterations).  Without the FP64 ones, each field
+// passes through a single FP64 field: kept, they are a seventh of a level's
+// memory.
 struct LinkSet {
     double2 *u64 = nullptr;
     int4 *fx = nullptr;
@@ -179,21 +183,23 @@ struct LinkSet {
 };
 
 LinkSet make_links(psms_ctx *c, const double2 *U, const double2 *Up, int N, int mode, int i0, int n, int kind,
-                   bool need32, const char *tag) {
+                   bool need64, bool need32, const char *tag) {
+    const long long V = c->g.V;
     LinkSet ls;
-    ls.nel = 36 * c->g.V;
-    ls.nf = mode == PSMS_EST_INDEPENDENT ? 2 : n + 1;
-    ls.u64 = (double2 *)scratch(c, std::string("ol64_") + tag, sizeof(double2) * ls.nel * ls.nf);
-    if (mode == PSMS_EST_INDEPENDENT)
-        interpolate(c, U, Up, ls.u64, nullptr, 1, 0, 2);
-    else
-        interpolate(c, U, Up, ls.u64, nullptr, N, i0, n + 1);
-    if (kind) mask_links(c, ls.u64, ls.nel, ls.nf, kind);
-    ls.fx = (int4 *)scratch(c, std::string("olfx_") + tag, sizeof(int4) * fx_field(c->g.V) * ls.nf);
-    links_to_fx(c, ls.u64, ls.nel, ls.fx, ls.nf);
-    if (need32) {
-        ls.u32 = (float2 *)scratch(c, std::string("ol32_") + tag, sizeof(float2) * ls.nel * ls.nf);
-        for (int f = 0; f < ls.nf; ++f) links_to_f32(c, ls.u64 + f * ls.nel, ls.u32 + f * ls.nel, ls.nel);
+    ls.nel = 36 * V;
+    const bool ind = mode == PSMS_EST_INDEPENDENT;
+    ls.nf = ind ? 2 : n + 1;
+    const std::string t(tag);
+    if (need64) ls.u64 = (double2 *)scratch(c, "ol64_" + t, sizeof(double2) * ls.nel * ls.nf);
+    double2 *one = need64 ? nullptr : (double2 *)scratch(c, "ol64_one", sizeof(double2) * ls.nel);
+    ls.fx = (int4 *)scratch(c, "olfx_" + t, sizeof(int4) * fx_field(V) * ls.nf);
+    if (need32) ls.u32 = (float2 *)scratch(c, "ol32_" + t, sizeof(float2) * ls.nel * ls.nf);
+    for (int f = 0; f < ls.nf; ++f) {
+        double2 *u = need64 ? ls.u64 + f * ls.nel : one;
+        interpolate(c, U, Up, u, nullptr, ind ? 1 : N, ind ? f : i0 + f, 1);
+        if (kind) mask_links(c, u, ls.nel, 1, kind);
+        links_to_fx(c, u, ls.nel, ls.fx + f * fx_field(V), 1);
+        if (need32) links_to_f32(c, u, ls.u32 + f * ls.nel, ls.nel);
     }
     return ls;
 }
@@ -210,7 +216,7 @@ struct LP {
 LP pair_of(const LinkSet &ls, int mode) {
     LP p;
     p.a64 = ls.u64;
-    p.b64 = ls.u64 + ls.nel;
+    p.b64 = ls.u64 ? ls.u64 + ls.nel : nullptr;
     p.a32 = ls.u32;
     p.b32 = ls.u32 ? ls.u32 + ls.nel : nullptr;
     p.bs = mode == PSMS_EST_INDEPENDENT ? 0 : ls.nel;
@@ -314,7 +320,7 @@ long long sub_chunk(psms_ctx *c, const double2 *U, const double2 *Up, int N, int
     const Geom &g = c->g;
     const long long V = g.V, fs = 12 * V;
     const int nbh = g.nbh, nr = g.nblocks;
-    LinkSet ls = make_links(c, U, Up, N, mode, i0, n, 1, inner != P64, "sub");
+    LinkSet ls = make_links(c, U, Up, N, mode, i0, n, 1, inner == P64, inner != P64, "sub");
     LP pr = pair_of(ls, mode);
     auto buf = [&](const char *name) { return (double2 *)scratch(c, name, sizeof(double2) * fs * n); };
     double2 *xi = buf("sub_xi"), *v = buf("sub_v"), *w = buf("sub_w"), *t1 = buf("sub_t1"), *t2 = buf("sub_t2");
@@ -413,14 +419,14 @@ long long outer_global_chunk(psms_ctx *c, const double2 *U, const double2 *Up, i
     // the whole-lattice FP32 solves read shared endpoint links: no FP32
     // copies of the interpolated fields
     const bool shared = inner != P64 && c->shared_links;
-    LinkSet lf = make_links(c, U, Up, N, mode, i0, n, 0, inner != P64 && !shared, "ogf");
-    LinkSet lm = make_links(c, U, Up, N, mode, i0, n, 1, inner != P64 && !shared, "ogm");
+    LinkSet lf = make_links(c, U, Up, N, mode, i0, n, 0, inner == P64, inner != P64 && !shared, "ogf");
+    LinkSet lm = make_links(c, U, Up, N, mode, i0, n, 1, inner == P64, inner != P64 && !shared, "ogm");
     LinkInterp lim, lif;
     if (shared) {
         lim = link_interp(c, outer_ends(c, U, Up, 1, "ogm"), N, i0, n, 0, mode, "ogm");
         lif = link_interp(c, outer_ends(c, U, Up, 0, "ogf"), N, i0, n, 1, mode, "ogf");
     }
-    LinkSet lc = make_links(c, U, Up, N, mode, i0, n, 2, false, "ogc");
+    LinkSet lc = make_links(c, U, Up, N, mode, i0, n, 2, false, false, "ogc");
     LP pf = pair_of(lf, mode), pm = pair_of(lm, mode), pc = pair_of(lc, mode);
     auto buf = [&](const char *name) { return (double2 *)scratch(c, name, sizeof(double2) * fs * n); };
     double2 *xi = buf("og_xi"), *v = buf("og_v"), *w = buf("og_w"), *t1 = buf("og_t1"), *t2 = buf("og_t2");
@@ -489,7 +495,7 @@ void set_outer(psms_ctx *c, const int *B) {
 long long sub_level(psms_ctx *c, const double2 *U, const double2 *Up, int N, int mode, uint64_t seed,
                     uint64_t counter, double tol, int inner, double *h_delta) {
     if (!has_outer(c)) fail(PSMS_EINVAL, "no outer blocks set (psms_set_outer_blocks)");
-    const int ch = chunk_size(c, N, 2600.0);
+    const int ch = chunk_size(c, N, level_bytes(LV_SUB, inner == P64, c->shared_links));
     std::vector<double> h((long long)n_outer(c) * N, 0.0);
     long long tot = 0;
     for (int i0 = 0; i0 < N; i0 += ch)
@@ -501,7 +507,7 @@ long long sub_level(psms_ctx *c, const double2 *U, const double2 *Up, int N, int
 long long outer_global_level(psms_ctx *c, const double2 *U, const double2 *Up, int N, int mode, uint64_t seed,
                              uint64_t counter, double tol, int inner, double *h_delta) {
     if (!has_outer(c)) fail(PSMS_EINVAL, "no outer blocks set (psms_set_outer_blocks)");
-    const int ch = chunk_size(c, N, 4800.0);
+    const int ch = chunk_size(c, N, level_bytes(LV_OUTER, inner == P64, c->shared_links));
     std::vector<double> h(N, 0.0);
     long long tot = 0;
     for (int i0 = 0; i0 < N; i0 += ch)

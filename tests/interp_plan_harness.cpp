@@ -8,6 +8,10 @@ void interp_coefs_host(int N, int i0, int n, int shift, int independent, float *
     psms::interp_coefs(N, i0, n, shift, independent != 0, ab);
 }
 
+double level_bytes_host(int lv, int fp64_inner, int shared) {
+    return psms::level_bytes((psms::LevelKind)lv, fp64_inner != 0, shared != 0);
+}
+
 int balanced_chunk_host(int N, int k) { return psms::balanced_chunk(N, k); }
 
 }  // extern "C"

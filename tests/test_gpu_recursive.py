@@ -3,6 +3,10 @@ the 5-step filter of Sec. 5) with oracle/recursive.py on identical Philox
 draws: the stage-2 estimates of the outer blocks' Schur complements, the
 global level of the outer decomposition, and filter steps with one level of
 recursion (identical decisions, Delta within 1e-8, links within 1e-12)."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -230,3 +234,38 @@ def test_filter_step_recursive_learned_gauge_fixed():
     assert np.array_equal(ps.psms_filter_record(ctx, ps.REC_ACCEPT_SUB).astype(bool), rec["accept_sub"])
     assert np.array_equal(r["accept_block"], rec["accept_after_sub"])
     assert np.abs(get_links(ctx, 0) - U2).max() < 1e-12
+
+
+LEVELS = [ps.LEVEL_BLOCK, ps.LEVEL_GLOBAL, ps.LEVEL_SUB, ps.LEVEL_OUTER_GLOBAL]
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("plan") / "libplan.so")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "interp_plan_harness.cpp")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-o", out, src], check=True)
+    lib = ctypes.CDLL(out)
+    lib.level_bytes_host.restype = ctypes.c_double
+    return lib
+
+
+@pytest.mark.parametrize("kind", range(4))
+@pytest.mark.parametrize("inner,shared", [(ps.PREC_F32, 1), (ps.PREC_F32, 0), (ps.PREC_F64, 1)])
+def test_level_memory_is_what_the_chunks_are_sized_with(plan, kind, inner, shared):
+    """Scratch that one more system takes, per site, against the figure that
+    divides a level into chunks (csrc/interp_plan.hpp: level_bytes)."""
+    held = []
+    for n in (3, 7):
+        ctx = ps.psms_create((16, 16, 16, 16), (4, 4, 4, 4), 0.14, 2)
+        ps.psms_set_outer_blocks(ctx, (8, 8, 8, 8))
+        ps.psms_shared_links(ctx, bool(shared))
+        ps.psms_gauge_init(ctx, 0, 0.5, 5)
+        ps.psms_gauge_copy(ctx, 1, 0)
+        ps.psms_gauge_sweep(ctx, 1, ps.ACTIVE_BLOCKS, 1, 0, 5.3, 5, 3)
+        start = ps.psms_scratch_bytes(ctx)
+        ps.psms_logdet_ratio(ctx, LEVELS[kind], 0, 1, n, ps.EST_INTERP, 5, 3, 1e-8, inner)
+        held.append(ps.psms_scratch_bytes(ctx) - start)
+    per = (held[1] - held[0]) / 4 / 16 ** 4
+    want = plan.level_bytes_host(kind, int(inner == ps.PREC_F64), shared)
+    # (reductions and per-block results are left out: below 1 %)
+    assert 0.99 * want < per < 1.01 * want
