@@ -337,9 +337,9 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
     if (j < 6) sm.x[j * CG_XS + 128] = make_float4(0, 0, 0, 0);
     const CgSite st_e = cg_site(g, 0, j), st_o = cg_site(g, 1, j);
     const float A = (float)a.A, c4 = (float)(-1.0 / (4.0 * a.A)), h2A = (float)(0.5 / a.A), iA = (float)(1.0 / a.A);
-    const float delta2 = (float)(a.delta * a.delta);
     int total_it = 0, status = 0, slot = 0;
     double rel = 0, rn = bn, rn_old = 0;
+    bool met = false;  // the tolerance, in the step before
     for (int outer = 0;; ++outer) {
         // FP64 true residual r64 = b - D_b x (r64 = b on the first step)
         if (outer > 0) {
@@ -372,12 +372,20 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
             }
             rn = cg_sum64(rn, sm.sh);
         }
+        // BiCGStab ends an inner solve anywhere below its target, up to a
+        // decade, so that two steps of 1e-6 may land just below a tolerance of
+        // 1e-13, where CGNR takes a third: one more step when aim asks for it
         rel = sqrt(rn / bn);
-        if (rel <= a.tol) break;
-        if (outer >= a.max_outer || total_it >= a.maxit) {
+        const double aim = bicg ? a.aim : a.tol;
+        const bool last = outer >= a.max_outer || total_it >= a.maxit;
+        if (rel <= aim || (rel <= a.tol && (met || last))) break;
+        if (last) {
             status = 1;
             break;
         }
+        met = rel <= a.tol;
+        // inner reduction, no further than the rounding of FP64
+        const float delta = (float)(bicg ? fmax(a.delta, 0x1.0p-54 / rel) : a.delta), delta2 = delta * delta;
         const double2 *src = outer ? r64 : b;
         const long long scs = outer ? a.r64.cs : a.b.cs;
         const double scale = 1.0 / sqrt(rn);

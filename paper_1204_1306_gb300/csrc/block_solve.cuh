@@ -267,6 +267,7 @@ struct BlockSolveArgs {
     void *vin;                       // inner scratch base
     long long vin_bs;                // per-system stride of the inner scratch (elements)
     double tol, delta;
+    double aim;                      // block_cg.cuh's BiCGStab: where to stop once tol is met, if one more step gets there
     int maxit, max_outer;
     const int *sys_active;           // per system (nullable)
     const int *block_active;         // per lexicographic block (nullable)

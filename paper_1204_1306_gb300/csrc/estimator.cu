@@ -286,6 +286,7 @@ static long long block_level_chunk(psms_ctx *c, const double2 *U, const double2 
     q.fx = lb.fx;
     q.fx_bs = lb.fx_bs;
     q.tol = tol;
+    q.aim = 0.0625 * tol;
     q.inner_prec = inner;
     q.iters = iters;
     q.resid = resid;
@@ -344,6 +345,7 @@ static long long one_minus_PQ(psms_ctx *c, const OpLinks &l, int N, const double
         q.fx = l.fx;
         q.fx_bs = l.fx_bs;
         q.tol = tol;
+        q.aim = 0.0625 * tol;
         q.inner_prec = inner;
         q.iters = iters;
         q.resid = resid;

@@ -344,6 +344,7 @@ long long sub_chunk(psms_ctx *c, const double2 *U, const double2 *Up, int N, int
         q.fx = pr.afx;
         q.fx_bs = pr.fx_bs;
         q.tol = tol;
+        q.aim = 0.0625 * tol;
         q.inner_prec = inner;
         q.iters = iters;
         q.resid = resid;

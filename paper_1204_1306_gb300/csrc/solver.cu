@@ -118,6 +118,7 @@ void block_solve(psms_ctx *c, const BlockSolveReq &q) {
     a.Uin = in64 ? (const void *)q.U64 : (const void *)q.U32;
     a.Uin_bs = q.U64_bs;  // same element count per field
     a.tol = q.tol;
+    a.aim = q.aim > 0 ? q.aim : q.tol;
     a.delta = in64 ? std::max(0.1 * q.tol, 1e-15) : 1e-6;
     a.maxit = q.maxit;
     a.max_outer = in64 ? 4 : 12;
@@ -1206,7 +1207,7 @@ extern "C" psms_status psms_block_solve_noalloc(psms_ctx *ctx, int field, int op
         a.Uin_bs = 0;
         a.vin = vin;
         a.vin_bs = per_sys;
-        a.tol = tol;
+        a.tol = a.aim = tol;
         a.delta = std::max(0.1 * tol, 1e-15);
         a.maxit = maxit;
         a.max_outer = 4;
@@ -1425,7 +1426,7 @@ psms_status psms_block_plan_create(const psms_block_problem *probs, int n_probs,
             plan_alloc(pl, &vin, (in64 ? sizeof(double2) : sizeof(float2)) * (size_t)per_sys * q.n_rhs);
             a.vin = vin;
             a.vin_bs = per_sys;
-            a.tol = tol;
+            a.tol = a.aim = tol;
             a.delta = in64 ? std::max(0.1 * tol, 1e-15) : 1e-6;
             a.maxit = maxit;
             a.max_outer = in64 ? 4 : 12;

@@ -266,6 +266,25 @@ def test_sweep_lists_are_made_once():
     assert min(later) < 0.5 * first
 
 
+def test_block_level_is_as_accurate_as_with_cgnr():
+    """The estimates' error against a tighter solve, at the tolerance that two
+    BiCGStab corrections of 1e-6 may just meet."""
+    ctx = ps.psms_create((8, 8, 8, 8), (4, 4, 4, 4), 0.156, 2)
+    ps.psms_gauge_init(ctx, 0, 0.5, 21)
+    ps.psms_gauge_copy(ctx, 1, 0)
+    ps.psms_gauge_sweep(ctx, 1, ps.ACTIVE_BLOCKS, 1, 1, 5.3, 22, 0)
+
+    def level(tol):
+        return np.asarray(ps.psms_logdet_ratio(ctx, ps.LEVEL_BLOCK, 0, 1, 12, ps.EST_INTERP, 23, 7, tol, ps.PREC_F32))
+
+    got = level(1e-13)
+    ps.psms_block_krylov(ctx, ps.SOLVER_CGNR)
+    ref = level(1e-14)
+    # |x|^2 of 3072 numbers of unit variance: 4 x 3072 roundings of 2^-53 at most, 1.4e-12; a residual of 1e-13 / 16
+    # moves it by 2 |D_b^-1 r| |x| / sqrt(3072) = 2 |D_b^-1| |b| 6e-15 < 2 x 2 x 110 x 6e-15 = 2.7e-12
+    assert np.sqrt(np.mean((got - ref) ** 2)) < 4e-12
+
+
 # 16 sites (one sub-panel row per thread), 64, 256, and 512 sites (the tall panels)
 @pytest.mark.parametrize("dims,block", [((4, 4, 4, 2), (2, 2, 2, 2)), ((4, 4, 4, 4), (4, 4, 2, 2)),
                                         ((4, 4, 4, 8), (4, 4, 4, 4)), ((8, 4, 4, 4), (8, 4, 4, 4))])
