@@ -10,8 +10,12 @@
 // remain (two Heron steps for the root, the final products and conversions):
 // 0.38 ms.
 //
-// Errors: |z - exact| <= 2^-52 max(1, |z|) (tests/test_gauss_host.py), as for
-// the FP64 functions.
+// Errors (tests/test_gauss_host.py, on the device tests/test_gpu_gauss.py):
+// |z - exact| below 1.6 x 2^-52 of the radius sqrt(-ln u_a); over 8e6 pairs the
+// largest 2.9 and the rms 0.51 units of 2^-53, both those of the FP64
+// functions.  The angle functions are good to 2 units of 2^-62 of the radius,
+// so that a component next to an axis has fewer digits of its own than FP64
+// functions give it (2^-53 of itself).
 #pragma once
 
 #include <math.h>
