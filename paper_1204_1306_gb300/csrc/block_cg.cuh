@@ -4,8 +4,9 @@
 // system) by one CTA of 128 threads.  The inner method is BiCGStab unless the
 // context asks for CGNR: a 1e-6 reduction takes 10 iterations of two Dhat
 // against 24 of Dhat and Dhat^dag (4^4 blocks, beta 5.3, kappa 0.156).  An
-// item whose BiCGStab breaks down or fails to reduce the true residual drops
-// that correction and goes on with CGNR.
+// item whose BiCGStab breaks down, does not get there in CG_BICG_MAX
+// iterations or fails to reduce the true residual starts over with CGNR, with
+// all of its iterations and steps.
 //
 // What bounds it: the FP32 pipe and shared memory (a hop direction is 108 FP32
 // instructions on 11 shared-memory loads; an iteration has four half hops).
@@ -36,6 +37,13 @@ namespace psms {
 constexpr int CG_NT = 128;
 constexpr int CG_XF = 12 * 128 + 16;  // 16-byte elements of a parity's fixed-point spinors (fixed.cuh)
 constexpr int CG_XS = 132;  // sites of an exchange row: 128, one zero site for hops that leave the block, padding
+
+// BiCGStab iterations of one inner solve.  Where it suits the operator it needs
+// far fewer (10 at kappa 0.156 and beta 5.3; 20 on a random field at kappa
+// 0.25, where CGNR takes 130), where it takes more CGNR is the better one: on a
+// smooth field (eps 0.3) 50 against 26 at kappa 0.2, 700 against 35 at 0.25, and
+// at 0.4 it does not converge.
+constexpr int CG_BICG_MAX = 48;
 
 // sum of a CTA's FP32 numbers as hi + lo
 struct ff {
@@ -337,12 +345,13 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
     if (j < 6) sm.x[j * CG_XS + 128] = make_float4(0, 0, 0, 0);
     const CgSite st_e = cg_site(g, 0, j), st_o = cg_site(g, 1, j);
     const float A = (float)a.A, c4 = (float)(-1.0 / (4.0 * a.A)), h2A = (float)(0.5 / a.A), iA = (float)(1.0 / a.A);
-    int total_it = 0, status = 0, slot = 0;
+    int total_it = 0, spent = 0, status = 0, slot = 0;  // (spent: by BiCGStab, before CGNR started over)
     double rel = 0, rn = bn, rn_old = 0;
-    bool met = false;  // the tolerance, in the step before
+    bool met = false;   // the tolerance, in the step before
+    bool quit = false;  // BiCGStab gave up
     for (int outer = 0;; ++outer) {
         // FP64 true residual r64 = b - D_b x (r64 = b on the first step)
-        if (outer > 0) {
+        if (outer > 0 && !quit) {
             // x in fixed point takes the place of the links in shared memory
             longlong2 *xs = reinterpret_cast<longlong2 *>(sm.links);
             rn = 0;
@@ -378,11 +387,21 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
         rel = sqrt(rn / bn);
         const double aim = bicg ? a.aim : a.tol;
         const bool last = outer >= a.max_outer || total_it >= a.maxit;
-        if (rel <= aim || (rel <= a.tol && (met || last))) break;
-        if (last) {
+        if (!quit && (rel <= aim || (rel <= a.tol && (met || last)))) break;
+        if (bicg && (quit || last || (outer > 0 && !(rn <= 0.25 * rn_old)))) {
+            // BiCGStab does not get there: the item starts over with CGNR
+            bicg = quit = false;
+            spent = total_it;
+            total_it = outer = 0;
+            for (int p = 0; p < 2; ++p)
+                for (int q = 0; q < 12; ++q) x[q * a.x.cs + site[p]] = make_double2(0, 0);
+            rn = bn;
+            rel = 1.0;
+        } else if (last) {
             status = 1;
             break;
         }
+        rn_old = rn;
         met = rel <= a.tol;
         // inner reduction, no further than the rounding of FP64
         const float delta = (float)(bicg ? fmax(a.delta, 0x1.0p-54 / rel) : a.delta), delta2 = delta * delta;
@@ -410,8 +429,6 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
         }
         // inner rhs = r64 / |r64| in FP32: even half to the exchange buffer
         // (and kept in global memory for the end), odd half in q
-        if (bicg && outer > 0 && !(rn <= 0.25 * rn_old)) bicg = false;  // no use here: CGNR from now on
-        rn_old = rn;
         Spinor<float> res, pp, q;
         for (int c = 0; c < 12; ++c) {
             const double2 v = src[c * scs + site[0]];
@@ -498,11 +515,9 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
                 cg_dot(load_spinor<Store<float>>(rhov, Vh, site[1]), q, t);
                 ff d[2];
                 cg_sum<2>(t, d, sm.sums, slot);
-                if (!(fabsf(d[0].hi) + fabsf(d[1].hi) > 0)) {  // breakdown (NaN included): the correction so far
-                    bicg = false;
-                    q = load_spinor<Store<float>>(ev, V, site[1]);
-                    cg_put(sm.x, j, q);
-                    step = 7;
+                if (!(fabsf(d[0].hi) + fabsf(d[1].hi) > 0)) {  // breakdown (NaN included)
+                    quit = true;
+                    break;
                 } else {
                     al = cg_div(rho, {d[0].hi, d[1].hi});
                     cg_cadd({-al.re, -al.im}, q, res);  // s
@@ -532,15 +547,13 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
                 cg_cadd({-om.re, -om.im}, t, res);   // r
                 const ff r2 = cg_sum1(cg_norm(res), sm.sums, slot);
                 ++it;
-                if (!(r2.hi > target) || stalled || total_it + it >= a.maxit) {
-                    if (!(r2.hi <= target)) bicg = false;  // stalled, NaN or out of iterations
+                if (r2.hi <= target) {
                     q = e;
-                    if (!(r2.hi * delta2 < target)) {  // no better than e = 0
-                        zero(q);
-                        store_spinor<Store<float>>(ev, V, site[1], q);
-                    }
                     cg_put(sm.x, j, q);
                     step = 7;
+                } else if (stalled || !(r2.hi == r2.hi) || it >= CG_BICG_MAX || total_it + it >= a.maxit) {
+                    quit = true;
+                    break;
                 } else {
                     const cpx<float> be = cmul(cg_div(rho1, rho), cg_div(al, om));
                     rho = rho1;
@@ -583,7 +596,7 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
         xn = cg_sum64(xn, sm.sh);
     }
     if (j == 0) {
-        a.iters[out_i] = total_it;
+        a.iters[out_i] = spent + total_it;
         a.resid[out_i] = rel;
         a.status[out_i] = status;
         if (a.xnorm2) a.xnorm2[out_i] = xn;

@@ -266,6 +266,44 @@ def test_sweep_lists_are_made_once():
     assert min(later) < 0.5 * first
 
 
+# BiCGStab: the better method; slow; stagnating; without convergence
+@pytest.mark.parametrize("kappa,eps", [(0.25, 3.0), (0.2, 0.3), (0.25, 0.3), (0.4, 0.3), (1.0, 0.3), (20.0, 0.3)])
+def test_block_bicgstab_gives_way_to_cgnr(kappa, eps):
+    """Whatever CGNR solves is solved, with BiCGStab's attempts as the only extra
+    cost: 48 iterations at most for each of up to 12 corrections before one fails,
+    which they do at once where they are many."""
+    dims, block = (8, 4, 4, 4), (4, 4, 4, 4)
+    b = seeded.spinor(dims, 7)
+    geom = lattice.Geometry(dims, block)
+    its = {}
+    for krylov in (None, ps.SOLVER_CGNR):
+        ctx, U = _ctx(dims, block, seed=3, kappa=kappa, eps=eps)
+        if krylov is not None:
+            ps.psms_block_krylov(ctx, krylov)
+        nat = native(ctx, b)
+        x = torch.zeros_like(nat)
+        info = ps.psms_solve(ctx, 0, ps.OP_BLOCKS, nat, x, 1e-12, 20000, ps.PREC_F32)
+        r = b - dirac.apply_D(U, canonical(ctx, x), kappa, geom, mode="block")
+        assert np.sqrt(np.sum(np.abs(r) ** 2) / np.sum(np.abs(b) ** 2)) < 2e-12
+        its[krylov] = info["inner_iters"]
+    assert its[None] <= its[ps.SOLVER_CGNR] + 2 * 2 * 48  # two blocks, a failure in the first or second correction
+
+
+@pytest.mark.parametrize("kappa,eps", [(0.4, 0.3), (0.156, 0.5)])
+def test_block_iteration_cap_is_that_of_cgnr(kappa, eps):
+    """A cap that CGNR meets exactly suffices, one below it does not (one block)."""
+    dims = (4, 4, 4, 4)
+    ctx, _ = _ctx(dims, dims, seed=3, kappa=kappa, eps=eps)
+    nat = native(ctx, seeded.spinor(dims, 7))
+    x = torch.zeros_like(nat)
+    ps.psms_block_krylov(ctx, ps.SOLVER_CGNR)
+    need = ps.psms_solve(ctx, 0, ps.OP_BLOCKS, nat, x, 1e-12, 20000, ps.PREC_F32)["inner_iters"]
+    with pytest.raises(ps.PsmsError):
+        ps.psms_solve(ctx, 0, ps.OP_BLOCKS, nat, x, 1e-12, need // 3, ps.PREC_F32)
+    fresh, _ = _ctx(dims, dims, seed=3, kappa=kappa, eps=eps)
+    assert ps.psms_solve(fresh, 0, ps.OP_BLOCKS, nat, x, 1e-12, need, ps.PREC_F32)["true_residual"] <= 1e-12
+
+
 def test_block_level_is_as_accurate_as_with_cgnr():
     """The estimates' error against a tighter solve, at the tolerance that two
     BiCGStab corrections of 1e-6 may just meet."""
