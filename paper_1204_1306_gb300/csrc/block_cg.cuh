@@ -369,7 +369,7 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
 #pragma unroll 1
             for (int p = 0; p < 2; ++p) {
                 const FxHop h{x, a.x.cs, 0, a.fx + k * a.fx_bs, HOP_INTRA, 0, xs + (1 - p) * CG_XF, 128,
-                              site[1 - p] - j};
+                              site[1 - p] - j, a.U64 ? a.U64 + k * a.U64_bs : nullptr};
                 double2 hx[12];
                 fx_site<false>(h, g, bi, r, p, j, 0.5, hx);
                 for (int q = 0; q < 12; ++q) {

@@ -372,7 +372,8 @@ __device__ void block_solve_item(const BlockSolveArgs &a, const int rl, const in
             rn = bn;
         } else if (a.fx) {
             // the same in fixed point: r64 = (b + H(x)/2) - A x in one pass
-            const FxHop h{x, a.x.cs, a.x.off, a.fx + k * a.fx_bs, HOP_INTRA, 0};
+            const FxHop h{x, a.x.cs, a.x.off, a.fx + k * a.fx_bs, HOP_INTRA, 0, nullptr, 0, 0,
+                          a.U64 ? a.U64 + k * a.U64_bs : nullptr};
             for (int p = 0; p < 2; ++p)
                 for (int j = jlo + threadIdx.x; j < jhi; j += NT) {
                     const long long s = blo[p] + j;

@@ -30,6 +30,8 @@ struct HopArgs {
     const int *rank_active;          // per rank: 0 skips its output sites (null: none skipped)
     const longlong2 *fxs;            // P64: the input spinors in fixed point (fixed.cuh)
     long long fxs_bs;
+    const double2 *u64;              // P64: the FP64 links beside the fixed-point ones in U (nullable)
+    long long u64_bs;
     LinkInterp li;                   // shared-endpoint FP32 links (li.U0 null: U, U_bs)
     int nsf;                         // > 0: nsf systems fastest in blockIdx.x (gridDim.y = 1)
     int nct;                         // CTAs per system
@@ -482,7 +484,8 @@ __global__ void __launch_bounds__(NT, MINB) hop_fx_kernel(const HopArgs<double2>
         const int ll = local_lex(g, p, j, y);
         const BlockInfo &bi = a.binfo[r];
         const FxHop h{a.in.p + k * a.in.bs, a.in.cs, a.in.off, (const int4 *)a.U + k * a.U_bs, a.mode, a.dag,
-                      CONV ? nullptr : a.fxs + k * a.fxs_bs, a.in.cs, a.in.off};
+                      CONV ? nullptr : a.fxs + k * a.fxs_bs, a.in.cs, a.in.off,
+                      a.u64 ? a.u64 + k * a.u64_bs : nullptr};
         FxAcc acc;
         fx_zero(acc);
         double f;
@@ -541,7 +544,8 @@ __global__ void __launch_bounds__(256) hop_fx_split_kernel(const HopArgs<double2
         if (l == 0 && cnt) atomicAdd(a.prof_sites, (unsigned long long)cnt);
     }
     const long long s = (long long)p * g.Vh + (long long)r * g.Vbh + j;
-    const FxHop h{a.in.p + k * a.in.bs, a.in.cs, a.in.off, (const int4 *)a.U + k * a.U_bs, a.mode, a.dag};
+    const FxHop h{a.in.p + k * a.in.bs, a.in.cs, a.in.off, (const int4 *)a.U + k * a.U_bs, a.mode, a.dag,
+                  nullptr, 0, 0, a.u64 ? a.u64 + k * a.u64_bs : nullptr};
     FxAcc acc;
     fx_zero(acc);
     bool ok = true;
@@ -864,6 +868,8 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     a.rank_active = h.rank_active;
     a.fxs = nullptr;
     a.fxs_bs = 0;
+    a.u64 = h.prec == P64 ? (const double2 *)h.U : nullptr;
+    a.u64_bs = h.U_bs;
     const bool shared_links = h.li.U0 != nullptr;
     a.li = h.li;
     a.dot = h.dot.dot;

@@ -13,15 +13,18 @@
 // A row of U h is then
 //     sum u h = (HI 2^29 + MID) 2^29 + sum lo lo,
 // HI = sum hi hi and MID = sum (hi lo + lo hi) exact in 64 bits (6 x 2^60 and
-// 12 x 2^59 at most); the last sum, below 2^-58 of the largest product, is
-// dropped.  The eight hops add up as 64-bit integers on one exponent (the
+// 12 x 2^59 at most); the last sum, six products below 2^58 where the largest
+// product is 2^114 at least (below 2^-53 of it in the worst case, 2^-57 in the
+// mean), is dropped.  The eight hops add up as 64-bit integers on one exponent (the
 // largest so far, give or take one), rounded to 2^-54 of the largest product of a link entry
 // and a spinor entry, and become FP64 again once per output.
 //
 // The error of H psi against exact arithmetic is below that of the FP64
 // chain, whose 2^-53 is relative to every partial sum: it is measured in
-// tests/test_fixed_point_host.py.  Numbers outside 2^-823 .. 2^877 (and NaN,
-// infinity) are left to the FP64 form.
+// tests/test_fixed_point_host.py.  That holds for the norm of the error; for
+// every single output it holds where no colour or chirality of a spinor is
+// small against the others, and spinors for which it is not so (fx_spinor),
+// numbers outside 2^-823 .. 2^877, NaN and infinity are left to the FP64 form.
 #pragma once
 
 #include "common.cuh"
@@ -268,18 +271,40 @@ __host__ __device__ __forceinline__ void fx_reconstruct(int mu, const int64_t w[
 // A spinor (24 FP64 numbers, raw bits) as integers on the exponent of its
 // largest number; returns that exponent, 0 for a zero spinor, FX_BAD out of
 // range (v is then zero).
-__host__ __device__ __forceinline__ int fx_spinor(const uint64_t p[12][2], int64_t v[12][2]) {
-    uint32_t em = 0;
+//
+// alike: whether its numbers are so alike that a common exponent costs none of
+// the hops' outputs its FP64 accuracy: every colour of every chirality (spins
+// 0, 1 and spins 2, 3) has a number within 2^-6 of the largest.  Each output
+// number draws on all four numbers of its colour and the other chirality,
+// whatever the links, so that it is then not small against what it is rounded
+// to.  Spinors with a colour or a chirality that is zero or small are left to
+// the FP64 form: in a field whose links do not mix the colours (the unit field,
+// abelian fields) or for a point source an output may hold nothing else.
+// Gaussian spinors are alike but for one in 10^5 (FX_ALIKE = 5: 3 in 10^4).
+constexpr int FX_ALIKE = 6;
+
+__host__ __device__ __forceinline__ int fx_spinor(const uint64_t p[12][2], int64_t v[12][2], bool &alike) {
+    uint32_t em = 0, low = 0xFFFFFFFFu;
     uint64_t any = 0;
 #pragma unroll
-    for (int c = 0; c < 12; ++c)
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const uint32_t e = (uint32_t)(p[c][k] >> 32) & 0x7FF00000u;
-            em = e > em ? e : em;
-            any |= p[c][k];
+        for (int c = 0; c < 3; ++c) {
+            uint32_t m = 0;
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const uint64_t b = p[6 * h + 3 * q + c][k];
+                    const uint32_t e = (uint32_t)(b >> 32) & 0x7FF00000u;
+                    m = e > m ? e : m;
+                    any |= b;
+                }
+            em = m > em ? m : em;
+            low = m < low ? m : low;
         }
     const int ep = (int)(em >> 20);
+    alike = em - low <= (uint32_t)FX_ALIKE << 20;
     if (ep < FX_EMIN || ep > FX_EMAX) {
 #pragma unroll
         for (int c = 0; c < 12; ++c) v[c][0] = v[c][1] = 0;
@@ -290,6 +315,11 @@ __host__ __device__ __forceinline__ int fx_spinor(const uint64_t p[12][2], int64
 #pragma unroll
         for (int k = 0; k < 2; ++k) v[c][k] = fx_convert<FX_UP_SPINOR>(p[c][k], ep);
     return ep;
+}
+
+__host__ __device__ __forceinline__ int fx_spinor(const uint64_t p[12][2], int64_t v[12][2]) {
+    bool alike;
+    return fx_spinor(p, v, alike);
 }
 
 // projected spinor of hop d as limbs

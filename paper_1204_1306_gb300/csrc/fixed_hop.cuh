@@ -16,8 +16,11 @@ struct FxHop {
     // component c of site s at x[c xcs + s - xoff], exponents behind
     const longlong2 *x = nullptr;
     long long xcs = 0, xoff = 0;
+    const double2 *U64 = nullptr;  // the FP64 links, if there are any (for the FP64 form)
 };
 
+// a spinor in fixed point and its exponent word (FX_BAD: out of range or not
+// alike, left to the FP64 form)
 __device__ __forceinline__ int fx_load_spinor(const double2 *q, long long cs, int64_t v[12][2]) {
     uint64_t w[12][2];
 #pragma unroll
@@ -26,12 +29,13 @@ __device__ __forceinline__ int fx_load_spinor(const double2 *q, long long cs, in
         w[c][0] = f64_bits(z.x);
         w[c][1] = f64_bits(z.y);
     }
-    return fx_spinor(w, v);
+    bool alike;
+    const int e = fx_spinor(w, v, alike);
+    return alike ? e : FX_BAD;
 }
 
-// FP64 form of one output site with fixed-point links, for spinors that
-// fixed point does not cover (NaN, infinity, numbers near the ends of the
-// FP64 range).
+// FP64 form of one output site (with the fixed-point links if there are no others), for spinors that
+// fixed point does not cover (fx_load_spinor).
 static __device__ __noinline__ void fx_site_f64(const FxHop &a, const Geom &g, const BlockInfo &bi, int r, int p, int j,
                                                 double2 out[12]) {
     int y[4];
@@ -46,11 +50,15 @@ static __device__ __noinline__ void fx_site_f64(const FxHop &a, const Geom &g, c
             int bs;
             if (!neighbour(g, bi, r, p, y, ll, mu, b ? -1 : 1, a.mode, sn, bs)) continue;
             const long long sl = b ? sn : s;
-            const int ue = fx_exps(a.U, g.V)[(long long)mu * g.V + sl];
             SU3<double> u;
-            for (int e = 0; e < 9; ++e) {
-                const int4 v = a.U[((long long)mu * 9 + e) * g.V + sl];
-                u.e[e / 3][e % 3] = {fx_value(v.x, v.y, ue), fx_value(v.z, v.w, ue)};
+            if (a.U64) {
+                u = load_link<Store<double>>(a.U64, g.V, mu, sl);
+            } else {
+                const int ue = fx_exps(a.U, g.V)[(long long)mu * g.V + sl];
+                for (int e = 0; e < 9; ++e) {
+                    const int4 v = a.U[((long long)mu * 9 + e) * g.V + sl];
+                    u.e[e / 3][e % 3] = {fx_value(v.x, v.y, ue), fx_value(v.z, v.w, ue)};
+                }
             }
             const Spinor<double> v = load_spinor<Store<double>>(a.in, a.cs, sn - a.off);
             const double tt = b ? sg : -sg;

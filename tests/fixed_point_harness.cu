@@ -58,6 +58,19 @@ extern "C" int fx_hops_host(const double *u, const double *psi, int dag, int n, 
     return left;
 }
 
+// out[i] = 1 where the hops take spinor i (psi[n][12] complex) in fixed point
+extern "C" void fx_alike_host(const double *psi, int n, int *out) {
+    for (int i = 0; i < n; ++i) {
+        uint64_t p[12][2];
+        for (int c = 0; c < 12; ++c)
+            for (int k = 0; k < 2; ++k) p[c][k] = f64_bits(psi[(i * 12 + c) * 2 + k]);
+        int64_t x[12][2];
+        bool alike;
+        const int e = fx_spinor(p, x, alike);
+        out[i] = e != 0 && e != FX_BAD && alike;
+    }
+}
+
 // a link through its fixed-point form and back
 extern "C" int fx_link_host(const double *u, double *out) {
     cpx<double> e[9];

@@ -200,6 +200,64 @@ def test_range_and_scaling(lib):
     assert np.array_equal(out, w)
 
 
+def _alike(lib, psi):
+    psi = np.ascontiguousarray(psi.reshape(-1, 4, 3))
+    out = np.zeros(len(psi), dtype=np.int32)
+    lib.fx_alike_host(psi.ctypes.data_as(ctypes.c_void_p), len(psi), out.ctypes.data_as(ctypes.c_void_p))
+    return out.astype(bool)
+
+
+def test_which_spinors_are_left_to_fp64(lib):
+    g = np.random.default_rng(3)
+    psi = (g.standard_normal((200000, 4, 3)) + 1j * g.standard_normal((200000, 4, 3))) / np.sqrt(2)
+    assert (~_alike(lib, psi)).sum() <= 20  # expected: 6 of 200000 x 6 groups of four numbers below 2^-6 of the largest
+    one = psi[:1000]
+    for small in (0.0, 1e-12, 1e-3):
+        q = one.copy()
+        q[:, :, 2] *= small  # a colour
+        assert not _alike(lib, q).any()
+        q = one.copy()
+        q[:, 2:] *= small  # a chirality
+        assert not _alike(lib, q).any()
+        q = one * small
+        q[:, 1, 0] = 1.0  # all but one component
+        assert not _alike(lib, q).any()
+
+
+@pytest.mark.parametrize("kind", ["unit", "abelian", "su3"])
+def test_every_output_is_as_accurate_as_its_terms(lib, kind):
+    """Spinors taken in fixed point whose colours and spins differ as much as they
+    may: the error of each output number against the sum of its terms' sizes."""
+    n, g = 24, np.random.default_rng(4)
+    u, psi = _inputs("su3", n, 6)
+    if kind != "su3":
+        u = np.zeros_like(u)
+        for c in range(3):
+            u[..., c, c] = np.exp(1j * g.uniform(0, 2 * np.pi, (n, 8))) if kind == "abelian" else 1.0
+    psi = psi * 2.0 ** g.uniform(-8, 0, (n, 8, 1, 3)) * 2.0 ** g.uniform(-3, 0, (n, 8, 4, 1))
+    ok = _alike(lib, psi).reshape(n, 8)
+    psi[~ok] = _inputs("su3", n, 8)[1][~ok]
+    assert ok.sum() > n and _alike(lib, psi).all()
+    got, left = _fixed(lib, u, psi, T)
+    assert left == 0
+    exact = _exact(u, psi, T)
+    size = np.zeros((n, 4, 3))  # of the terms of an output
+    for d in range(8):
+        up, dn = np.abs(psi[:, d, :2]), np.abs(psi[:, d, 2:])
+        h = up + (dn if d >> 1 in (0, 3) else dn[:, ::-1])
+        m = np.abs(u[:, d]) if d % 2 == 0 else np.abs(np.swapaxes(u[:, d], -1, -2))
+        w = np.einsum("nab,nsb->nsa", m, h)
+        size[:, :2] += w
+        size[:, 2:] += w if d >> 1 in (0, 3) else w[:, ::-1]
+    for i in range(n):
+        for s in range(4):
+            for c in range(3):
+                q = exact[i][s][c]
+                e = max(abs(float(Fraction(got[i, s, c].real) - q.re)), abs(float(Fraction(got[i, s, c].imag) - q.im)))
+                # eight roundings of 2^-54 of the largest product, which is at most 2^8 x the smallest group's terms
+                assert e <= 2.0 ** -43 * size[i, s, c]
+
+
 def _lu_rows(kind, n, w, seed):
     g = np.random.default_rng(seed)
     l = g.standard_normal((n, w)) + 1j * g.standard_normal((n, w))

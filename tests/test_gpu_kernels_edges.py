@@ -170,6 +170,31 @@ def test_hops_at_the_ends_of_the_fp64_range(dims, block, scale):
     assert float((got / scale - ref).abs().max() / ref.abs().max()) < 64 * 2.0 ** -53
 
 
+@pytest.mark.parametrize("dims,block", [((4, 4, 4, 4), (2, 2, 2, 2)), ((16, 16, 16, 8), (4, 4, 4, 4))])
+def test_hops_of_colours_of_different_size(dims, block):
+    """The unit field does not mix colours: each keeps the accuracy of FP64."""
+    ctx = ps.psms_create(dims, block, 0.15, 1)
+    psi = seeded.spinor(dims, 12) * np.array([1.0, 1e-6, 1e-12])
+    nat = native(ctx, psi)
+    a = canonical(ctx, _apply(ctx, nat, ps.OP_FULL).view(torch.uint8))
+    b = canonical(ctx, _apply(ctx, nat, ps.OP_FULL, graph=True).view(torch.uint8))
+    for c in range(3):
+        assert np.abs(a[..., c] - b[..., c]).max() < 64 * 2.0 ** -53 * np.abs(b[..., c]).max()
+
+
+@pytest.mark.parametrize("dims,block", [((4, 4, 4, 4), (2, 2, 2, 2)), ((16, 16, 16, 8), (4, 4, 4, 4))])
+def test_hops_of_a_point_source(dims, block):
+    """Entries of links next to the unit matrix: each output number is one product."""
+    ctx = ps.psms_create(dims, block, 0.15, 1)
+    ps.psms_gauge_init(ctx, 0, 1e-6, 13)
+    psi = np.zeros(dims + (4, 3), dtype=np.complex128)
+    psi[1, 2, 0, 3, 1, 2] = 1.0
+    nat = native(ctx, psi)
+    a, b = _apply(ctx, nat, ps.OP_FULL), _apply(ctx, nat, ps.OP_FULL, graph=True)
+    assert int((b != 0).sum()) > 60
+    assert bool(((a - b).abs() <= 4 * 2.0 ** -53 * b.abs()).all())
+
+
 @pytest.mark.parametrize("bad", [float("nan"), float("inf")])
 @pytest.mark.parametrize("dims,block", [((4, 4, 4, 4), (2, 2, 2, 2)), ((16, 16, 16, 8), (4, 4, 4, 4))])
 def test_non_finite_spinors_spread_as_in_fp64(dims, block, bad):
