@@ -487,10 +487,9 @@ psms_status psms_max_chunk(psms_ctx *ctx, int n);
  * output site, and on blocks of 2 x 128 sites (4^4) the variants that stage
  * each block's input of the other parity in shared memory by per-thread or
  * bulk (TMA) copies; for FP32 links in the whole-lattice mode 14 variants on
- * such blocks, 10 on others, 15 with shared-endpoint links, 4 otherwise; for
- * FP64 arithmetic 4 in the whole-lattice mode, 1 otherwise (FP64 operators
- * run in fixed point where they can, which has one form); used modulo their
- * count) instead of the autotuned one; -1 returns to autotuning.  All
+ * such blocks, 10 on others, 15 with shared-endpoint links, 4 otherwise; one
+ * form for FP64 operators, in fixed point or, in captured calls, in FP64
+ * arithmetic; used modulo their count) instead of the autotuned one; -1 returns to autotuning.  All
  * variants compute the same operator.  *n_variants (may be NULL) receives
  * 15.  PSMS_EINVAL outside -1..14. */
 psms_status psms_hop_variant(psms_ctx *ctx, int variant, int *n_variants);
