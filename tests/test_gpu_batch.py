@@ -68,3 +68,30 @@ def test_multi_lattice_plan(inner):
         r = dirac.extract_block(rhs[1][0], geom, blk) - dirac.apply_D_open(Ub, dirac.extract_block(got, geom, blk), KAPPA)
         assert np.sqrt(linalg.norm2(r) / linalg.norm2(dirac.extract_block(rhs[1][0], geom, blk))) <= TOL
     plan.close()
+
+
+@pytest.mark.parametrize("blocks,krylov", [(((4, 4, 4, 4), (4, 4, 4, 4)), ps.SOLVER_CGNR),
+                                           (((4, 4, 4, 4), (8, 4, 4, 2)), None),
+                                           (((4, 4, 4, 4), (2, 2, 2, 2)), None)])
+def test_plan_of_one_method_or_several_block_volumes(blocks, krylov):
+    """A plan whose contexts ask for CGNR, one with two shapes of 256 sites, and
+    one that mixes block volumes (which all run the general solver)."""
+    probs, keep = [], []
+    for k, block in enumerate(blocks):
+        ctx = ps.psms_create((8, 8, 4, 4), block, KAPPA, 1)
+        ps.psms_gauge_init(ctx, 0, 0.5, 40 + k)
+        if krylov is not None:
+            ps.psms_block_krylov(ctx, krylov)
+        b = native(ctx, seeded.spinor(ctx.dims, 50 + k))
+        x = torch.zeros_like(b)
+        probs.append((ctx, 0, 1, b, x))
+        ref = torch.zeros_like(b)
+        keep.append((ctx, b, x, ref, ps.psms_solve(ctx, 0, ps.OP_BLOCKS, b, ref, TOL, 20000, ps.PREC_F32)))
+    plan = ps.psms_block_plan_create(probs, TOL, 20000, ps.PREC_F32)
+    info = plan.run()
+    assert info["true_residual"] <= TOL
+    if krylov == ps.SOLVER_CGNR:
+        assert info["inner_iters"] == sum(k[4]["inner_iters"] for k in keep)
+    for ctx, b, x, ref, _ in keep:
+        assert rel_err(canonical(ctx, x), canonical(ctx, ref)) < 1e-10
+    plan.close()

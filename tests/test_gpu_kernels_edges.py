@@ -291,6 +291,19 @@ def test_sweep_lists_are_made_once():
     assert min(later) < 0.5 * first
 
 
+@pytest.mark.parametrize("op", [ps.OP_FULL, ps.OP_BLOCKS])
+def test_solves_whose_sums_overflow_end(op):
+    """Links of 1e25: the FP32 inner iterations' sums become infinite, and the
+    solve ends without convergence."""
+    dims = (8, 4, 4, 4)
+    ctx, U = _ctx(dims, (4, 4, 4, 4))
+    set_links(ctx, 0, U * 1e25)
+    nat = native(ctx, seeded.spinor(dims, 14))
+    with pytest.raises(ps.PsmsError) as e:
+        ps.psms_solve(ctx, 0, op, nat, torch.zeros_like(nat), 1e-12, 500, ps.PREC_F32)
+    assert e.value.status == 4  # PSMS_ENOCONV
+
+
 # BiCGStab: the better method; slow; stagnating; without convergence
 @pytest.mark.parametrize("kappa,eps", [(0.25, 3.0), (0.2, 0.3), (0.25, 0.3), (0.4, 0.3), (1.0, 0.3), (20.0, 0.3)])
 def test_block_bicgstab_gives_way_to_cgnr(kappa, eps):
