@@ -156,12 +156,29 @@ def allsum(ws, v):
 # DRAM bytes (ncu dram__bytes_read.sum + write.sum) / algorithmic bytes of
 # captured launches of the current kernels (profiles/; None: no capture of
 # the current code -- set back to None whenever the kernel changes)
-TRAFFIC_RATIO = {# 16^4 block level, 256 blocks x 12 systems: 12.48 GB of DRAM traffic
-                 # for 118.9 GB of algorithmic bytes in one launch
-                 "block_solve_cluster_kernel": 0.105,
-                 # shared-endpoint-link FP32 hop, 32^3x64 global level, 8 systems:
+TRAFFIC_RATIO = {# shared-endpoint-link FP32 hop, 32^3x64 global level, 8 systems:
                  # 3.75 GB of DRAM traffic for 6.4-7.3 GB of algorithmic bytes
+                 # (captured with the two or three sums of a stage in the hop's
+                 # epilogue; the present form with up to seven reads one more
+                 # spinor field per half hop of the second kind)
                  "hop_kernel": 0.55}
+
+# Block solves with FP32 inner iterations: an iteration (BiCGStab or CGNR) is
+# four half hops of 1320 flop per half-block site; the library reports 4416 B
+# for it, which the solver of blocks of 256 sites does not move (links and
+# vectors stay on the SM), so its rate is given in flop.
+BLOCK_FLOP, BLOCK_BYTES = 4 * 1320.0, 4416.0
+FP32_PEAK = 152 * 128 * 2 * 2.07e9  # SMs x lanes x multiply-add x maximum clock (nominal)
+
+
+def block_flop_entry(kernel, n, ms, nbytes):
+    """Hop flop of the block solver's iterations (nbytes: the library's
+    algorithmic bytes of them) over the summed times of its launches."""
+    achieved = nbytes / BLOCK_BYTES * BLOCK_FLOP / (ms * 1e-3) if ms > 0 else 0.0
+    return {"kernel": kernel, "bound": "fp32", "achieved": round(achieved / 1e12, 2),
+            "peak": round(FP32_PEAK / 1e12, 1), "unit": "TFLOP/s", "frac": round(achieved / FP32_PEAK, 4),
+            "traffic": None, "peak_kind": "nominal", "launches": n, "avg_launch_ms": round(ms / max(n, 1), 4),
+            "total_ms": round(ms, 2)}
 
 
 def roofline_entry(kernel, n, ms, nbytes, peak, peak_kind):
@@ -288,11 +305,11 @@ def dw_only(args):
 def solve_only(args):
     """Whole-lattice and all-blocks solves of one system on the workload
     lattice (FP32 inner iterations, FP64 defect correction to the workload
-    tolerance), with the solvers' algorithmic bytes per Krylov iteration:
-      block CG iteration (per block, FP32): 4 half hops over the block
-        (in, out, 8 links per output site; y on the second hop of a pair) and
-        the vector updates (12 half-vector passes) = 4416 B per half-block site;
-      whole-lattice CG iteration: the same per half-lattice site.
+    tolerance).  Per Krylov iteration and half-lattice (half-block) site: 4
+    half hops (in, out, 8 links per output site; y on the second hop of a
+    pair) and the vector updates (12 half-vector passes), 4416 B as the
+    whole-lattice solver moves them, and the hops' 5280 flop, which is what
+    the block solver is measured by (its blocks stay on the SM).
     This is the small case for Nsight Compute captures of the solver kernels."""
     import torch
 
@@ -312,7 +329,6 @@ def solve_only(args):
     ps.psms_spinor_import(ctx, canon, b, ps.PREC_F64)
     peak, kind = peaks()
     out = {"workload": args.workload, "peak_gbs": peak, "peak_kind": kind}
-    per_site = 4416.0
     for name, op in (("blocks", ps.OP_BLOCKS), ("full", ps.OP_FULL)):
         for _ in range(max(1, args.warmup - 2)):
             ps.psms_solve(ctx, 0, op, b, x, wl["tol"], 20000, ps.PREC_F32)
@@ -330,9 +346,11 @@ def solve_only(args):
         if op == ps.OP_BLOCKS:
             nblk = int(np.prod([d // l for d, l in zip(wl["dims"], wl["block"])]))
         half_sites = (V / 2) / nblk
-        gbs = its * half_sites * per_site / (ms * 1e-3) / 1e9
         out[name] = {"ms": round(ms, 2), "inner_iters": its, "true_residual": info["true_residual"],
-                     "algorithmic_GB/s": round(gbs, 1), "frac": round(gbs / peak, 4)}
+                     "hop_TFLOP/s": round(its * half_sites * BLOCK_FLOP / (ms * 1e-3) / 1e12, 2)}
+        if op == ps.OP_FULL:
+            gbs = its * half_sites * BLOCK_BYTES / (ms * 1e-3) / 1e9
+            out[name].update({"algorithmic_GB/s": round(gbs, 1), "frac": round(gbs / peak, 4)})
     print(json.dumps(out), flush=True)
 
 
@@ -453,12 +471,11 @@ def measure_batch(ps, torch, steps=3, warmup=3):
     sched = plan.schedule()
     items = infos[0]["n_systems"]
     iters = infos[0]["inner_iters"]
-    gbs = iters * 128 * 4416.0 / (ms * 1e-3) / 1e9
-    peak, kind = peaks()
+    flops = iters * 128 * BLOCK_FLOP / (ms * 1e-3)
     out = {"workload": "8^4 + 12^4 + 16^3x32, 4^4 blocks x 16 noises", "systems": items,
            "batch_ms": round(ms, 3), "per_solve_latency_ms": round(ms * sched["ctas"] / items, 4),
-           "block_cg_iterations": iters, "algorithmic_GB/s": round(gbs, 1), "frac": round(gbs / peak, 4),
-           "peak_gbs": peak, "peak_kind": kind, "schedule": sched,
+           "block_iterations": iters, "hop_TFLOP/s": round(flops / 1e12, 2),
+           "frac_fp32": round(flops / FP32_PEAK, 4), "peak_kind": "nominal", "schedule": sched,
            "true_residual": max(i["true_residual"] for i in infos)}
     plan.close()
     for c in ctxs:
@@ -594,9 +611,10 @@ def block_only(args):
     n interpolation steps (--block-n, default 12) between the gauge-fixed
     endpoints of one domain-sweep proposal, FP32 inner iterations to the
     workload tolerance, one persistent launch of the block solver per call.
-    The first call autotunes the solver variant; --steps calls are timed
-    with CUDA events.  The small case for Nsight Compute captures of
-    block_solve_cluster_kernel (about 1 GB on the device at n = 12)."""
+    --steps calls are timed with CUDA events.  The small case for Nsight
+    Compute captures of block_cg_kernel, and with --block-variant of the
+    general solver, block_solve_cluster_kernel (about 1 GB on the device at
+    n = 12)."""
     import torch
 
     import paper_1204_1306_gb300 as ps
@@ -626,13 +644,12 @@ def block_only(args):
         torch.cuda.synchronize()
         ms.append(e0.elapsed_time(e1))
     nl, bms, bbytes = ps.psms_profile_read_block(ctx)
-    peak, kind = peaks()
     nb = ps.psms_geometry_info(ctx)[0]
     print(json.dumps({"workload": "16^4 block level", "n": n, "blocks": nb, "variant": args.block_variant,
                       "ms_per_call": statistics.median(ms),
                       "estimates_per_s": nb * n / (statistics.median(ms) * 1e-3),
-                      "block_solver": {"launches": nl, "ms": round(bms, 3), "algorithmic_GB/s": round(
-                          bbytes / (bms * 1e-3) / 1e9, 1) if bms > 0 else None, "peak_gbs": peak, "peak_kind": kind}}),
+                      "block_solver": {"launches": nl, "ms": round(bms, 3), "hop_TFLOP/s": round(
+                          bbytes / BLOCK_BYTES * BLOCK_FLOP / (bms * 1e-3) / 1e12, 2) if bms > 0 else None}}),
           flush=True)
     ctx.close()
 
@@ -956,8 +973,17 @@ def our_arm(args):
                             "site); the whole-lattice solves form them from two shared endpoint fields that HBM "
                             "delivers about once per launch, so 'achieved' is an effective rate above the DRAM "
                             "traffic ('traffic')")
-    rl_blk = roofline_entry("block_solve_cluster_kernel<float> (persistent Dirichlet-block CG, FP32 inner)", blk_n,
-                            blk_ms, blk_bytes, peak, peak_kind)
+    if int(np.prod(wl["block"])) == 256:
+        rl_blk = block_flop_entry("block_cg_kernel (Dirichlet blocks of 256 sites resident in one CTA, FP32 inner)",
+                                  blk_n, blk_ms, blk_bytes)
+        rl_blk["bound_note"] = ("flop of the hops alone (the vector updates and sums come on top); bound by FP32 "
+                                "issue, shared memory and the barriers of an iteration")
+    else:
+        rl_blk = roofline_entry("block_solve_cluster_kernel<float> (persistent Dirichlet-block CG, FP32 inner)",
+                                blk_n, blk_ms, blk_bytes, peak, peak_kind)
+        rl_blk["bound_note"] = ("effective rate: 'achieved' counts every CG pass over a block as memory traffic "
+                                "(the det-ratio metric's per-iteration bytes) while L1/L2 serve most of it, so it "
+                                "can exceed the HBM copy rate; the kernel is bound by instruction issue and latency")
     ratio = TRAFFIC_RATIO.get("hop_kernel")
     if ratio is not None and hop_n:
         rl_hop["traffic"] = ratio * hop_bytes / hop_n
@@ -965,16 +991,6 @@ def our_arm(args):
                                   f"shared-endpoint-link FP32 hop (32^3x64 global level) = {ratio}, times the mean "
                                   "algorithmic bytes per launch of the timed steps; below 1 because the systems of "
                                   "a launch read the endpoint links from L2")
-    ratio = TRAFFIC_RATIO.get("block_solve_cluster_kernel")
-    if ratio is not None and blk_n:
-        # DRAM bytes per launch, scaled from the capture by the algorithmic
-        # bytes (block-CG iterations x sites) of the timed launches
-        rl_blk["traffic"] = ratio * blk_bytes / blk_n
-        rl_blk["traffic_note"] = ("ncu dram__bytes_read+write of one launch / its algorithmic bytes = "
-                                  f"{ratio}, times the mean algorithmic bytes per launch of the timed steps")
-    rl_blk["bound_note"] = ("effective rate: 'achieved' counts every CG pass over a block as memory traffic "
-                            "(the det-ratio metric's per-iteration bytes) while L1/L2 serve most of it, so it can "
-                            "exceed the HBM copy rate; the kernel is bound by instruction issue and latency")
     # the dominant kernel of the step: the larger measured time
     rl_main, rl_other = (rl_blk, rl_hop) if blk_ms >= hop_ms else (rl_hop, rl_blk)
     if rank != 0:
