@@ -405,7 +405,7 @@ __global__ void residual_flags_kernel(const double *rn, const double *bn, double
     if (k >= n) return;
     double r = bn[k] > 0 ? sqrt(rn[k] / bn[k]) : 0.0;
     rel[k] = r;
-    act[k] = (r > tol) ? 1 : 0;
+    act[k] = (r <= tol) ? 0 : 1;  // (NaN has not converged)
 }
 
 __global__ void set_int_kernel(int *p, int v, int n) {
@@ -1011,7 +1011,7 @@ void solve_full_batch(psms_ctx *c, const FullSolveReq &q, psms_solve_info *info)
         cuda_check(cudaMemcpyAsync(hrn.data(), rn, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream), "rn");
         cuda_check(cudaStreamSynchronize(c->stream), "solve sync");
         bool any = false;
-        for (int k = 0; k < n; ++k) any |= hact[k] != 0;
+        for (int k = 0; k < n; ++k) any |= hact[k] != 0 && hrn[k] == hrn[k];  // (no way on from a NaN)
         if (!any || outer >= max_outer) break;
         if (bicg && outer > 0)
             for (int k = 0; k < n; ++k)
@@ -1073,7 +1073,7 @@ void solve_full_batch(psms_ctx *c, const FullSolveReq &q, psms_solve_info *info)
     double worst = 0;
     long long tot = 0;
     for (int k = 0; k < n; ++k) {
-        worst = std::max(worst, hrel[k]);
+        if (worst == worst && !(hrel[k] <= worst)) worst = hrel[k];  // (a NaN is the worst)
         tot += hit[k];
     }
     if (info) {
