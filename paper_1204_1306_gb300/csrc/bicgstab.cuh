@@ -58,6 +58,32 @@ __device__ __forceinline__ void bcg_stage(BCS *st, int k, const double v[BCG_SUM
     flags[k] = s.active;
 }
 
+// The same for iterations that take rho' from the new residual (solver.cu says
+// which).  stage 0 as above; 1: omega alone; 2: sums 0, 1: <rh, r>; 2: |r|^2;
+// rho', beta, convergence
+__device__ __forceinline__ void bcg_stage_direct(BCS *st, int k, const double v[BCG_SUMS], int stage, int maxit,
+                                                 int *flags) {
+    if (stage == 0) {
+        bcg_stage(st, k, v, 0, maxit, flags);
+        return;
+    }
+    BCS s = st[k];
+    if (stage == 1) {
+        s.omega = v[2] > 0.0 ? make_double2(v[0] / v[2], v[1] / v[2]) : make_double2(0.0, 0.0);
+        s.stalled = !(s.omega.x * s.omega.x + s.omega.y * s.omega.y > 0.0);
+    } else {
+        const double2 rho = make_double2(v[0], v[1]);
+        s.stalled = s.stalled || !(rho.x * rho.x + rho.y * rho.y > 0.0);
+        s.beta = s.stalled ? make_double2(0.0, 0.0) : cmul2(cdiv(rho, s.rho), cdiv(s.alpha, s.omega));
+        s.rho = rho;
+        s.iters += 1;
+        s.rr = v[2];
+        if (v[2] <= s.target || s.iters >= maxit || s.stalled || !(v[2] == v[2])) s.active = 0;
+    }
+    st[k] = s;
+    flags[k] = s.active;
+}
+
 // Sums over a warp of P values per lane (P = 1, 2, 4, 8): while there are
 // several, half of them go to the other half of the lanes, so that 8 sums
 // take 9 FP64 additions and not 40 (a warp's FP64 addition occupies the two
@@ -129,8 +155,8 @@ __device__ __forceinline__ int wsum_index(int l) {  // the leading bits of the l
 // finish (a counter per system, no waiting) sums all partials in a fixed
 // order and applies the scalar stage, so the result does not depend on
 // which CTA finishes last.  part: BCG_SUMS arrays of part_n doubles; the sums
-// [LO, HI) are taken.  Ends at a barrier.
-template <int NT, int LO, int HI, class T>
+// [LO, HI) are taken.  DIRECT: bcg_stage_direct.  Ends at a barrier.
+template <int NT, int LO, int HI, bool DIRECT = false, class T>
 __device__ __forceinline__ void bcg_partials_and_stage(BCS *st, const T in[BCG_SUMS], double *part,
                                                        long long part_n, unsigned int *counters, int stage, int maxit,
                                                        int *flags, double (*sh)[NT / 32], int k, int cta, int nct) {
@@ -180,7 +206,8 @@ __device__ __forceinline__ void bcg_partials_and_stage(BCS *st, const T in[BCG_S
             v[a] = t;
         }
         counters[k] = 0;
-        bcg_stage(st, k, v, stage, maxit, flags);
+        if constexpr (DIRECT) bcg_stage_direct(st, k, v, stage, maxit, flags);
+        else bcg_stage(st, k, v, stage, maxit, flags);
     }
     __syncthreads();
 }

@@ -627,9 +627,9 @@ __global__ void __launch_bounds__(NT) bcg_s_kernel(const BCS *st, View<typename 
 }
 
 // the dot products of a stage over whole vectors, for storage precisions
-// whose hops do not take them: stage 0: <rh, v>; 1: <t, s>, |t|^2, <rh, t>, <rh, s>
-// (a = v or t, b = s)
-template <class S, int NT>
+// whose hops do not take them: stage 0: <rh, v>; 1: <t, s>, |t|^2 and, unless
+// DIRECT, <rh, t>, <rh, s> (a = v or t, b = s)
+template <class S, int NT, bool DIRECT>
 __global__ void __launch_bounds__(NT) bcg_dot_stage_kernel(BCS *st, View<typename S::elem> a, View<typename S::elem> b,
                                                            View<typename S::elem> rh, long long s_lo, long long n,
                                                            double *part, long long part_n, unsigned int *counters,
@@ -644,7 +644,9 @@ __global__ void __launch_bounds__(NT) bcg_dot_stage_kernel(BCS *st, View<typenam
     if (i < n && (!rank_active || rank_active[(int)(i >> vbh_sh)])) {
         const long long sx = s_lo + i;
         const Spinor<R> av = load_spinor<S>(a.p + k * a.bs, a.cs, sx - a.off);
-        const Spinor<R> hv = load_spinor<S>(rh.p + k * rh.bs, rh.cs, sx - rh.off);
+        Spinor<R> hv;
+        if (DIRECT && stage == 1) zero(hv);  // (not used)
+        else hv = load_spinor<S>(rh.p + k * rh.bs, rh.cs, sx - rh.off);
         R xr = 0, xi = 0, yr = 0, yi = 0, aa = 0, zr = 0, zi = 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q)
@@ -679,8 +681,8 @@ __global__ void __launch_bounds__(NT) bcg_dot_stage_kernel(BCS *st, View<typenam
             sum[1] = xi;
         }
     }
-    bcg_partials_and_stage<NT, 0, BCG_SUMS>(st, sum, part, part_n, counters, stage, maxit, flags, sh, k,
-                                            (int)blockIdx.x, (int)gridDim.x);
+    bcg_partials_and_stage<NT, 0, DIRECT ? 3 : BCG_SUMS, DIRECT>(st, sum, part, part_n, counters, stage, maxit, flags,
+                                                                 sh, k, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v), then
@@ -688,7 +690,15 @@ __global__ void __launch_bounds__(NT) bcg_dot_stage_kernel(BCS *st, View<typenam
 // site unit by unit, which keeps it at few registers and the SMs full (42 us for
 // 12 systems at 16^4, 7.2 TB/s, part of it from L2; whole spinors at once: 12 %
 // occupancy and 60 us), with one reduction per site (one per unit: 71 us).
-template <class S, int NT>
+//
+// DIRECT (FP64 iterations): p is left to bcg_p_kernel, and stage 2 gets <rh, r>
+// of the new r (rh in v's place).  rho' from the sums of the second operator is
+// uncertain by the rounding of s and t, which grows against <rh, r> as r falls:
+// FP64 iterations, which run to the tolerance in one go, stalled at the cap on
+// ill-conditioned operators (over kappa 0.12 to 1 on fields of eps 0.3 and 0.5,
+// two lattices: 1.66 times the iterations in the mean); FP32 ones, restarted every
+// six digits, need as many either way (1.03 times).
+template <class S, int NT, bool DIRECT>
 __global__ void __launch_bounds__(NT) bcg_update_stage_kernel(BCS *st, View<typename S::elem> x,
                                                               View<typename S::elem> p, View<typename S::elem> r,
                                                               View<typename S::elem> s_, View<typename S::elem> t,
@@ -707,7 +717,7 @@ __global__ void __launch_bounds__(NT) bcg_update_stage_kernel(BCS *st, View<type
         const double2 a = st[k].alpha, o = st[k].omega, b = st[k].beta;
         const cpx<R> al = {(R)a.x, (R)a.y}, om = {(R)o.x, (R)o.y}, be = {(R)b.x, (R)b.y};
         const long long sx = s_lo + i;
-        R aa = 0;
+        R aa = 0, hr = 0, hi = 0;
 #pragma unroll 1
         for (int u = 0; u < 12 / NC; ++u) {
             auto at = [&](const View<typename S::elem> &w) { return w.p + k * w.bs + (u * w.cs + sx - w.off) * NC; };
@@ -721,18 +731,55 @@ __global__ void __launch_bounds__(NT) bcg_update_stage_kernel(BCS *st, View<type
             for (int c = 0; c < NC; ++c) {
                 xv[c] = xv[c] + cmul(al, pv[c]) + cmul(om, sv[c]);
                 const cpx<R> rv = sv[c] - cmul(om, tv[c]);
-                pv[c] = rv + cmul(be, pv[c] - cmul(om, vv[c]));
+                if constexpr (DIRECT) {
+                    hr += vv[c].re * rv.re + vv[c].im * rv.im;
+                    hi += vv[c].re * rv.im - vv[c].im * rv.re;
+                } else {
+                    pv[c] = rv + cmul(be, pv[c] - cmul(om, vv[c]));
+                }
                 sv[c] = rv;
                 aa += rv.re * rv.re + rv.im * rv.im;
             }
             store_unit<S>(at(x), xv);
             store_unit<S>(at(r), sv);
-            store_unit<S>(at(p), pv);
+            if constexpr (!DIRECT) store_unit<S>(at(p), pv);
+        }
+        if constexpr (DIRECT) {
+            sum[0] = hr;
+            sum[1] = hi;
         }
         sum[2] = aa;
     }
-    bcg_partials_and_stage<NT, 2, 3>(st, sum, part, part_n, counters, 2, maxit, flags, sh, k, (int)blockIdx.x,
-                                     (int)gridDim.x);
+    bcg_partials_and_stage<NT, DIRECT ? 0 : 2, 3, DIRECT>(st, sum, part, part_n, counters, 2, maxit, flags, sh, k,
+                                                          (int)blockIdx.x, (int)gridDim.x);
+}
+
+// p = r + beta (p - omega v)
+template <class S, int NT>
+__global__ void __launch_bounds__(NT) bcg_p_kernel(const BCS *st, View<typename S::elem> p, View<typename S::elem> r,
+                                                   View<typename S::elem> v, long long s_lo, long long n,
+                                                   const int *map, const int *rank_active, int vbh_sh) {
+    using R = typename S::R;
+    constexpr int NC = 1 << S::VSH;
+    const int k = map ? map[blockIdx.y] : (int)blockIdx.y;
+    if (!st[k].active) return;
+    const long long i = (long long)blockIdx.x * NT + threadIdx.x;
+    if (i >= n) return;
+    if (rank_active && !rank_active[(int)(i >> vbh_sh)]) return;
+    const double2 o = st[k].omega, b = st[k].beta;
+    const cpx<R> om = {(R)o.x, (R)o.y}, be = {(R)b.x, (R)b.y};
+    const long long sx = s_lo + i;
+#pragma unroll
+    for (int u = 0; u < 12 / NC; ++u) {
+        auto at = [&](const View<typename S::elem> &w) { return w.p + k * w.bs + (u * w.cs + sx - w.off) * NC; };
+        cpx<R> pv[NC], rv[NC], vv[NC];
+        load_unit<S>(at(p), pv);
+        load_unit<S>(at(r), rv);
+        load_unit<S>(at(v), vv);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) pv[c] = rv[c] + cmul(be, pv[c] - cmul(om, vv[c]));
+        store_unit<S>(at(p), pv);
+    }
 }
 
 __global__ void iters_bcg_kernel(const BCS *st, int *out, int n) {
@@ -812,6 +859,7 @@ static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long lo
     // last CTA of a system applies the stage), saving two passes over two
     // vectors per iteration
     const bool fuse = prec == P32;
+    constexpr bool direct = std::is_same<SV, Store<double>>::value;  // rho' from the residual itself
     // w = Dhat u = A u + c4 H_o(H_e u); dot 1: stage 0 on <x, w>; dot 2:
     // stage 1 on <w, u>, |w|^2, <x, w>
     auto apply_dhat = [&](View<void> u, View<void> w, int dot, View<void> x, int stage) {
@@ -863,25 +911,28 @@ static void inner_bicgstab_full(psms_ctx *c, int n_sys, const void *Uin, long lo
             // alpha = rho / <rh, v>
             apply_dhat(pp, vv, 1, rh, 0);
             if (!fuse) {
-                bcg_dot_stage_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(vv), tv(ss), tv(rh), Vh, n, part,
-                                                                          part_n, cnt, 0, maxit, flags, map,
-                                                                          rank_active, vsh);
+                bcg_dot_stage_kernel<SV, NT, direct><<<gridm, NT, 0, c->stream>>>(
+                    st, tv(vv), tv(ss), tv(rh), Vh, n, part, part_n, cnt, 0, maxit, flags, map, rank_active, vsh);
                 PSMS_LAUNCH_CHECK("bcg_alpha");
             }
             bcg_s_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(r), tv(vv), tv(ss), Vh, n, map, rank_active, vsh);
             PSMS_LAUNCH_CHECK("bcg_s");
-            // omega, rho, beta
+            // omega, rho, beta (FP64 iterations: omega)
             apply_dhat(ss, tt, 2, rh, 1);
             if (!fuse) {
-                bcg_dot_stage_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(tt), tv(ss), tv(rh), Vh, n, part,
-                                                                          part_n, cnt, 1, maxit, flags, map,
-                                                                          rank_active, vsh);
+                bcg_dot_stage_kernel<SV, NT, direct><<<gridm, NT, 0, c->stream>>>(
+                    st, tv(tt), tv(ss), tv(rh), Vh, n, part, part_n, cnt, 1, maxit, flags, map, rank_active, vsh);
                 PSMS_LAUNCH_CHECK("bcg_omega");
             }
             // x, r, p and convergence
-            bcg_update_stage_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(e), tv(pp), tv(r), tv(ss), tv(tt),
-                                                                         tv(vv), Vh, n, part, part_n, cnt, maxit,
-                                                                         flags, map, rank_active, vsh);
+            bcg_update_stage_kernel<SV, NT, direct><<<gridm, NT, 0, c->stream>>>(
+                st, tv(e), tv(pp), tv(r), tv(ss), tv(tt), tv(direct ? rh : vv), Vh, n, part, part_n, cnt, maxit, flags,
+                map, rank_active, vsh);
+            if constexpr (direct) {
+                PSMS_LAUNCH_CHECK("bcg_update");
+                bcg_p_kernel<SV, NT><<<gridm, NT, 0, c->stream>>>(st, tv(pp), tv(r), tv(vv), Vh, n, map, rank_active,
+                                                                  vsh);
+            }
             PSMS_LAUNCH_CHECK("bcg_update");
         }
         cuda_check(cudaMemcpyAsync(hflags.data(), flags, sizeof(int) * n_sys, cudaMemcpyDeviceToHost, c->stream),

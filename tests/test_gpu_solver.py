@@ -225,3 +225,20 @@ def test_profile_precision_filter_and_inner_reduction():
     with pytest.raises(ps.PsmsError):
         ps.psms_inner_reduction(ctx, 0.9)
     ps.psms_inner_reduction(ctx, 0.0)
+
+
+@pytest.mark.parametrize("kappa", [0.25, 0.4])
+@pytest.mark.parametrize("seed", [0, 1])
+def test_fp64_bicgstab_on_ill_conditioned_operators(kappa, seed):
+    """FP64 iterations run to the tolerance in one go; rho from the residual
+    itself keeps them going (450 to 1942 iterations), rho from the sums of the
+    second operator stalled them at the cap of 3000."""
+    dims = (8, 8, 8, 8)
+    ctx = ps.psms_create(dims, (4, 4, 4, 4), kappa, 1)
+    ps.psms_gauge_init(ctx, 0, 0.3, seed)
+    n = int(np.prod(dims)) * 24
+    b = torch.randn(n, generator=torch.Generator().manual_seed(seed), dtype=torch.float64).cuda()
+    nat = torch.empty(ps.psms_spinor_bytes(ctx, ps.PREC_F64), dtype=torch.uint8, device="cuda")
+    ps.psms_spinor_import(ctx, b, nat, ps.PREC_F64)
+    info = ps.psms_solve(ctx, 0, ps.OP_FULL, nat, torch.zeros_like(nat), 1e-8, 3000, ps.PREC_F64)
+    assert info["true_residual"] <= 1e-8 and info["inner_iters"] < 3000
