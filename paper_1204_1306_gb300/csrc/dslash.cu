@@ -454,10 +454,11 @@ static __device__ __noinline__ double hop_f64_site(const HopArgs<double2> &a, co
 }
 
 // One thread per output site: b (sum of hops) in integers, a y + a2 y2 and
-// the result in FP64.  Issue and latency bound it (7.9k instructions per site;
-// the loop over directions is kept rolled: unrolled, its code misses the
-// instruction cache and it is 2.4 times slower).  D_w of 32^3 x 64: 3340 us with
-// FP64 arithmetic, 1332 us at three CTAs per SM, 1166 us at four (1.7 TB/s).
+// the result in FP64.  Latency and issue bound it (8.8k instructions per site,
+// 43 % of the issue slots, FP64 pipe 38 %; the loop over directions is kept
+// rolled: unrolled, its code misses the instruction cache and it is 2.4 times
+// slower).  D_w of 32^3 x 64: 3340 us with FP64 arithmetic, 1332 us at three
+// CTAs per SM, 1166 us at four (1.7 TB/s).
 // CONV: without room for the converted input, each site is converted by the
 // threads that read it.
 template <int NT, int MINB, bool DAG, bool CONV>
@@ -958,9 +959,12 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
     }
     // Register cap (minimum resident CTAs per SM) chosen by the autotuner:
     // on the first launch of each (precision, parity shape) every variant is
-    // timed twice with CUDA events and the fastest is kept.  All variants do
-    // identical arithmetic; a launch is idempotent (out is a function of in, y,
-    // y2, U only), so the extra tuning launches leave the result unchanged.
+    // timed twice with CUDA events and the fastest is kept, among those that do
+    // identical arithmetic: the forms with two threads per site add the hops in
+    // another order, and a choice by time must not change the bits (an
+    // ill-conditioned solve takes another number of steps with them).  A launch
+    // is idempotent (out is a function of in, y, y2, U only), so the extra tuning
+    // launches leave the result unchanged.
     using KFn = void (*)(const HopArgs<E>);
     constexpr bool f32 = sizeof(typename SL::R) == 4;
     const bool all = h.mode == HOP_ALL;
@@ -996,6 +1000,7 @@ static int hop_launch_t(psms_ctx *c, const HopCall &h) {
         cuda_check(cudaEventCreate(&e1), "tune event");
         float best = 1e30f;
         for (int v = 0; v < nvar; ++v) {
+            if (thr && thr[v] != HOP_NT) continue;  // (two threads per site)
             vars[v]<<<grid, thr ? thr[v] : HOP_NT, 0, c->stream>>>(a);
             cuda_check(cudaEventRecord(e0, c->stream), "tune record");
             vars[v]<<<grid, thr ? thr[v] : HOP_NT, 0, c->stream>>>(a);

@@ -123,7 +123,8 @@ __device__ __forceinline__ bool fx_dir(const FxHop &a, const Geom &g, const Bloc
 }
 
 // all eight, as a rolled loop: unrolled, the code misses the instruction
-// cache (5.5 instead of 0.2 stalls for instructions per issue)
+// cache (D_w of 32^3 x 64 3147 us instead of 1332; rolled, 0.15 stalls for
+// instructions per issue)
 template <bool CONV, bool DAG>
 __device__ __forceinline__ bool fx_dirs(const FxHop &a, const Geom &g, const BlockInfo &bi, int r, int p, const int y[4],
                                         int ll, long long s, FxAcc &acc) {

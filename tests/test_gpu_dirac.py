@@ -211,3 +211,23 @@ def test_nonfinite_inputs_and_allocation_failure():
     assert e.value.status == 2
     # the library stays usable
     ps.psms_dw_apply(ctx, 0, ps.OP_FULL, b, x, ps.PREC_F64)
+
+
+@pytest.mark.parametrize("prec", [ps.PREC_F32, ps.PREC_BF16])
+@pytest.mark.parametrize("dims", [(8, 8, 8, 8), (16, 8, 8, 4)])
+def test_tuned_hop_choice_never_changes_the_bits(prec, dims):
+    """Whatever the timings choose, the operator is that of every form of one
+    thread per site, bit for bit (fresh contexts tune again)."""
+    outs = []
+    for v in (0, 1, 2, 3, 4, 5, 6, 7, 10, 11, 12, 13) + (None,) * 6:
+        ctx = ps.psms_create(dims, (4, 4, 4, 4), 0.15, 1)
+        ps.psms_gauge_init(ctx, 0, 0.5, 31)
+        if v is not None:
+            ps.psms_hop_variant(ctx, v)
+        nat = native(ctx, seeded.spinor(dims, 32), prec)
+        out = torch.zeros_like(nat)
+        for _ in range(2):  # the tuning call and a tuned one
+            ps.psms_dw_apply(ctx, 0, ps.OP_FULL, nat, out, prec)
+        torch.cuda.synchronize()
+        outs.append(out)
+    assert all(torch.equal(o, outs[0]) for o in outs)
