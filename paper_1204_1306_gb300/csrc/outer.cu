@@ -171,9 +171,9 @@ void sub_projected(psms_ctx *c, int mode, double2 *out, const double2 *y, double
 // interpolated link fields U_{i0} .. U_{i0+n} (or U, U' when independent),
 // masked by `kind` (0 none, 1 crossing links zeroed, 2 only crossing kept):
 // fixed-point copies (the FP64 hops and true residuals) and, when asked, the
-// FP64 or FP32 ones (inner iterations).  Without the FP64 ones, each field
-// passes through a single FP64 field: kept, they are a seventh of a level's
-// memory.
+// FP64 or FP32 ones (inner iterations).  The endpoints are masked, so that one
+// pass over them writes every field (32^3 x 64, 24 systems: masking the fields
+// one by one read the endpoints 24 times, 30 ms a filter step).
 struct LinkSet {
     double2 *u64 = nullptr;
     int4 *fx = nullptr;
@@ -191,16 +191,16 @@ LinkSet make_links(psms_ctx *c, const double2 *U, const double2 *Up, int N, int 
     ls.nf = ind ? 2 : n + 1;
     const std::string t(tag);
     if (need64) ls.u64 = (double2 *)scratch(c, "ol64_" + t, sizeof(double2) * ls.nel * ls.nf);
-    double2 *one = need64 ? nullptr : (double2 *)scratch(c, "ol64_one", sizeof(double2) * ls.nel);
     ls.fx = (int4 *)scratch(c, "olfx_" + t, sizeof(int4) * fx_field(V) * ls.nf);
     if (need32) ls.u32 = (float2 *)scratch(c, "ol32_" + t, sizeof(float2) * ls.nel * ls.nf);
-    for (int f = 0; f < ls.nf; ++f) {
-        double2 *u = need64 ? ls.u64 + f * ls.nel : one;
-        interpolate(c, U, Up, u, nullptr, ind ? 1 : N, ind ? f : i0 + f, 1);
-        if (kind) mask_links(c, u, ls.nel, 1, kind);
-        links_to_fx(c, u, ls.nel, ls.fx + f * fx_field(V), 1);
-        if (need32) links_to_f32(c, u, ls.u32 + f * ls.nel, ls.nel);
+    if (kind) {
+        double2 *ends = (double2 *)scratch(c, "ol64_ends", sizeof(double2) * 2 * ls.nel);
+        interpolate(c, U, Up, ends, nullptr, 1, 0, 2);
+        mask_links(c, ends, ls.nel, 2, kind);
+        U = ends;
+        Up = ends + ls.nel;
     }
+    interpolate(c, U, Up, ls.u64, ls.u32, ind ? 1 : N, ind ? 0 : i0, ls.nf, ls.fx);
     return ls;
 }
 
