@@ -19,7 +19,7 @@
 //
 // Measured with CGNR against the general solver: the block level of 16^4 with
 // twelve systems 18.7 -> 10.8 ms, 243 blocks of 12^4 1.10 -> 0.52 ms; with
-// BiCGStab 6.9 and 0.41 ms (960 us for the 512 blocks of a 16^3 x 32 lattice).
+// BiCGStab 7.0 and 0.41 ms (960 us for the 512 blocks of a 16^3 x 32 lattice).
 //
 // FP64 has two lanes per SM here, a warp's FP64 instruction costs 16 clocks
 // of them, so the iterations have none: the norms are summed exactly in
@@ -347,6 +347,7 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
     const float A = (float)a.A, c4 = (float)(-1.0 / (4.0 * a.A)), h2A = (float)(0.5 / a.A), iA = (float)(1.0 / a.A);
     int total_it = 0, spent = 0, status = 0, slot = 0;  // (spent: by BiCGStab, before CGNR started over)
     double rel = 0, rn = bn, rn_old = 0;
+    double reach = 1;   // of the steps so far, with CGNR
     bool met = false;   // the tolerance, in the step before
     bool quit = false;  // BiCGStab gave up
     for (int outer = 0;; ++outer) {
@@ -383,11 +384,13 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
         }
         // BiCGStab ends an inner solve anywhere below its target, up to a
         // decade, so that two steps of 1e-6 may land just below a tolerance of
-        // 1e-13, where CGNR takes a third: one more step when aim asks for it
+        // 1e-13, where CGNR, which ends within a factor three of the target,
+        // takes a third: one more step when aim asks for it and the tolerance is
+        // below what that many steps of CGNR reach
         rel = sqrt(rn / bn);
         const double aim = bicg ? a.aim : a.tol;
         const bool last = outer >= a.max_outer || total_it >= a.maxit;
-        if (!quit && (rel <= aim || (rel <= a.tol && (met || last)))) break;
+        if (!quit && (rel <= aim || (rel <= a.tol && (met || last || a.tol >= reach)))) break;
         if (bicg && (quit || last || (outer > 0 && !(rn <= 0.25 * rn_old)))) {
             // BiCGStab does not get there: the item starts over with CGNR
             bicg = quit = false;
@@ -403,6 +406,7 @@ __device__ void block_cg_item(const Args &a, int rl, int k, bool bicg, CgShared 
         }
         rn_old = rn;
         met = rel <= a.tol;
+        reach *= a.delta * (1.0 / 3.0);
         // inner reduction, no further than the rounding of FP64
         const float delta = (float)(bicg ? fmax(a.delta, 0x1.0p-54 / rel) : a.delta), delta2 = delta * delta;
         const double2 *src = outer ? r64 : b;

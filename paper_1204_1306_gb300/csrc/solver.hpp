@@ -20,9 +20,9 @@ struct BlockSolveReq {
     const int4 *fx = nullptr;
     long long fx_bs = 0;
     double tol = 1e-13;
-    // the residual wanted of solves that BiCGStab ends anywhere below tol (<= tol;
-    // 0: tol): the levels' estimates ask for a sixteenth, which bounds their error
-    // by that of the CGNR solves
+    // the residual wanted of solves that BiCGStab ends just below tol where CGNR
+    // would have taken one more step (<= tol; 0: tol): the levels' estimates ask
+    // for a sixteenth, which bounds their error by that of the CGNR solves
     double aim = 0;
     int maxit = 100000;
     int inner_prec = P64;
