@@ -316,12 +316,16 @@ psms_status psms_filter_record(psms_ctx *ctx, int what, double *out, int n, int 
  * own context, possibly of different sizes; same device) solved by one
  * persistent launch (Sec. 3: the block levels are independent per block):
  * CTAs take (lattice, block, system) items from an atomic counter; every
- * item runs the even-odd CGNR with its FP64 defect correction on the device.
+ * item runs the whole solve on the device, FP64 defect correction around
+ * inner iterations.  With FP32 inner iterations and blocks of 256 sites on
+ * every lattice these are each context's (psms_block_krylov as it is at
+ * creation: BiCGStab unless called); a plan with a lattice of other blocks
+ * and one with FP64 inner iterations run CGNR.
  * psms_block_plan_create allocates the scratch, autotunes the schedule
  * (persistent grid of 1..4 CTAs per SM x three work orders, each timed once
  * on the given inputs; the results do not depend on the schedule) and
  * captures the tuned launch sequence in a CUDA graph.  psms_block_plan_run
- * replays the graph on `stream` (refreshing FP32 link copies first) and
+ * replays the graph on `stream` (refreshing the link copies first) and
  * returns the summed inner iterations and the worst relative residual.
  * Problem i: b_dev / x_dev hold n_rhs native FP64 fields back to back; the
  * pointers and fields are fixed at plan creation. */
@@ -393,8 +397,10 @@ psms_status psms_profile_enable(psms_ctx *ctx, int enable);
 psms_status psms_profile_read(psms_ctx *ctx, long long *launches, double *total_ms,
                               double *bytes_per_launch_sum);
 /* The same for the block-solver launches while profiling is enabled: count,
- * summed milliseconds and algorithmic bytes (per block-CG iteration and
- * half-block site: 4416 B with FP32 inner iterations, 8832 B with FP64). */
+ * summed milliseconds and algorithmic bytes (per Krylov iteration and
+ * half-block site: 4416 B with FP32 inner iterations, 8832 B with FP64; a
+ * measure of the iterations: blocks of 256 sites stay on the SM and move
+ * less). */
 psms_status psms_profile_read_block(psms_ctx *ctx, long long *launches, double *total_ms, double *bytes);
 /* Per block-solver launch since profiling was enabled (the first 4096, in
  * launch order): CUDA-event milliseconds and algorithmic bytes.  Writes
@@ -467,14 +473,15 @@ psms_status psms_inner_reduction(psms_ctx *ctx, double delta);
  * the two endpoint fields of Eq. (gfparam), with the systems of a launch
  * walked side by side so that every endpoint link leaves HBM about once per
  * launch; on = 0 reads one materialised FP32 field per interpolation step.
- * The FP64 true residuals use the FP64 interpolated fields either way, so
- * both reach the same tolerance.  PSMS_EINVAL for another value. */
+ * The FP64 true residuals use the interpolated fields in 59-bit fixed point
+ * either way, so both reach the same tolerance.  PSMS_EINVAL for another value. */
 psms_status psms_shared_links(psms_ctx *ctx, int on);
 /* Inner Krylov method of the Dirichlet block solves (the autotuner then
  * chooses among that method's variants only, so every tuned choice gives
  * identical results).  Unless called, blocks of 256 sites with FP32 inner
- * iterations use BiCGStab and fall back to CGNR per block where it stalls,
- * all others CGNR.  PSMS_EINVAL for another kind. */
+ * iterations use BiCGStab, and a block it does not solve in 48 iterations a
+ * correction starts over with CGNR (the iteration cap holds for each method by
+ * itself; the counts add up); all others use CGNR.  PSMS_EINVAL for another kind. */
 psms_status psms_block_krylov(psms_ctx *ctx, int kind);
 
 /* Largest number of interpolation steps (systems) batched into one launch
@@ -489,8 +496,10 @@ psms_status psms_max_chunk(psms_ctx *ctx, int n);
  * bulk (TMA) copies; for FP32 links in the whole-lattice mode 14 variants on
  * such blocks, 10 on others, 15 with shared-endpoint links, 4 otherwise; one
  * form for FP64 operators, in fixed point or, in captured calls, in FP64
- * arithmetic; used modulo their count) instead of the autotuned one; -1 returns to autotuning.  All
- * variants compute the same operator.  *n_variants (may be NULL) receives
+ * arithmetic; used modulo their count) instead of the autotuned one; -1
+ * returns to autotuning.  All variants compute the same operator, those the
+ * autotuner chooses among bit for bit (the forms with two threads per site add
+ * in another order and are only forced).  *n_variants (may be NULL) receives
  * 15.  PSMS_EINVAL outside -1..14. */
 psms_status psms_hop_variant(psms_ctx *ctx, int variant, int *n_variants);
 
@@ -506,8 +515,10 @@ psms_status psms_checkpoint_load(psms_ctx *ctx, int field, const char *path, uin
 
 /* Autotuning of launch variants (on by default; an implementation control).
  * The hop kernel's register cap and branch-free specialisation and the
- * block solver's (cluster size, register cap, hop form) are timed on their
- * first use per shape and the fastest kept.  block_variant >= 0 forces block-solver variant
+ * block solver's (cluster size, register cap, hop form; blocks of 256 sites
+ * with FP32 inner iterations have one form) are timed on their first use per
+ * shape and the fastest kept, except while the stream is captured.
+ * block_variant >= 0 forces the general block solver and its variant
  * (cluster size, min CTAs per SM) = (1,1),(1,4),(2,1),(2,4),(4,1),(4,4),
  * (8,1),(8,4) for index 0..7, (1,1),(1,4) with one out-of-line copy of
  * the hop for 8, 9, and (1,1),(1,4),(4,4),(8,4) with the branch-free hop
